@@ -66,17 +66,19 @@ enum cc_status {
 /* Arithmetic used for the two contractions (integral build and ladder GEMM). */
 enum cc_precision {
     CC_FP64 = 0,       /* FP64 tensor-core MMA (DMMA), FP64 accumulation              */
-    CC_OZAKI_BF16 = 1, /* FP64 emulated by split BF16 integer slices (Ozaki scheme) on
-                          tcgen05 tensor cores: each operand row is scaled by a power of two and
-                          rounded once to a 42-bit integer cut into 6 balanced 7-bit digits (2..8
-                          slices selectable); the slice products of each level are summed in FP32
-                          on the tensor cores and drained to exact int64 at most every
-                          4096 / (products in the level) contraction elements, so every FP32 sum
-                          stays an exact integer below 2^24 for ANY input (sign-aligned data,
-                          constant matrices, Gram diagonals included); levels are recombined in
-                          int64 and converted to FP64 once.  Error: the 42-bit rounding of the
-                          inputs and the dropped levels, about 1e-11 relative.  NaN / Inf inputs
-                          give CC_ERR_NONFINITE. */
+    CC_OZAKI_BF16 = 1, /* FP64 emulated by integers on tcgen05 BF16 tensor cores (Ozaki scheme): each
+                          operand row is scaled by a power of two and rounded once to 42-bit integers.
+                          Default precision (slices = 0 or 6): the integers' residues modulo 12 or 13
+                          coprime numbers up to 256 go through one BF16 GEMM each, and the Chinese
+                          remainder theorem returns the exact sum for ANY input; error: the rounding of
+                          the inputs and of the intermediate rows, about 2e-12 relative.  Other slice
+                          counts, and workspaces that only hold the older form: balanced 7-bit digits
+                          (6 for 42 bits, 2..8 selectable), the products of each level summed in FP32 and
+                          drained to exact int64 at most every 4096 / (products in the level)
+                          contraction elements, levels recombined in int64 (exact up to the dropped
+                          levels, about 1e-11 relative with 6).  Every FP32 sum in either form stays an
+                          exact integer up to 2^24 for any input (sign-aligned data, constant matrices,
+                          Gram diagonals included).  NaN / Inf inputs give CC_ERR_NONFINITE. */
     CC_OZAKI_INT8 = 2, /* INT8-slice emulation: tcgen05 has no kind::i8 on sm_103a;
                           always returns CC_ERR_UNSUPPORTED                           */
     CC_TF32 = 3,       /* TF32 inputs, FP32 accumulation per K-chunk, FP64 across chunks */
@@ -139,7 +141,7 @@ typedef struct cc_ladder_args {
     int order;             /* cc_order                                                          */
     int a_block;           /* 0 = planner's choice; else the number of `a` values per block     */
     int flags;             /* cc_flags                                                          */
-    int slices;            /* Ozaki modes: BF16 slices per operand (0 = default 6; 2..8)         */
+    int slices;            /* CC_OZAKI_BF16: 7-bit slices of precision per operand (0 = default 6; 2..8) */
     void* workspace;       /* device scratch, 256-byte aligned                                  */
     size_t ws_bytes;       /* its size                                                          */
     size_t budget_bytes;   /* workspace_size_ex only: upper bound for the plan (0 = 150 GB)     */
@@ -167,7 +169,9 @@ typedef struct cc_ladder_plan {
     int pairs;             /* GEMM rows used for (i,j): o*o, or o(o+1)/2 with symmetry */
     size_t ws_bytes;       /* workspace the plan needs                           */
     double flops_algorithmic; /* 2(o^2+n)v^4 (integral-first) or 4 n o^2 v^3     */
-    double flops_issued;      /* tensor-core flops actually issued (slice products, padding) */
+    double flops_issued;      /* tensor-core flops issued (slice products, padding), counted in the digit form:
+                                 s(s+1)/2 products per multiply-add (the residue form issues 12 or 13 instead;
+                                 cc_ladder_profile_read counts what a call issues) */
     int pair_blocks;          /* blocks of pairs (i <= j) the device holds one at a time (1 unless
                                  CC_FLAG_HOST_T2R splits them to fit the workspace) */
 } cc_ladder_plan;
@@ -286,7 +290,7 @@ void cc_ladder_set_wait_limit_ns(unsigned long long ns);
  * in the arithmetic of `mode` (CC_FP64: DMMA; CC_OZAKI_BF16: split BF16 slices on tcgen05 with
  * FP64 recombination; CC_TF32 / CC_BF16: one rounded copy, FP32 accumulation per K-chunk).
  * accumulate != 0 adds into C.  Workspace from cc_ladder_gemm_workspace_size.
- * CC_OZAKI_BF16 is exact in its FP32 level sums for any K and any input (see cc_precision). */
+ * CC_OZAKI_BF16 is exact in its FP32 sums for any K and any input (see cc_precision). */
 int cc_ladder_gemm_workspace_size(int mode, int M, int N, int K, int slices, size_t* bytes);
 int cc_ladder_gemm(int mode, int M, int N, int K, const double* A, int lda, const double* B, int ldb, double* C,
                    int ldc, int accumulate, int slices, void* workspace, size_t ws_bytes, void* stream);

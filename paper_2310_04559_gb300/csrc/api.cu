@@ -39,6 +39,7 @@
 #include <mutex>
 
 #include "cc_internal.cuh"
+#include "crt.cuh"
 
 using namespace cc;
 
@@ -82,6 +83,10 @@ struct Ctx {
     long long PB;     // packed path: pairs (i <= j) per pair block (o(o+1)/2 unless host)
     bool hostL;       // L is page-locked host memory, streamed to the device in chunks of Cholesky vectors
     long long PC;     // hostL: Cholesky vectors per chunk (n otherwise)
+    // Residue form (crt.cuh) of the default 42-bit precision of the emulated mode: nm1 moduli for the first
+    // contraction of the order, nm2 for the second; false: the digit slices of gemm_tc.cu.
+    bool crt = false;
+    int nm1 = 0, nm2 = 0;
     int* status = nullptr;  // device status word of the call (the splits flag non-finite inputs there)
 };
 
@@ -103,7 +108,28 @@ std::vector<std::pair<int, int>> block_list(const Ctx& c, long long P, int alo, 
 }
 
 // ------------------------------------------------------------------ workspace
+// Row pitch of the residue stacks: whole 128-byte lines, one TMA box row each (rows of 1000 elements at a pitch of
+// 1000 made every box row straddle two lines: KG1 of o=20/v=200/n=1000 ran at 1098 TFLOP/s, square GEMMs with K = 1024 at 1518).
+inline long long pitch_crt(long long K) { return (K + 63) & ~63ll; }
+inline long long pitch_of(const Ctx& c, long long K) { return c.crt ? pitch_crt(K) : pitch_for(K, c.mode == CC_TF32 ? 4 : 2); }
+
+// Byte planes of an M x N residue GEMM with nm moduli: rows of pitch16(N) bytes, and a little slack after the
+// last (the consumers read whole 4-byte words).
+inline long long pitch16(long long n) { return (n + 15) & ~15ll; }
+inline size_t planes_bytes(long long nm, long long M, long long N) { return (size_t)(nm * M * pitch16(N)) + 256; }
+
+// Padded length of a row K = (o, i), o < outer, i < inner (crt_prep.cu).
+inline long long k_pad(long long outer, long long inner) { return outer * ((inner + 3) & ~3ll); }
+
+// Bytes for the result planes of an M x N residue GEMM, either orientation; small results get room for K splits.
+size_t result_bytes(long long nm, long long M, long long N)
+{
+    const size_t b = std::max(planes_bytes(nm, M, N), planes_bytes(nm, N, M));
+    return std::max(b, std::min(8 * b, (size_t)32 << 20));
+}
+
 struct FwdLayout {
+    size_t Rw, Rw_bytes;  // residue form: planes of the final GEMMs
     size_t status, pairtab, t2x, Rc, epart, epair;
     // packed path
     size_t pairtab_m, rtab, Tp, eTp, Tm, eTm, Vp, eVp, Vm, eVm, Rpc, Rmc;
@@ -129,24 +155,32 @@ FwdLayout layout_packed(const Ctx& c, long long P)
     if (c.exch) L.t2x = cv.take(8 * o * o * vv);
     L.epart = cv.take(8 * energy_scratch_doubles(c.o, c.v));
     L.epair = cv.take(8 * o * o);
-    L.V = cv.take(8 * P * vv);
+    // (residue planes: blocks of Ab rows (a, .) with Nb columns each, Ab Nb <= P and Ab <= v, rows padded to 16)
+    L.V = cv.take(c.crt ? c.nm1 * (P * vv + 15 * vv) + 256 : 8 * P * vv);
     if (c.hostL) L.Lraw = cv.take(2 * 8 * c.PC * vv);  // two FP64 chunks of L: one arriving, one in use
     const long long nk = c.hostL ? c.PC : n;           // K of the L slices held at once
     if (!f64) {
-        L.Lw = cv.take(es * s * vv * pitch_for(nk, es));
+        L.Lw = cv.take(es * (c.crt ? c.nm1 : s) * vv * pitch_of(c, nk));
         L.eL = cv.take(4 * vv);
         L.colmax = cv.take(8 * vv);
     }
     const long long pbm = std::min(c.PB, c.pm);  // pairs i < j in one pair block
-    L.Tp = cv.take(es * s * c.PB * pitch_for(c.Kp, es));
+    const long long s2 = c.crt ? c.nm2 : s;      // slices or residues of the packed operands
+    const long long kp = c.crt ? crt_kq_total(v) : c.Kp, km = c.crt ? kp : c.Km;
+    auto pk = [&](long long K) { return c.crt ? pitch_crt(K) : pitch_for(K, es); };
+    L.Tp = cv.take(es * s2 * c.PB * pk(kp));
     L.eTp = cv.take(4 * c.PB);
-    L.Tm = cv.take(es * s * pbm * pitch_for(c.Km, es));
+    L.Tm = cv.take(es * s2 * pbm * pk(km));
     L.eTm = cv.take(4 * pbm);
     L.rtab = cv.take(8 * P);
-    L.Vp = cv.take(es * s * P * pitch_for(c.Kp, es));
+    L.Vp = cv.take(es * s2 * P * pk(kp));
     L.eVp = cv.take(4 * P);
-    L.Vm = cv.take(es * s * P * pitch_for(c.Km, es));
+    L.Vm = cv.take(es * s2 * P * pk(km));
     L.eVm = cv.take(4 * P);
+    if (c.crt) {
+        L.Rw_bytes = result_bytes(c.nm2, c.PB, P);
+        L.Rw = cv.take(L.Rw_bytes);
+    }
     L.Rpc = cv.take(8 * c.PB * P);
     L.Rmc = cv.take(8 * pbm * P);
     L.total = cv.cur;
@@ -166,37 +200,43 @@ FwdLayout layout_fwd(const Ctx& c, long long A)
     L.epart = cv.take(8 * energy_scratch_doubles(c.o, c.v));
     L.epair = cv.take(8 * o * o);
     const int es = esz_of(c.mode);
-    const long long s = c.s;
+    const long long s1 = c.crt ? c.nm1 : c.s, s2 = c.crt ? c.nm2 : c.s;
     if (c.order == CC_ORDER_INTEGRAL_FIRST) {
-        L.V = cv.take(8 * (long long)A * v * vv);
+        const long long kk = c.crt ? k_pad(v, v) : vv;
+        L.V = cv.take(c.crt ? planes_bytes(s1, A * v, vv) : 8 * (long long)A * v * vv);
         if (is_tc(c.mode)) {
-            L.Lw = cv.take(es * s * vv * pitch_for(n, es));
+            L.Lw = cv.take(es * s1 * vv * pitch_of(c, n));
             L.eL = cv.take(4 * vv);
             L.colmax = cv.take(8 * vv);
-            L.tw = cv.take(es * s * P * pitch_for(vv, es));
+            L.tw = cv.take(es * s2 * P * pitch_of(c, kk));
             L.et = cv.take(4 * P);
-            L.Vw = cv.take(es * s * (long long)A * v * pitch_for(vv, es));
+            L.Vw = cv.take(es * s2 * (long long)A * v * pitch_of(c, kk));
             L.eV = cv.take(4 * (long long)A * v);
         }
+        if (c.crt) L.Rw_bytes = result_bytes(s2, P, A * v);
     } else {
-        L.X2 = cv.take(8 * P * (long long)A * n * v);
+        const long long kk = c.crt ? k_pad(n, v) : n * v;
+        L.X2 = cv.take(c.crt ? planes_bytes(s1, A * n, P * v) : 8 * P * (long long)A * n * v);
         if (is_tc(c.mode)) {
-            L.LwA = cv.take(es * s * v * n * pitch_for(v, es));
+            L.LwA = cv.take(es * s1 * v * n * pitch_of(c, v));
             L.eLA = cv.take(4 * v * n);
-            L.twB = cv.take(es * s * P * v * pitch_for(v, es));
+            L.twB = cv.take(es * s1 * P * v * pitch_of(c, v));
             L.etB = cv.take(4 * P * v);
             L.colmax = cv.take(8 * P * v);
-            L.X2w = cv.take(es * s * P * (long long)A * pitch_for(n * v, es));
+            L.X2w = cv.take(es * s2 * P * (long long)A * pitch_of(c, kk));
             L.eX2 = cv.take(4 * P * (long long)A);
-            L.LwB = cv.take(es * s * v * pitch_for(n * v, es));
+            L.LwB = cv.take(es * s2 * v * pitch_of(c, kk));
             L.eLB = cv.take(4 * v);
         }
+        if (c.crt) L.Rw_bytes = result_bytes(s2, P * A, v);
     }
+    if (c.crt) L.Rw = cv.take(L.Rw_bytes);
     L.total = cv.cur;
     return L;
 }
 
 struct BwdLayout {
+    size_t Rw, Rw_bytes;
     size_t status, LT, Wx, tx, M1, fwd;  // fwd = nested forward workspace for dt2
     size_t Lw, eL, Ww, eW, tw, et, colmax, M1w, eM1;
     size_t total;
@@ -287,7 +327,7 @@ long long pick_block_host(Ctx& c, size_t bytes, int requested, size_t* need);
 
 // Streamed L: the chunk of Cholesky vectors starts at the caller's chol_chunk or at the one whose
 // two FP64 buffers and slices take an eighth of the budget, and halves until a plan fits.
-long long pick_block(Ctx& c, size_t bytes, int requested, size_t* need)
+long long pick_block_form(Ctx& c, size_t bytes, int requested, size_t* need)
 {
     if (!c.hostL) return pick_block_host(c, bytes, requested, need);
     const long long vv = (long long)c.v * c.v;
@@ -299,6 +339,21 @@ long long pick_block(Ctx& c, size_t bytes, int requested, size_t* need)
         const long long P = pick_block_host(c, bytes, requested, need);
         if (P >= 0 || pc == 1) return P;
     }
+}
+
+// The residue form needs up to about twice the slices' memory (bf16 residues for 12 or 13 moduli instead of 6
+// digits): where it does not fit -- or, with host-resident amplitudes, would not hold all pairs at once next to
+// blocks of 4 `a` values, so that t2 would be split again for every block -- the digit slices run as before.
+long long pick_block(Ctx& c, size_t bytes, int requested, size_t* need)
+{
+    if (c.crt) {
+        Ctx t = c;
+        const long long P = pick_block_form(t, bytes, requested, need);
+        const bool whole = !(t.host && t.packed) || (t.PB == t.pp && P >= (long long)std::min(t.v, 4) * t.v);
+        if (P >= 0 && whole) { c = t; return P; }
+        c.crt = false;
+    }
+    return pick_block_form(c, bytes, requested, need);
 }
 
 long long pick_block_host(Ctx& c, size_t bytes, int requested, size_t* need)
@@ -339,6 +394,15 @@ long long pick_block_pb(const Ctx& c, size_t bytes, int requested, size_t* need)
     }
     *need = layout_fwd(c, P).total;
     return P;
+}
+
+// Residue form of the default precision for contractions of K1 terms (rows from FP64) and K2 terms (rows from FP64
+// and rows from the first one's planes); padded lengths stay below 2^31.
+void set_crt(Ctx* c, long long K1, long long K2)
+{
+    c->nm1 = crt_moduli(K1);
+    c->nm2 = crt_moduli(K2, kCrtBits, kPlaneBits);
+    c->crt = c->mode == CC_OZAKI_BF16 && c->s == kDefaultSlices && c->nm1 > 0 && c->nm2 > 0 && 4 * K2 < (1ll << 31);
 }
 
 int make_ctx(const cc_ladder_args* a, Ctx* c)
@@ -383,6 +447,10 @@ int make_ctx(const cc_ladder_args* a, Ctx* c)
     // host-resident amplitudes run on the packed path only, without the exchange copy
     if (c->host && (!c->packed || c->exch)) return CC_ERR_UNSUPPORTED;
     if (c->hostL && !c->packed) return CC_ERR_UNSUPPORTED;
+    // K of the two contractions
+    const bool integral_first = c->order == CC_ORDER_INTEGRAL_FIRST;
+    const long long vv = (long long)a->v * a->v;
+    set_crt(c, integral_first ? a->n_chol : a->v, integral_first ? vv : (long long)a->n_chol * a->v);
     return CC_OK;
 }
 
@@ -588,6 +656,101 @@ int run_tc(const char* name, const Ctx& c, int M, int N, int K, const Operand& A
     return check_cuda(gemm_tc(g, st));
 }
 
+// ------------------------------------------------------------ residue form
+// MMA area of an M x N residue GEMM: whole 256-row tiles, columns rounded up to 32.
+double crt_tile_area(long long M, long long N)
+{
+    return (double)((M + 255) / 256 * 256) * (double)((N + 31) / 32 * 32);
+}
+
+int crt_gemm(const char* name, GemmCrt& g, cudaStream_t st)
+{
+    const double el = tri_elems(g.M, g.N, g.tri, 256, 256);
+    ProfScope ps(name, st, 2.0 * el * g.K * g.nm, 2.0 * g.nm * ((double)g.M + g.N) * g.K + el * g.nm * std::max(1, g.ksplit));
+    return check_cuda(gemm_crt(g, st));
+}
+
+// planes[l][m][n] = sum_k A(m,k) B(n,k) mod p_l, an intermediate (accumulate: added to the residues there).
+int run_crt(const char* name, const Ctx& c, int nm, int M, int N, int K, const Operand& A, long long rowA0, const Operand& B,
+            long long rowB0, unsigned char* planes, CrtPlanes* out, cudaStream_t st, long long tri = 0, bool accumulate = false)
+{
+    GemmCrt g{};
+    g.M = M; g.N = N; g.K = K; g.nm = nm;
+    g.A = A.D; g.pitchA = A.pitch; g.rowsA = A.rows; g.rowA0 = rowA0;
+    g.B = B.D; g.pitchB = B.pitch; g.rowsB = B.rows; g.rowB0 = rowB0;
+    g.planes = planes; g.pitch = pitch16(N);
+    g.ksplit = 1;
+    g.accumulate = accumulate ? 1 : 0;
+    g.tri = tri;
+    g.status = c.status;
+    g.wait_ns = g_wait_ns.load();
+    *out = CrtPlanes{planes, (long long)M * g.pitch, g.pitch, nm};
+    return crt_gemm(name, g, st);
+}
+
+// out = sum_k A(m,k) B(n,k) in FP64 through result planes of `cap` bytes.  nm_src > 0: B's rows were made from
+// the planes of a contraction with nm_src moduli (kPlaneBits, CrtRec::frac left out).  The GEMM runs in the orientation whose
+// tiles waste less (M comes in whole 256-row tiles, N in columns of 32), and K is split where the items
+// (modulus x tile) would leave SM pairs idle; the splits' residues are summed by the conversion.
+int run_crt_out(const char* name, const Ctx& c, int nm, int M, int N, int K, const Operand& A, const Operand& B,
+                const OutDesc& out, unsigned char* planes, size_t cap, cudaStream_t st, int nm_src)
+{
+    const int base = crt_base(crt_rec(nm), kCrtBits, nm_src > 0 ? kPlaneBits : kCrtBits);
+    const double factor = nm_src > 0 ? crt_rec(nm_src).frac : 1.0;
+    const bool swap = crt_tile_area(N, M) < crt_tile_area(M, N);
+    const Operand& Ao = swap ? B : A;
+    const Operand& Bo = swap ? A : B;
+    OutDesc o = out;
+    if (swap) { std::swap(o.rmap, o.cmap); std::swap(M, N); }
+    GemmCrt g{};
+    g.M = M; g.N = N; g.K = K; g.nm = nm;
+    g.A = Ao.D; g.pitchA = Ao.pitch; g.rowsA = Ao.rows;
+    g.B = Bo.D; g.pitchB = Bo.pitch; g.rowsB = Bo.rows;
+    g.planes = planes; g.pitch = pitch16(N);
+    g.status = c.status;
+    g.wait_ns = g_wait_ns.load();
+    const long long items = (long long)nm * ((M + 255) / 256) * ((N + 255) / 256);
+    const int pairs = std::max(1, device_sm_count() / 2);
+    auto eff = [&](int S) { const double w = (double)items * S / pairs; return w / std::ceil(w); };
+    int S = 1;
+    for (int t = 2; t <= 8 && K / t >= 2048 && planes_bytes((long long)nm * t, M, N) <= cap; ++t)
+        if (eff(t) > eff(S) + 0.05) S = t;
+    const int kper = ((K + S - 1) / S + 63) / 64 * 64;  // the kernel's split, in whole K-steps
+    g.ksplit = (K + kper - 1) / kper;
+    CC_TRY(crt_gemm(name, g, st));
+    ProfScope ps("crt_out", st);
+    const CrtPlanes pl{planes, (long long)M * g.pitch, g.pitch, nm};
+    return check_cuda(crt_to_f64(M, N, pl, g.ksplit, o, base, factor, swap, Ao.e, Bo.e, st));
+}
+
+// Rows of K = (o, i) from FP64 (ostride between outer indices).
+int prep_crt_rows(const Ctx& c, const RowSrc& src, int outer, int inner, long long ostride, int nm, Operand& op,
+                  cudaStream_t st)
+{
+    ProfScope ps("split", st);
+    op.rows = src.rows;
+    op.pitch = pitch_crt(k_pad(outer, inner));
+    return check_cuda(crt_rows(src, outer, inner, ostride, nm, op.D, op.pitch, op.e, c.status, st));
+}
+
+int prep_crt_cols(const Ctx& c, const ColSrc& src, int nm, Operand& op, unsigned long long* colmax, cudaStream_t st,
+                  bool premax = false)
+{
+    ProfScope ps("split", st);
+    op.rows = src.rows;
+    op.pitch = pitch_crt(src.K);
+    return check_cuda(crt_cols(src, nm, op.D, op.pitch, op.e, colmax, c.status, st, premax));
+}
+
+int prep_crt_planes(const CrtPlanes& src, int nal, int nq, bool q_major, int outer, int inner, const int* eA, const int* eB,
+                    int nm, Operand& op, cudaStream_t st)
+{
+    ProfScope ps("split", st);
+    op.rows = (long long)nal * nq;
+    op.pitch = pitch_crt(k_pad(outer, inner));
+    return check_cuda(crt_rows_planes(src, nal, nq, q_major, outer, inner, eA, eB, nm, op.D, op.pitch, op.e, st));
+}
+
 template <typename T>
 T* at(void* ws, size_t off) { return (T*)((char*)ws + off); }
 
@@ -612,8 +775,11 @@ int fwd_packed(const Ctx& c, const cc_ladder_args* a, const double* Lsrc, const 
     Lw.D = at<void>(ws, Lo.Lw); Lw.e = at<int>(ws, Lo.eL);
     Tp.D = at<void>(ws, Lo.Tp); Tp.e = at<int>(ws, Lo.eTp); Tp.rows = c.pp; Tp.pitch = pitch_for(c.Kp, es);
     Tm.D = at<void>(ws, Lo.Tm); Tm.e = at<int>(ws, Lo.eTm); Tm.rows = c.pm; Tm.pitch = pitch_for(c.Km, es);
+    const int kq = (int)(c.crt ? crt_kq_total(v) : 0);
+    if (c.crt) Tp.pitch = Tm.pitch = pitch_crt(kq);
     Vp.D = at<void>(ws, Lo.Vp); Vp.e = at<int>(ws, Lo.eVp); Vp.pitch = Tp.pitch;
     Vm.D = at<void>(ws, Lo.Vm); Vm.e = at<int>(ws, Lo.eVm); Vm.pitch = Tm.pitch;
+    unsigned char* Rw = c.crt ? at<unsigned char>(ws, Lo.Rw) : nullptr;
     unsigned long long* colmax = at<unsigned long long>(ws, Lo.colmax);
     // Streamed L (CC_FLAG_HOST_L): chunks of PC Cholesky vectors are copied from page-locked host
     // memory into two device buffers on a second stream, so that chunk q + 1 arrives while chunk q
@@ -660,7 +826,8 @@ int fwd_packed(const Ctx& c, const cc_ladder_args* a, const double* Lsrc, const 
     if (!f64 && !c.hostL) {
         // L rows (a,c) are contiguous in L[P][a][c]; K = P is strided
         ColSrc ls{Lsrc, vv, vv, n, 0, plain_map(0)};
-        CC_TRY(prep_cols(c, ls, Lw, colmax, st));
+        if (c.crt) CC_TRY(prep_crt_cols(c, ls, c.nm1, Lw, colmax, st));
+        else CC_TRY(prep_cols(c, ls, Lw, colmax, st));
     } else if (ozaki && c.hostL) {
         // row scales of the Ozaki split need every Cholesky vector: one streaming pass for the maxima
         CC_CU(cudaMemsetAsync(colmax, 0, 8 * vv, st));
@@ -685,6 +852,9 @@ int fwd_packed(const Ctx& c, const cc_ladder_args* a, const double* Lsrc, const 
         const long long s0 = strict_before(q0), s1 = strict_before(q1);
         Tp.rows = q1 - q0;
         Tm.rows = s1 - s0;
+        if (c.crt)
+            return check_cuda(crt_pm_f64(t2, pairtab + q0, c.o, c.v, q0, q1 - q0, s0, minus ? s1 - s0 : 0, c.nm2, Tp.D, Tp.e,
+                                         Tm.D, Tm.e, Tp.pitch, c.status, st));
         CC_CU(pm_split_f64(t2, pairtab + q0, 1, q1 - q0, c.v, +1, 1.0, kind, c.s, kBeta, Tp.D, Tp.pitch, Tp.e, c.status, st));
         if (minus && s1 > s0)
             CC_CU(pm_split_f64(t2, pairtab_m + s0, 1, s1 - s0, c.v, -1, 1.0, kind, c.s, kBeta, Tm.D, Tm.pitch, Tm.e,
@@ -701,10 +871,17 @@ int fwd_packed(const Ctx& c, const cc_ladder_args* a, const double* Lsrc, const 
         const long long nr = (long long)Ab * Nb - (long long)Ab * (Ab - 1) / 2;
         // KG1: V[al][b'][c][d] = sum_P L[P, a0+al, c] L[P, a0+b', d], tiles with b < a skipped
         OutDesc o1{V, split_map(v, (long long)Nb * vv, v), split_map(v, vv, 1), 0};
+        CrtPlanes vpl{};  // residue form: planes[l][(al, c)][(b', d)]
         if (c.hostL) {
             // the block's integrals summed over the chunks of Cholesky vectors (additive in P)
             CC_TRY(stream_L([&](const double* buf, long long P0, long long Pq) -> int {
                 OutDesc oq = o1;
+                if (c.crt) {
+                    const ColSrc lq{buf, vv, vv, Pq, 0, plain_map(0)};
+                    CC_TRY(prep_crt_cols(c, lq, c.nm1, Lw, colmax, st, true));
+                    return run_crt("kg1_tc", c, c.nm1, Ab * c.v, Nb * c.v, (int)Pq, Lw, (long long)a0 * v, Lw,
+                                   (long long)a0 * v, (unsigned char*)V, &vpl, st, v, P0 > 0);
+                }
                 if (f64) {
                     GemmF64 g{};
                     g.M = Ab * c.v; g.N = Nb * c.v; g.K = (int)Pq;
@@ -736,6 +913,9 @@ int fwd_packed(const Ctx& c, const cc_ladder_args* a, const double* Lsrc, const 
             g.out = o1;
             g.tri = v;
             CC_TRY(run_f64("kg1_f64", g, st, tri_elems(g.M, g.N, v, 64, 64)));
+        } else if (c.crt) {
+            CC_TRY(run_crt("kg1_tc", c, c.nm1, Ab * c.v, Nb * c.v, c.n, Lw, (long long)a0 * v, Lw, (long long)a0 * v,
+                           (unsigned char*)V, &vpl, st, v));
         } else {
             CC_TRY(run_tc("kg1_tc", c, Ab * c.v, Nb * c.v, c.n, Lw, (long long)a0 * v, Lw, (long long)a0 * v, o1,
                           status, st, true, v));
@@ -744,7 +924,10 @@ int fwd_packed(const Ctx& c, const cc_ladder_args* a, const double* Lsrc, const 
         Vp.rows = nr; Vm.rows = nr;
         {
             ProfScope ps("split", st);
-            if (ozaki) {
+            if (c.crt) {
+                CC_CU(crt_pm_planes(vpl, rtab, nr, Nb, c.v, Lw.e + (long long)a0 * v, c.nm2, Vp.D, Vp.e,
+                                    minus ? Vm.D : nullptr, minus ? Vm.e : nullptr, Vp.pitch, st));
+            } else if (ozaki) {
                 // V[al][b'][c][d] = X * 2^(eL[(a0+al)v + c] + eL[(a0+b')v + d] + base)
                 PmFixedSrc fs{(const long long*)V, rtab, nr, vv, c.v, Lw.e, split_map(Nb, v, 0, (long long)a0 * v),
                               Lw.e, split_map(Nb, 0, v, (long long)a0 * v), kFixedBase};
@@ -773,6 +956,9 @@ int fwd_packed(const Ctx& c, const cc_ladder_args* a, const double* Lsrc, const 
                     g.out = sg ? om : op;
                     CC_TRY(run_f64("kg2_f64", g, st));
                 }
+            } else if (c.crt) {
+                CC_TRY(run_crt_out("kg2_tc", c, c.nm2, (int)(q1 - q0), (int)nr, kq, Tp, Vp, op, Rw, Lo.Rw_bytes, st, c.nm1));
+                if (mb) CC_TRY(run_crt_out("kg2_tc", c, c.nm2, (int)(s1 - s0), (int)nr, kq, Tm, Vm, om, Rw, Lo.Rw_bytes, st, c.nm1));
             } else {
                 CC_TRY(run_tc("kg2_tc", c, (int)(q1 - q0), (int)nr, (int)c.Kp, Tp, 0, Vp, 0, op, status, st));
                 if (mb) CC_TRY(run_tc("kg2_tc", c, (int)(s1 - s0), (int)nr, (int)c.Km, Tm, 0, Vm, 0, om, status, st));
@@ -867,9 +1053,14 @@ int fwd_impl(const cc_ladder_args* a, const double* Lsrc_override = nullptr)
             Vw.D = at<void>(ws, Lo.Vw); Vw.e = at<int>(ws, Lo.eV);
             // L rows (a,c) are contiguous in L[P][a][c]; K = P is strided
             ColSrc ls{Lsrc, vv, vv, n, 0, plain_map(0)};
-            CC_TRY(prep_cols(c, ls, Lw, at<unsigned long long>(ws, Lo.colmax), st));
             RowSrc ts{t2, trows, plain_map(1), c.pairs, vv};
-            CC_TRY(prep_rows(c, ts, tw, st));
+            if (c.crt) {
+                CC_TRY(prep_crt_cols(c, ls, c.nm1, Lw, at<unsigned long long>(ws, Lo.colmax), st));
+                CC_TRY(prep_crt_rows(c, ts, c.v, c.v, v, c.nm2, tw, st));
+            } else {
+                CC_TRY(prep_cols(c, ls, Lw, at<unsigned long long>(ws, Lo.colmax), st));
+                CC_TRY(prep_rows(c, ts, tw, st));
+            }
         }
         for (int a0 = alo; a0 < ahi; a0 += A) {
             const int Ab = std::min(A, ahi - a0);
@@ -882,6 +1073,12 @@ int fwd_impl(const cc_ladder_args* a, const double* Lsrc_override = nullptr)
                 g.B = Lsrc; g.bm = plain_map(1); g.bk = plain_map(vv);
                 g.out = o1;
                 CC_TRY(run_f64("kg1_f64", g, st));
+            } else if (c.crt) {
+                // planes[l][(al, c)][(b, d)], then rows (al, b) of K = (c, d)
+                CrtPlanes pl;
+                CC_TRY(run_crt("kg1_tc", c, c.nm1, Ab * c.v, (int)vv, c.n, Lw, (long long)a0 * v, Lw, 0, (unsigned char*)V,
+                               &pl, st));
+                CC_TRY(prep_crt_planes(pl, Ab, c.v, false, c.v, c.v, Lw.e + (long long)a0 * v, Lw.e, c.nm2, Vw, st));
             } else {
                 CC_TRY(run_tc("kg1_tc", c, Ab * c.v, (int)vv, c.n, Lw, (long long)a0 * v, Lw, 0, o1, status, st, true));
             }
@@ -894,6 +1091,9 @@ int fwd_impl(const cc_ladder_args* a, const double* Lsrc_override = nullptr)
                 g.B = V; g.bm = plain_map(vv); g.bk = plain_map(1);
                 g.out = o2;
                 CC_TRY(run_f64("kg2_f64", g, st));
+            } else if (c.crt) {
+                CC_TRY(run_crt_out("kg2_tc", c, c.nm2, (int)c.pairs, Ab * c.v, (int)k_pad(v, v), tw, Vw, o2,
+                                   at<unsigned char>(ws, Lo.Rw), Lo.Rw_bytes, st, c.nm1));
             } else {
                 if (c.mode == CC_OZAKI_BF16) {
                     // V[al][b][c][d] = X * 2^(eL[(a0+al)v + c] + eL[b v + d] + base)
@@ -918,13 +1118,19 @@ int fwd_impl(const cc_ladder_args* a, const double* Lsrc_override = nullptr)
             LwB.D = at<void>(ws, Lo.LwB); LwB.e = at<int>(ws, Lo.eLB);
             // CF1 A: rows (a, P) over all a, K = c contiguous: L[P][a][c]
             RowSrc la{Lsrc, split_map(n, v, vv), plain_map(1), v * n, v};
-            CC_TRY(prep_rows(c, la, LwA, st));
             // CF1 B: rows (p, d), K = c: batched, rows d contiguous within t2[p]
             ColSrc tb{t2, v, c.pairs * v, v, v, c.sym ? table_map(pairtab) : plain_map(vv)};
-            CC_TRY(prep_cols(c, tb, twB, at<unsigned long long>(ws, Lo.colmax), st));
             // CF2 B: rows b, K = (P, d): L[P][b][d]
             RowSrc lb{Lsrc, plain_map(v), split_map(v, vv, 1), v, n * v};
-            CC_TRY(prep_rows(c, lb, LwB, st));
+            if (c.crt) {
+                CC_TRY(prep_crt_rows(c, la, 1, c.v, 0, c.nm1, LwA, st));
+                CC_TRY(prep_crt_cols(c, tb, c.nm1, twB, at<unsigned long long>(ws, Lo.colmax), st));
+                CC_TRY(prep_crt_rows(c, lb, c.n, c.v, vv, c.nm2, LwB, st));
+            } else {
+                CC_TRY(prep_rows(c, la, LwA, st));
+                CC_TRY(prep_cols(c, tb, twB, at<unsigned long long>(ws, Lo.colmax), st));
+                CC_TRY(prep_rows(c, lb, LwB, st));
+            }
         }
         for (int a0 = alo; a0 < ahi; a0 += A) {
             const int Ab = std::min(A, ahi - a0);
@@ -937,6 +1143,12 @@ int fwd_impl(const cc_ladder_args* a, const double* Lsrc_override = nullptr)
                 g.B = t2; g.bm = c.sym ? table_map(pairtab, v, 1) : split_map(v, vv, 1); g.bk = plain_map(v);
                 g.out = o1;
                 CC_TRY(run_f64("cf1_f64", g, st));
+            } else if (c.crt) {
+                // planes[l][(al, P)][(p, d)], then rows (p, al) of K = (P, d)
+                CrtPlanes pl;
+                CC_TRY(run_crt("cf1_tc", c, c.nm1, Ab * c.n, (int)(c.pairs * v), c.v, LwA, (long long)a0 * n, twB, 0,
+                               (unsigned char*)X2, &pl, st));
+                CC_TRY(prep_crt_planes(pl, Ab, (int)c.pairs, true, c.n, c.v, LwA.e + (long long)a0 * n, twB.e, c.nm2, X2w, st));
             } else {
                 CC_TRY(run_tc("cf1_tc", c, Ab * c.n, (int)(c.pairs * v), c.v, LwA, (long long)a0 * n, twB, 0, o1, status, st,
                               true));
@@ -950,6 +1162,9 @@ int fwd_impl(const cc_ladder_args* a, const double* Lsrc_override = nullptr)
                 g.B = Lsrc; g.bm = plain_map(v); g.bk = split_map(v, vv, 1);
                 g.out = o2;
                 CC_TRY(run_f64("cf2_f64", g, st));
+            } else if (c.crt) {
+                CC_TRY(run_crt_out("cf2_tc", c, c.nm2, (int)(c.pairs * Ab), c.v, (int)k_pad(n, v), X2w, LwB, o2,
+                                   at<unsigned char>(ws, Lo.Rw), Lo.Rw_bytes, st, c.nm1));
             } else {
                 if (c.mode == CC_OZAKI_BF16) {
                     // X2[(p, al)][(P, d)] = X * 2^(eLA[(a0+al) n + P] + etB[p v + d] + base)
@@ -992,6 +1207,7 @@ struct TermCtx {
 };
 
 struct TermLayout {
+    size_t Rw, Rw_bytes;
     size_t status, V, Aw, eA, Bw, eB, colmax, tw, et, Vw, eV, total;
 };
 
@@ -1002,21 +1218,26 @@ TermLayout layout_term(const TermCtx& tc, long long Pb)
     Carve cv;
     const long long o = c.o, v = c.v, n = c.n, vv = v * v;
     L.status = cv.take(256);
-    L.V = cv.take(8 * Pb * tc.nq * vv);
+    L.V = cv.take(c.crt ? planes_bytes(c.nm1, Pb * v, tc.nq * v) : 8 * Pb * tc.nq * vv);
     if (is_tc(c.mode)) {
         const int es = esz_of(c.mode);
-        const long long s = c.s;
-        L.Aw = cv.take(es * s * tc.np_ * v * pitch_for(n, es));
+        const long long s1 = c.crt ? c.nm1 : c.s, s2 = c.crt ? c.nm2 : c.s;
+        const long long kk = c.crt ? k_pad(v, v) : vv;
+        L.Aw = cv.take(es * s1 * tc.np_ * v * pitch_of(c, n));
         L.eA = cv.take(4 * tc.np_ * v);
         if (!tc.same) {
-            L.Bw = cv.take(es * s * tc.nq * v * pitch_for(n, es));
+            L.Bw = cv.take(es * s1 * tc.nq * v * pitch_of(c, n));
             L.eB = cv.take(4 * tc.nq * v);
         }
         L.colmax = cv.take(8 * std::max(tc.np_, tc.nq) * v);
-        L.tw = cv.take(es * s * o * o * pitch_for(vv, es));
+        L.tw = cv.take(es * s2 * o * o * pitch_of(c, kk));
         L.et = cv.take(4 * o * o);
-        L.Vw = cv.take(es * s * Pb * tc.nq * pitch_for(vv, es));
+        L.Vw = cv.take(es * s2 * Pb * tc.nq * pitch_of(c, kk));
         L.eV = cv.take(4 * Pb * tc.nq);
+        if (c.crt) {
+            L.Rw_bytes = result_bytes(s2, o * o, Pb * tc.nq);
+            L.Rw = cv.take(L.Rw_bytes);
+        }
     }
     L.total = cv.cur;
     return L;
@@ -1036,9 +1257,11 @@ int term_ctx(int which, int o, int v, int n, int mode, int slices, TermCtx* tc)
     return CC_OK;
 }
 
-// Largest block of p fitting `bytes` (-1 if one p does not fit), evened over the blocks.
-long long pick_term_block(const TermCtx& tc, size_t bytes, size_t* need)
+// Largest block of p fitting `bytes` (-1 if one p does not fit), evened over the blocks; the digit slices where the
+// residue form does not fit.
+long long pick_term_block(TermCtx& tc, size_t bytes, size_t* need)
 {
+    if (tc.c.crt && layout_term(tc, 1).total > bytes) tc.c.crt = false;
     if (layout_term(tc, 1).total > bytes) { *need = layout_term(tc, 1).total; return -1; }
     long long lo = 1, hi = tc.np_;
     while (lo < hi) {
@@ -1062,11 +1285,11 @@ int term_impl(int which, int o, int v, int n, const double* Lov, const double* L
     if (!A || !Bm || !t2 || !T || !ws) return CC_ERR_NULL;
     if (!aligned(A, 16) || !aligned(Bm, 16) || !aligned(t2, 16) || !aligned(T, 16) || !aligned(ws, 256))
         return CC_ERR_ALIGN;
-    Ctx c = tc.c;
-    if (is_tc(c.mode) && !tc_gemm_available()) return CC_ERR_UNSUPPORTED;
+    if (is_tc(tc.c.mode) && !tc_gemm_available()) return CC_ERR_UNSUPPORTED;
     size_t need = 0;
     const long long Pb = pick_term_block(tc, ws_bytes, &need);
     if (Pb < 0 || need > ws_bytes) return CC_ERR_WORKSPACE;
+    Ctx c = tc.c;
     const TermLayout Lo = layout_term(tc, Pb);
     cudaStream_t st = (cudaStream_t)stream;
     const long long v_ = v, vv = v_ * v, np_ = tc.np_, nq = tc.nq;
@@ -1081,16 +1304,20 @@ int term_impl(int which, int o, int v, int n, const double* Lov, const double* L
         Vw.D = at<void>(ws, Lo.Vw); Vw.e = at<int>(ws, Lo.eV);
         // rows (p, c) of A[P][p][c] are contiguous; K = P is strided
         ColSrc as{A, np_ * v_, np_ * v_, n, 0, plain_map(0)};
-        CC_TRY(prep_cols(c, as, Aw, at<unsigned long long>(ws, Lo.colmax), st));
+        unsigned long long* colmax = at<unsigned long long>(ws, Lo.colmax);
+        if (c.crt) CC_TRY(prep_crt_cols(c, as, c.nm1, Aw, colmax, st));
+        else CC_TRY(prep_cols(c, as, Aw, colmax, st));
         if (tc.same) {
             Bw = Aw;
         } else {
             Bw.D = at<void>(ws, Lo.Bw); Bw.e = at<int>(ws, Lo.eB);
             ColSrc bs{Bm, nq * v_, nq * v_, n, 0, plain_map(0)};
-            CC_TRY(prep_cols(c, bs, Bw, at<unsigned long long>(ws, Lo.colmax), st));
+            if (c.crt) CC_TRY(prep_crt_cols(c, bs, c.nm1, Bw, colmax, st));
+            else CC_TRY(prep_cols(c, bs, Bw, colmax, st));
         }
         RowSrc ts{t2, plain_map(vv), plain_map(1), (long long)o * o, vv};
-        CC_TRY(prep_rows(c, ts, tw, st));
+        if (c.crt) CC_TRY(prep_crt_rows(c, ts, v, v, v_, c.nm2, tw, st));
+        else CC_TRY(prep_rows(c, ts, tw, st));
     }
     for (long long p0 = 0; p0 < np_; p0 += Pb) {
         const int Ab = (int)std::min(Pb, np_ - p0);
@@ -1103,6 +1330,11 @@ int term_impl(int which, int o, int v, int n, const double* Lov, const double* L
             g.B = Bm; g.bm = plain_map(1); g.bk = plain_map(nq * v_);
             g.out = o1;
             CC_TRY(run_f64("term_kg1_f64", g, st));
+        } else if (c.crt) {
+            // planes[l][(pl, c)][(q, d)], then rows (pl, q) of K = (c, d)
+            CrtPlanes pl;
+            CC_TRY(run_crt("term_kg1_tc", c, c.nm1, Ab * v, (int)(nq * v_), n, Aw, p0 * v_, Bw, 0, (unsigned char*)V, &pl, st));
+            CC_TRY(prep_crt_planes(pl, Ab, (int)nq, false, v, v, Aw.e + p0 * v_, Bw.e, c.nm2, Vw, st));
         } else {
             CC_TRY(run_tc("term_kg1_tc", c, Ab * v, (int)(nq * v_), n, Aw, p0 * v_, Bw, 0, o1, status, st, true));
         }
@@ -1116,6 +1348,9 @@ int term_impl(int which, int o, int v, int n, const double* Lov, const double* L
             g.B = V; g.bm = plain_map(vv); g.bk = plain_map(1);
             g.out = o2;
             CC_TRY(run_f64("term_kg2_f64", g, st));
+        } else if (c.crt) {
+            CC_TRY(run_crt_out("term_kg2_tc", c, c.nm2, o * o, (int)(Ab * nq), (int)k_pad(v, v), tw, Vw, o2,
+                               at<unsigned char>(ws, Lo.Rw), Lo.Rw_bytes, st, c.nm1));
         } else {
             if (c.mode == CC_OZAKI_BF16) {
                 // V[pl][q][c][d] = X * 2^(eA[(p0+pl) v + c] + eB[q v + d] + base)
@@ -1137,7 +1372,7 @@ int term_impl(int which, int o, int v, int n, const double* Lov, const double* L
 // dL  = T1[W, t] + T1[W^swap, t^swap], T1[X,t][P,e,f] = sum_(b,d) L[P,b,d] M1[e,f,b,d],
 //       M1[e,f,b,d] = sum_ij X[ij,e,b] t[ij,f,d]; for pair-symmetric t this is T1[W + W^swap, t].
 struct BwdPlan {
-    Ctx c;      // c.pairs = o*o (W has no pair symmetry)
+    Ctx c;      // c.pairs = o*o (W has no pair symmetry); nm1, nm2: moduli of M1 (K = o^2) and T1 (K = v^2)
     int E;      // e-block for M1
     cc_ladder_args fa;  // nested forward for dt2
     size_t fwd_bytes;
@@ -1153,19 +1388,24 @@ BwdLayout layout_bwd(const Ctx& c, int E, size_t fwd_bytes, bool sym)
     L.LT = cv.take(8 * n * vv);
     L.Wx = cv.take(8 * P * vv);
     if (!sym) L.tx = cv.take(8 * P * vv);
-    L.M1 = cv.take(8 * (long long)E * v * vv);
+    L.M1 = cv.take(c.crt ? planes_bytes(c.nm1, E * v, vv) : 8 * (long long)E * v * vv);
     if (is_tc(c.mode)) {
         const int es = esz_of(c.mode);
-        const long long s = c.s;
-        L.Lw = cv.take(es * s * n * pitch_for(vv, es));
+        const long long s1 = c.crt ? c.nm1 : c.s, s2 = c.crt ? c.nm2 : c.s;
+        const long long kk = c.crt ? k_pad(v, v) : vv;
+        L.Lw = cv.take(es * s2 * n * pitch_of(c, kk));
         L.eL = cv.take(4 * n);
-        L.Ww = cv.take(es * s * (long long)E * v * pitch_for(P, es));
+        L.Ww = cv.take(es * s1 * (long long)E * v * pitch_of(c, P));
         L.eW = cv.take(4 * (long long)E * v);
-        L.tw = cv.take(es * s * vv * pitch_for(P, es));
+        L.tw = cv.take(es * s1 * vv * pitch_of(c, P));
         L.et = cv.take(4 * vv);
         L.colmax = cv.take(8 * vv);
-        L.M1w = cv.take(es * s * (long long)E * v * pitch_for(vv, es));
+        L.M1w = cv.take(es * s2 * (long long)E * v * pitch_of(c, kk));
         L.eM1 = cv.take(4 * (long long)E * v);
+        if (c.crt) {
+            L.Rw_bytes = result_bytes(s2, n, E * v);
+            L.Rw = cv.take(L.Rw_bytes);
+        }
     }
     L.fwd = cv.take(fwd_bytes);
     L.total = cv.cur;
@@ -1181,11 +1421,17 @@ int bwd_plan(int o, int v, int n, int mode, int flags, int slices, size_t bytes,
     CC_TRY(make_ctx(&fa, &c));
     const bool sym = (flags & CC_FLAG_SYMMETRIC_T) != 0;
     // Split the budget: find the largest block E (used for both the nested forward's
-    // integral block and the M1 block) such that everything fits.
+    // integral block and the M1 block) such that everything fits; in the residue form if one `a` fits
+    // there, in digit slices otherwise (the nested forward then takes the same form: its own smallest plan
+    // is at least the one counted here).
+    Ctx cf = c;  // the nested forward (K = n, then v^2)
+    set_crt(&c, (long long)o * o, (long long)v * v);
+    c.crt = cf.crt = c.crt && cf.crt;
     auto total_for = [&](int A) {
-        const size_t fb = layout_fwd(c, A).total;
+        const size_t fb = layout_fwd(cf, A).total;
         return layout_bwd(c, A, fb, sym).total;
     };
+    if (c.crt && total_for(1) > bytes) c.crt = cf.crt = false;
     if (total_for(1) > bytes) return for_query ? CC_ERR_BUDGET : CC_ERR_WORKSPACE;
     int lo = 1, hi = v;
     while (lo < hi) {
@@ -1196,7 +1442,7 @@ int bwd_plan(int o, int v, int n, int mode, int flags, int slices, size_t bytes,
     const int A = (v + nb - 1) / nb;
     bp->c = c;
     bp->E = A;
-    bp->fwd_bytes = layout_fwd(c, A).total;
+    bp->fwd_bytes = layout_fwd(cf, A).total;
     bp->L = layout_bwd(c, A, bp->fwd_bytes, sym);
     bp->fa = fa;
     bp->fa.a_block = A;
@@ -1265,12 +1511,15 @@ int bwd_impl(int o, int v, int n, const double* L, const double* t2, const doubl
             tw.D = at<void>(ws, Lo.tw); tw.e = at<int>(ws, Lo.et);
             M1w.D = at<void>(ws, Lo.M1w); M1w.e = at<int>(ws, Lo.eM1);
             RowSrc ls{L, plain_map(vv), plain_map(1), n, vv};  // T1 A: rows P, K = (b,d)
-            CC_TRY(prep_rows(c, ls, Lw, st));
+            if (c.crt) CC_TRY(prep_crt_rows(c, ls, v, v, v, c.nm2, Lw, st));
+            else CC_TRY(prep_rows(c, ls, Lw, st));
         }
         for (int pass = 0; pass < npass; ++pass) {
             if (is_tc(mode)) {
                 ColSrc ts{tt[pass], vv, vv, P, 0, plain_map(0)};  // M1 B: rows (f,d), K = ij
-                CC_TRY(prep_cols(c, ts, tw, at<unsigned long long>(ws, Lo.colmax), st));
+                unsigned long long* colmax = at<unsigned long long>(ws, Lo.colmax);
+                if (c.crt) CC_TRY(prep_crt_cols(c, ts, c.nm1, tw, colmax, st));
+                else CC_TRY(prep_cols(c, ts, tw, colmax, st));
             }
             for (int e0 = 0; e0 < v; e0 += E) {
                 const int Eb = std::min(E, v - e0);
@@ -1283,6 +1532,13 @@ int bwd_impl(int o, int v, int n, const double* L, const double* t2, const doubl
                     g.B = tt[pass]; g.bm = plain_map(1); g.bk = plain_map(vv);
                     g.out = o1;
                     CC_TRY(run_f64("m1_f64", g, st));
+                } else if (c.crt) {
+                    // planes[l][(el, b)][(f, d)], then rows (el, f) of K = (b, d)
+                    ColSrc wc{Xs[pass] + (long long)e0 * v, vv, (long long)Eb * v, P, 0, plain_map(0)};
+                    CC_TRY(prep_crt_cols(c, wc, c.nm1, Ww, at<unsigned long long>(ws, Lo.colmax), st));
+                    CrtPlanes pl;
+                    CC_TRY(run_crt("m1_tc", c, c.nm1, Eb * v, (int)vv, (int)P, Ww, 0, tw, 0, (unsigned char*)M1, &pl, st));
+                    CC_TRY(prep_crt_planes(pl, Eb, v, false, v, v, Ww.e, tw.e, c.nm2, M1w, st));
                 } else {
                     ColSrc ws_{Xs[pass] + (long long)e0 * v, vv, (long long)Eb * v, P, 0, plain_map(0)};
                     CC_TRY(prep_cols(c, ws_, Ww, at<unsigned long long>(ws, Lo.colmax), st));
@@ -1297,6 +1553,9 @@ int bwd_impl(int o, int v, int n, const double* L, const double* t2, const doubl
                     g.B = M1; g.bm = plain_map(vv); g.bk = plain_map(1);
                     g.out = o2;
                     CC_TRY(run_f64("t1_f64", g, st));
+                } else if (c.crt) {
+                    CC_TRY(run_crt_out("t1_tc", c, c.nm2, n, Eb * v, (int)k_pad(v, v), Lw, M1w, o2,
+                                       at<unsigned char>(ws, Lo.Rw), Lo.Rw_bytes, st, c.nm1));
                 } else {
                     if (mode == CC_OZAKI_BF16) {
                         // M1[el][f][b][d] = X * 2^(eW[el v + b] + et[f v + d] + base)
@@ -1554,18 +1813,31 @@ int cc_ladder_energy(int o, int v, const double* R, const double* t2, double* en
     return CC_OK;
 }
 
-static size_t gemm_ws(int mode, int M, int N, int K, int s)
+// nm > 0: the residue form with that many moduli and `res` bytes of result planes
+static size_t gemm_ws(int mode, int M, int N, int K, int s, int nm = 0, size_t* res = nullptr)
 {
     Carve cv;
     cv.take(256);
     if (is_tc(mode)) {
         const int es = esz_of(mode);
-        cv.take((size_t)es * s * M * pitch_for(K, es));
+        const size_t st = nm > 0 ? nm : s;
+        cv.take((size_t)es * st * M * (nm > 0 ? pitch_crt(K) : pitch_for(K, es)));
         cv.take(4 * (size_t)M);
-        cv.take((size_t)es * s * N * pitch_for(K, es));
+        cv.take((size_t)es * st * N * (nm > 0 ? pitch_crt(K) : pitch_for(K, es)));
         cv.take(4 * (size_t)N);
+        if (nm > 0) {
+            const size_t rb = result_bytes(nm, M, N);
+            cv.take(rb);
+            if (res) *res = rb;
+        }
     }
     return cv.cur;
+}
+
+// Moduli of a GEMM that runs in the residue form (0: it does not).
+static int gemm_nm(int mode, int K, int s)
+{
+    return mode == CC_OZAKI_BF16 && s == kDefaultSlices && K < (1 << 30) ? crt_moduli(K) : 0;
 }
 
 int cc_ladder_gemm_workspace_size(int mode, int M, int N, int K, int slices, size_t* bytes)
@@ -1575,7 +1847,8 @@ int cc_ladder_gemm_workspace_size(int mode, int M, int N, int K, int slices, siz
     if (mode == CC_OZAKI_INT8) return CC_ERR_UNSUPPORTED;
     if (mode < CC_FP64 || mode > CC_BF16) return CC_ERR_ARG;
     if (mode == CC_OZAKI_BF16 && slices != 0 && (slices < 2 || slices > 8)) return CC_ERR_ARG;
-    *bytes = gemm_ws(mode, M, N, K, slices_of(mode, slices));
+    const int s = slices_of(mode, slices);
+    *bytes = std::max(gemm_ws(mode, M, N, K, s), gemm_ws(mode, M, N, K, s, gemm_nm(mode, K, s)));
     return CC_OK;
 }
 
@@ -1584,6 +1857,11 @@ int cc_ladder_gemm(int mode, int M, int N, int K, const double* A, int lda, cons
 {
     size_t need = 0;
     CC_TRY(cc_ladder_gemm_workspace_size(mode, M, N, K, slices, &need));
+    // the residue form where its workspace is there, the digit slices in less
+    const int ns = slices_of(mode, slices);
+    int nm = gemm_nm(mode, K, ns);
+    if (nm > 0 && ws_bytes < need) nm = 0;
+    if (nm == 0) need = gemm_ws(mode, M, N, K, ns);
     if (!A || !B || !C || !workspace) return CC_ERR_NULL;
     if (lda < K || ldb < K || ldc < N) return CC_ERR_ARG;
     if (!aligned(A, 16) || !aligned(B, 16) || !aligned(C, 16) || !aligned(workspace, 256)) return CC_ERR_ALIGN;
@@ -1609,12 +1887,22 @@ int cc_ladder_gemm(int mode, int M, int N, int K, const double* A, int lda, cons
         Carve cv;
         cv.take(256);
         Operand oa{}, ob{};
-        oa.D = at<void>(workspace, cv.take((size_t)es * c.s * M * pitch_for(K, es)));
+        const size_t stack = nm > 0 ? nm : c.s;
+        oa.D = at<void>(workspace, cv.take((size_t)es * stack * M * (nm > 0 ? pitch_crt(K) : pitch_for(K, es))));
         oa.e = at<int>(workspace, cv.take(4 * (size_t)M));
-        ob.D = at<void>(workspace, cv.take((size_t)es * c.s * N * pitch_for(K, es)));
+        ob.D = at<void>(workspace, cv.take((size_t)es * stack * N * (nm > 0 ? pitch_crt(K) : pitch_for(K, es))));
         ob.e = at<int>(workspace, cv.take(4 * (size_t)N));
         RowSrc ra{A, plain_map(lda), plain_map(1), M, K};
         RowSrc rb{B, plain_map(ldb), plain_map(1), N, K};
+        if (nm > 0) {
+            size_t res = 0;
+            gemm_ws(mode, M, N, K, c.s, nm, &res);
+            unsigned char* planes = at<unsigned char>(workspace, cv.take(res));
+            CC_TRY(prep_crt_rows(c, ra, 1, K, 0, nm, oa, st));
+            CC_TRY(prep_crt_rows(c, rb, 1, K, 0, nm, ob, st));
+            CC_TRY(run_crt_out("gemm_tc", c, nm, M, N, K, oa, ob, out, planes, res, st, 0));
+            return finish(status, 0, st);
+        }
         CC_TRY(prep_rows(c, ra, oa, st));
         CC_TRY(prep_rows(c, rb, ob, st));
         CC_TRY(run_tc("gemm_tc", c, M, N, K, oa, 0, ob, 0, out, status, st));

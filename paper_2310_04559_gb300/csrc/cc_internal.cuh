@@ -174,6 +174,47 @@ cudaError_t fill_pairs(int o, int v, int strict, long long* tab, cudaStream_t st
 cudaError_t convert_rows_tf32(const RowSrc& src, float* D, long long pitch, cudaStream_t st);
 cudaError_t convert_cols_tf32(const ColSrc& src, float* D, long long pitch, cudaStream_t st);
 
+// ------------------------------------------------- residue form of the emulated mode
+// (crt.cuh, gemm_crt.cu, crt_prep.cu)
+// Operands are bf16 residue stacks D[l][row][pitch], l < nm, with one exponent per row; K is the padded length
+// of the rows' order (crt_prep.cu).  planes: [ksplit][nm][M][pitch] bytes, pitch a multiple of 16 and >= N.
+struct GemmCrt {
+    int M, N, K, nm;
+    const void* A; long long pitchA, rowsA, rowA0;
+    const void* B; long long pitchB, rowsB, rowB0;
+    unsigned char* planes; long long pitch;
+    int ksplit;        // K split into this many partial results (1 = none)
+    int accumulate;    // add to the residues in the planes
+    long long tri;     // triangular tile skip, a(m) = m / tri, b(n) = n / tri (0 = off)
+    int* status;
+    unsigned long long wait_ns;
+};
+cudaError_t gemm_crt(const GemmCrt& g, cudaStream_t s);
+struct CrtPlanes {
+    const unsigned char* planes;
+    long long plane, pitch;  // bytes between planes, bytes per GEMM row
+    int nm;
+};
+// Rows r at src.X + rm(r), K = (o, i) at o * ostride + i, padded order o * inner4 + i.
+cudaError_t crt_rows(const RowSrc& src, int outer, int inner, long long ostride, int nm, void* D, long long pitch, int* e,
+                     int* status, cudaStream_t st);
+cudaError_t crt_cols(const ColSrc& src, int nm, void* D, long long pitch, int* e, unsigned long long* scratch_max,
+                     int* status, cudaStream_t st, bool premax = false);
+// T+ (rows_p pairs i <= j from pair q0, offsets rowtab) and T- (their rows_m pairs i < j from strict pair s0), packed
+// order crt_kq.
+cudaError_t crt_pm_f64(const double* t2, const long long* rowtab, int o, int v, long long q0, long long rows_p, long long s0,
+                       long long rows_m, int nm, void* Dp, int* ep, void* Dm, int* em, long long pitch, int* status,
+                       cudaStream_t st);
+// V+ and (Dm not NULL) V- of the rows (al, b') = rtab[r] = al * Nb + b' from planes[l][(al, c)][(b', d)], packed order.
+cudaError_t crt_pm_planes(const CrtPlanes& src, const long long* rtab, long long rows, int Nb, int v, const int* eL,
+                          int nm, void* Dp, int* ep, void* Dm, int* em, long long pitch, cudaStream_t st);
+// Rows (al, q) of K = (o, i) from planes[l][(al, o)][(q, i)]; row index al * nq + q, or q * nal + al (q_major).
+cudaError_t crt_rows_planes(const CrtPlanes& src, int nal, int nq, bool q_major, int outer, int inner, const int* eA,
+                            const int* eB, int nm, void* D, long long pitch, int* e, cudaStream_t st);
+// C[rmap(m) + cmap(n)] (= or +=) the planes' integers (summed over nsplit) times 2^(eA[m] + eB[n] + base) * factor.
+cudaError_t crt_to_f64(int M, int N, const CrtPlanes& src, int nsplit, const OutDesc& out, int base, double factor,
+                       bool mfast, const int* eA, const int* eB, cudaStream_t st);
+
 // -------------------------------------------------------------------- misc
 // R[i,j,a,b] (=|+=) Rc[p, a, b] for p = pair(i<=j), and R[j,i,b,a] likewise for i<j,
 // for a in [a_lo, a_hi).

@@ -1,0 +1,644 @@
+// gemm_crt.cu -- Blackwell (sm_103a) residue GEMM of the emulated-FP64 mode (see crt.cuh):
+//
+//   planes[l][m][n] = 128 + ( sum_k A_l(m,k) B_l(n,k) ) mod p_l (balanced),   one byte each, l = 0 .. nm-1
+//
+// for K-major bf16 residue stacks A[l][row][pitch], B[l][row][pitch] with |A|, |B| <= 128.
+//
+// One pair of SMs (a cluster of two CTAs) owns a 256 x 256 output tile of one modulus at a time and
+// issues tcgen05.mma.cta_group::2 (M = 256, N = 256, K = 16) into both SMs' tensor memory: per K-step
+// of 64 each CTA stages only its 128 rows of A and 128 rows of B (32 KB) for 512 clocks of MMAs, so the
+// copies ask for 64 B/clk/SM where 128 x 128 tiles of one CTA ask for 128.  The kernel is persistent:
+// pairs take (modulus, K-split, tile) items in raster order from a global counter, so that the items
+// resident at once share operand rows in L2.  The tile columns share N evenly in units of 32 columns: a ladder GEMM
+// has o(o+1)/2 columns, and 820 of them become 224 + 224 + 192 + 192 instead of 3 x 256 + 64 (whose last tile
+// would load 256 rows of A for 64 columns).
+//
+// Exactness: a pass covers at most kCrtChunk = 1024 K elements, so every FP32 partial sum is an integer
+// of at most 128 * 128 * 1024 = 2^24 and exact for any input.  Two 256-column accumulators (all of
+// TMEM) alternate between passes: the epilogue reduces pass p modulo p_l into registers while the MMAs of
+// pass p + 1 run, and the item's sum once more, to the byte it stores.  The reductions are packed FP32
+// (r = x - p rint(x / p), exact), 1.5 instructions per element and pass: converting to integers instead took 8000
+// clocks per tile, as long as the MMAs of K = 1000 (8192 x 8192 x 1024, 12 moduli: 1518 TFLOP/s then, see below).
+//
+// Bound: tensor pipe (power-capped).  o=40/v=400/n=2000 integral blocks: see the table in the design notes.
+//
+// Roles (384 threads): warp 0 issues the A copies and fetches items (leader CTA), warp 3 the B copies,
+// one thread of the leader's warp 2 the MMAs, warps 4-11 are the epilogue (one row and 128 columns per
+// thread).  Copies of both CTAs complete on the leader's barriers; slot releases and accumulator
+// hand-overs are multicast commits to both CTAs.
+//
+// Every wait is bounded (globaltimer); on expiry the CTA raises the pair's abort flags and the device
+// status word, waits (again bounded) for what it has in flight, frees TMEM and exits.
+#include <cuda.h>
+#include <cudaTypedefs.h>
+#include <cuda_runtime.h>
+
+#include <atomic>
+#include <mutex>
+
+#include "cc_internal.cuh"
+#include "crt.cuh"
+
+namespace cc {
+namespace {
+
+constexpr int BM = 128;                        // tile rows per CTA (256 per pair)
+constexpr int TM = 2 * BM;                     // tile rows per pair
+constexpr int TN = 256;                        // widest tile
+constexpr int KSTEP = 64;                      // bf16 elements per 128-byte swizzle atom
+constexpr int TILE_BYTES = 128 * 128;          // 128 rows x 128 bytes
+constexpr int NS = 6;                          // ring slots (one K-step of A and B each)
+constexpr int RING_BYTES = NS * 2 * TILE_BYTES;  // 192 KB
+constexpr int QN = 16;                         // item queue slots
+constexpr int kCounterSlots = 64;              // item counters, one per launch in flight
+constexpr int EPI_WARPS = 8;
+constexpr int THREADS = 128 + 32 * EPI_WARPS;  // 384
+constexpr int TMEM_COLS = 512;                 // two accumulators of 256 columns
+constexpr int CPT = TN / 2;                    // accumulator columns per epilogue thread
+constexpr int kReduceEvery = 60;               // passes between reductions of the running sums (far below 2^24)
+// setmaxnreg split of the launch's 384 x 168 registers: 128 x 56 + 256 x 216 = 62464 <= 64512
+constexpr int REG_LOW = 56, REG_HIGH = 216;
+static_assert(128 * REG_LOW + 256 * REG_HIGH <= THREADS * 168, "register split exceeds the launch's share");
+constexpr unsigned long long kSettleNs = 5000000ull;      // abort path: copies in flight land within this
+constexpr unsigned long long kDrainLimitNs = 1000000000ull;  // abort path: bound on the MMA drain
+constexpr int WARP_A = 0, WARP_MMA = 2, WARP_B = 3;
+
+__device__ int g_crt_counter[kCounterSlots];
+
+struct SmemCtl {
+    unsigned long long full[NS], empty[NS];
+    unsigned long long tfull[2], tempty[2];
+    unsigned long long drain;
+    int item_q[QN];                            // this pair's items in order (-1: no work left)
+    unsigned int items_pub;                    // items written to item_q
+    unsigned int tmem_base;
+    volatile int abort;
+};
+constexpr size_t SMEM_BYTES = 1024 + RING_BYTES + sizeof(SmemCtl);
+static_assert(SMEM_BYTES <= 227 * 1024, "shared memory");
+
+struct Params {
+    int M, N, K, nm;
+    long long rowA0, rowB0;
+    int ksplit, kper;                // K split s owns [s*kper, min(K, (s+1)*kper))
+    long long tri;                   // triangular tile skip (0 = off): b(n) = n / tri < a(m) = m / tri
+    int tiles_m, tiles_n, group_m, nitems;
+    uint32_t step_bytes;             // bytes both CTAs copy per K-step
+    int ubase, urem;                 // tile column j: ubase units of 32 columns, one more where j < urem
+    unsigned char* planes;           // [ksplit][nm][M][pitch]
+    long long pitch;
+    int accumulate;                  // add to the residues that are there (modulo p_l)
+    float inv[kCrtMax], neg[kCrtMax];  // 1 / p_l, -p_l
+    int* counter;                    // items handed out beyond the first of each pair (zero at launch)
+    int* status;
+    unsigned long long wait_ns;
+};
+
+__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+__device__ __forceinline__ uint32_t cluster_rank()
+{
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+
+// shared::cluster address of the object at the same offset in CTA `rank` of the pair
+__device__ __forceinline__ uint32_t in_cta(const void* p, uint32_t rank)
+{
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(p)), "r"(rank));
+    return r;
+}
+
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+__device__ __forceinline__ unsigned long long gtime()
+{
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return t;
+}
+
+__device__ __forceinline__ void mbar_init(unsigned long long* b, unsigned count)
+{
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(b)), "r"(count));
+}
+
+__device__ __forceinline__ bool mbar_try(unsigned long long* b, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+        " selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok)
+        : "r"(smem_u32(b)), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+
+// Raises the abort flag of both CTAs and the status word.
+__device__ __forceinline__ void raise_abort(SmemCtl* ctl, uint32_t rank, int* status)
+{
+    ctl->abort = 1;
+    asm volatile("st.volatile.shared::cluster.u32 [%0], %1;" ::"r"(in_cta((const void*)&ctl->abort, rank ^ 1)), "r"(1)
+                 : "memory");
+    atomicOr(status, kStatusWaitExpired);
+}
+
+// Bounded wait; false (and the abort flags raised) when the bound expires or another role has aborted.
+__device__ __forceinline__ bool mbar_wait(unsigned long long* b, uint32_t parity, SmemCtl* ctl, uint32_t rank,
+                                          const Params& p)
+{
+    if (mbar_try(b, parity)) return true;
+    const unsigned long long t0 = gtime();
+    for (unsigned it = 1;; ++it) {
+        if (mbar_try(b, parity)) return true;
+        if (it == 1 || (it & 7) == 0) {
+            if (ctl->abort) return false;
+            if (gtime() - t0 > p.wait_ns) {
+                raise_abort(ctl, rank, p.status);
+                return false;
+            }
+        }
+    }
+}
+
+// Item k of this pair (-1: no work left, or abort); bounded.
+__device__ __forceinline__ int item_at(SmemCtl* ctl, uint32_t k, uint32_t rank, const Params& p)
+{
+    unsigned long long t0 = 0;
+    for (unsigned it = 0;; ++it) {
+        uint32_t n;
+        asm volatile("ld.acquire.cluster.shared::cta.u32 %0, [%1];" : "=r"(n) : "r"(smem_u32(&ctl->items_pub)) : "memory");
+        if ((int)(n - k) > 0) return *(volatile int*)&ctl->item_q[k % QN];
+        if (it == 0) t0 = gtime();
+        __nanosleep(32);
+        if ((it & 15) == 15) {
+            if (ctl->abort) return -1;
+            if (gtime() - t0 > p.wait_ns) {
+                raise_abort(ctl, rank, p.status);
+                return -1;
+            }
+        }
+    }
+}
+
+__device__ __forceinline__ void mbar_expect_tx(unsigned long long* b, uint32_t bytes)
+{
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(b)), "r"(bytes) : "memory");
+}
+
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t addr)
+{
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
+}
+
+// Copy into this CTA's shared memory, completing on the barrier at shared::cluster address `bar`.
+__device__ __forceinline__ void tma_load(void* dst, const CUtensorMap* map, uint32_t bar, int x, int y, int z)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%2, %3, %4}], [%5];"
+        ::"r"(smem_u32(dst)), "l"((unsigned long long)map), "r"(x), "r"(y), "r"(z), "r"(bar)
+        : "memory");
+}
+
+// tcgen05 shared-memory matrix descriptor: K-major, 128-byte swizzle, 8-row groups 1024 bytes apart.
+__device__ __forceinline__ unsigned long long smem_desc(const void* p)
+{
+    const unsigned long long addr = smem_u32(p);
+    return ((addr >> 4) & 0x3fffull) | (1ull << 16) | ((unsigned long long)(1024 >> 4) << 32) | (1ull << 46) | (2ull << 61);
+}
+
+// FP32 accumulate, bf16 x bf16, both K-major, M = 256, N = width.
+__device__ __forceinline__ uint32_t instr_desc(int width)
+{
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(width >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
+}
+
+__device__ __forceinline__ void mma(uint32_t d, unsigned long long a, unsigned long long b, uint32_t idesc, uint32_t acc)
+{
+    asm volatile(
+        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+        " tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n"
+        ::"r"(d), "l"(a), "l"(b), "r"(idesc), "r"(acc));
+}
+
+// Arrive on `bar` (same offset) in both CTAs once this thread's prior MMAs complete.
+__device__ __forceinline__ void commit_both(unsigned long long* bar)
+{
+    asm volatile(
+        "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
+        ::"r"(smem_u32(bar)), "h"((unsigned short)3) : "memory");
+}
+
+__device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+
+// 32 lanes x 32 columns, waited for.
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32])
+{
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,"
+        "%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
+          "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+          "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        : "r"(taddr));
+}
+
+// x - p rint(x / p) of two integers |x| <= 2^24 at once: exact, and at most p / 2 + 1 in magnitude (the quotient is
+// within 2^-8 of x / p, so it is off by one at most next to a tie); at most p / 2 for |x| < 2^16.
+__device__ __forceinline__ unsigned long long reduce2(unsigned long long x, unsigned long long inv, unsigned long long neg)
+{
+    const unsigned long long big = f2(12582912.0f, 12582912.0f), nbig = f2(-12582912.0f, -12582912.0f);
+    return fma2(add2(fma2(x, inv, big), nbig), neg, x);
+}
+
+// Item i: modulus-major, then K split, then tiles rastered in groups of group_m tile rows.
+struct Item {
+    int l, split, m0, n0, width;  // width: columns of the MMAs (a multiple of 32)
+    bool skip;
+};
+
+__device__ __forceinline__ Item item_of(const Params& p, int i)
+{
+    const int ntiles = p.tiles_m * p.tiles_n;
+    const int per_l = ntiles * p.ksplit;
+    Item it;
+    it.l = i / per_l;
+    const int rem = i % per_l;
+    it.split = rem / ntiles;
+    const int t = rem % ntiles;
+    const int per_group = p.group_m * p.tiles_n;
+    const int first_m = (t / per_group) * p.group_m;
+    const int gm = min(p.tiles_m - first_m, p.group_m);
+    it.m0 = (first_m + (t % per_group) % gm) * TM;
+    const int j = (t % per_group) / gm;
+    it.n0 = 32 * (j * p.ubase + min(j, p.urem));
+    it.width = 32 * (p.ubase + (j < p.urem ? 1 : 0));
+    // every element of the tile has b(n) < a(m)
+    it.skip = p.tri > 0 && min(p.N - 1, it.n0 + it.width - 1) / (int)p.tri < it.m0 / (int)p.tri;
+    return it;
+}
+
+// Leader: publishes the pair's item k to both CTAs, `item` being the counter's answer (the first one the pair's own
+// index), moved on past skipped tiles.  Slot k % QN is free: when item k is published, every copy of item k - 2 has
+// been issued, so the MMAs of item k - 8 have completed (a ring of 6 slots, at least one per item), so both epilogues
+// have drained item k - 10 and read its queue slot before.
+__device__ __forceinline__ int publish_item(SmemCtl* ctl, const Params& p, uint32_t k, int item, int npairs)
+{
+    while (item < p.nitems && item_of(p, item).skip) item = npairs + atomicAdd(p.counter, 1);
+    if (item >= p.nitems || ctl->abort) item = -1;
+    for (uint32_t r = 0; r < 2; ++r) {
+        asm volatile("st.relaxed.cluster.shared::cluster.u32 [%0], %1;" ::"r"(in_cta(&ctl->item_q[k % QN], r)), "r"(item)
+                     : "memory");
+        asm volatile("st.release.cluster.shared::cluster.u32 [%0], %1;" ::"r"(in_cta(&ctl->items_pub, r)), "r"(k + 1)
+                     : "memory");
+    }
+    return item;
+}
+
+__global__ void __launch_bounds__(THREADS, 1)
+gemm_crt_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const Params p)
+{
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    unsigned char* base = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    unsigned char* aring = base;
+    unsigned char* bring = base + NS * TILE_BYTES;
+    SmemCtl* ctl = (SmemCtl*)(base + RING_BYTES);
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t rank = cluster_rank();
+    const int pair = (int)(blockIdx.x >> 1), npairs = (int)(gridDim.x >> 1);
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < NS; ++s) {
+            mbar_init(&ctl->full[s], 1);
+            mbar_init(&ctl->empty[s], 1);
+        }
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(&ctl->tfull[b], 1);
+            mbar_init(&ctl->tempty[b], 2 * EPI_WARPS);
+        }
+        mbar_init(&ctl->drain, 1);
+        ctl->items_pub = 0;
+        ctl->abort = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == WARP_MMA) {
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&ctl->tmem_base)),
+                     "r"(TMEM_COLS));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;");
+    }
+    fence_before();
+    __syncthreads();
+    cluster_sync();  // the peer's barriers are initialised before any copy, commit or store reaches them
+    fence_after();
+    const uint32_t tmem = ctl->tmem_base;
+
+    if (warp < 4) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REG_LOW));
+        if ((warp == WARP_A || warp == WARP_B) && lane == 0) {
+            // ------------------------------------------------------------ producers
+            const bool isA = warp == WARP_A;
+            const CUtensorMap* map = isA ? &tmA : &tmB;
+            asm volatile("prefetch.tensormap [%0];" ::"l"((unsigned long long)map) : "memory");
+            unsigned char* ring = isA ? aring : bring;
+            const bool fetcher = isA && rank == 0;
+            uint32_t u = 0;  // K-steps issued
+            bool ok = true;
+            // The fetcher publishes the item after the one being copied, and asks the counter for one more whose answer
+            // it only looks at an item later: the atomic's latency (about 1 us, as long as an item of K = 256) then
+            // overlaps the copies.
+            uint32_t pub = 0;   // items published
+            int raw = pair;     // the counter's next answer
+            bool more = true;   // no -1 published yet
+            for (uint32_t k = 0; ok; ++k) {
+                if (fetcher) {
+                    while (more && pub <= k + 1) {
+                        more = publish_item(ctl, p, pub, raw, npairs) >= 0;
+                        ++pub;
+                        if (more) raw = npairs + atomicAdd(p.counter, 1);
+                    }
+                }
+                const int item = item_at(ctl, k, rank, p);
+                if (item < 0) break;
+                const Item w = item_of(p, item);
+                const int row = isA ? (int)(p.rowA0 + w.m0) + (int)rank * BM
+                                    : (int)(p.rowB0 + w.n0) + (int)rank * (w.width >> 1);
+                const int kbeg = w.split * p.kper, kend = min(p.K, kbeg + p.kper);
+                for (int kb = kbeg; kb < kend; kb += KSTEP, ++u) {
+                    const uint32_t s = u % NS;
+                    if (!mbar_wait(&ctl->empty[s], ((u / NS) & 1) ^ 1, ctl, rank, p)) { ok = false; break; }
+                    if (fetcher) mbar_expect_tx(&ctl->full[s], p.step_bytes);  // A and B tiles of both CTAs
+                    tma_load(ring + s * TILE_BYTES, map, in_cta(&ctl->full[s], 0), kb, row, w.l);
+                }
+            }
+            // the last use of every slot is released: no commit still targets this CTA's barriers when it leaves
+            for (uint32_t q = 1; q <= NS && q <= u && ok; ++q) {
+                const uint32_t v = u - q;
+                ok = mbar_wait(&ctl->empty[v % NS], (v / NS) & 1, ctl, rank, p);
+            }
+            if (!ok) {
+                // abort: copies into this CTA's ring may still be in flight, and the two CTAs may have stopped at
+                // different K-steps, so the leader's barriers need not complete: give the copies time to land
+                const unsigned long long t0 = gtime();
+                while (gtime() - t0 < kSettleNs) __nanosleep(1000);
+            }
+        } else if (warp == WARP_MMA && rank == 0 && lane == 0) {
+            // ------------------------------------------------------------ MMA
+            const unsigned long long adesc0 = smem_desc(aring), bdesc0 = smem_desc(bring);
+            uint32_t u = 0, npass = 0;
+            bool ok = true, any = false;
+            for (uint32_t k = 0; ok; ++k) {
+                const int item = item_at(ctl, k, rank, p);
+                if (item < 0) break;
+                const Item w = item_of(p, item);
+                const uint32_t idesc = instr_desc(w.width);
+                const int kbeg = w.split * p.kper, kend = min(p.K, kbeg + p.kper);
+                for (int k0 = kbeg; k0 < kend && ok; k0 += kCrtChunk) {
+                    const int buf = (int)(npass & 1);
+                    if (!mbar_wait(&ctl->tempty[buf], ((npass >> 1) & 1) ^ 1, ctl, rank, p)) { ok = false; break; }
+                    fence_after();
+                    const uint32_t d = tmem + (uint32_t)(buf * TN);
+                    const int k1 = min(kend, k0 + kCrtChunk);
+                    uint32_t acc = 0;
+                    for (int kb = k0; kb < k1; kb += KSTEP, ++u) {
+                        const uint32_t s = u % NS;
+                        if (!mbar_wait(&ctl->full[s], (u / NS) & 1, ctl, rank, p)) { ok = false; break; }
+                        fence_after();
+                        const unsigned long long ad = adesc0 + (unsigned long long)(s * (TILE_BYTES >> 4));
+                        const unsigned long long bd = bdesc0 + (unsigned long long)(s * (TILE_BYTES >> 4));
+                        any = true;
+                        // four MMAs per 128-byte row: advance the start address by 32 bytes each
+                        mma(d, ad, bd, idesc, acc);
+                        mma(d, ad + 2, bd + 2, idesc, 1u);
+                        mma(d, ad + 4, bd + 4, idesc, 1u);
+                        mma(d, ad + 6, bd + 6, idesc, 1u);
+                        acc = 1;
+                        commit_both(&ctl->empty[s]);
+                    }
+                    if (!ok) break;
+                    commit_both(&ctl->tfull[buf]);
+                    ++npass;
+                }
+            }
+            // both buffers' last drains (the peer's arrivals land here) are done
+            for (uint32_t q = npass > 2 ? npass - 2 : 0; q < npass && ok; ++q)
+                ok = mbar_wait(&ctl->tempty[q & 1], (q >> 1) & 1, ctl, rank, p);
+            if (any) {
+                // every MMA has completed before TMEM is released
+                commit_both(&ctl->drain);
+                const unsigned long long t0 = gtime();
+                while (!mbar_try(&ctl->drain, 0)) {
+                    if (gtime() - t0 > kDrainLimitNs) { atomicOr(p.status, kStatusDrainExpired); break; }
+                }
+            }
+        }
+    } else {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REG_HIGH));
+        // ------------------------------------------------------------ epilogue
+        // Warp 4 + e reads TMEM lanes 32 (warp % 4) .. + 31 (one tile row per thread) and columns
+        // 128 (e / 4) .. + 127.
+        const int q4 = warp & 3, half = (warp - 4) >> 2;
+        const int row = (int)rank * BM + q4 * 32 + lane;
+        const int col0 = half * CPT;
+        const uint32_t tl = tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)col0;
+        uint32_t npass = 0;
+        unsigned long long sum[CPT / 2];  // two columns each
+        bool ok = true;
+        for (uint32_t k = 0; ok; ++k) {
+            int item = -1;
+            if (lane == 0) item = item_at(ctl, k, rank, p);
+            item = __shfl_sync(0xffffffffu, item, 0);
+            if (item < 0) break;
+            const Item w = item_of(p, item);
+            const unsigned long long inv = f2(p.inv[w.l], p.inv[w.l]), neg = f2(p.neg[w.l], p.neg[w.l]);
+            const int kbeg = w.split * p.kper, kend = min(p.K, kbeg + p.kper);
+            int pass = 0;
+            for (int k0 = kbeg; k0 < kend; k0 += kCrtChunk, ++pass, ++npass) {
+                const int buf = (int)(npass & 1);
+                if (lane == 0) ok = mbar_wait(&ctl->tfull[buf], (npass >> 1) & 1, ctl, rank, p);
+                ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
+                if (!ok) break;
+                fence_after();
+#pragma unroll
+                for (int c = 0; c < CPT; c += 32) {
+                    if (col0 + c < w.width) {  // (uniform over the warp)
+                        uint32_t r[32];
+                        tmem_ld32(tl + (uint32_t)(buf * TN + c), r);
+#pragma unroll
+                        for (int q = 0; q < 16; ++q) {
+                            const unsigned long long x =
+                                reduce2(f2(__uint_as_float(r[2 * q]), __uint_as_float(r[2 * q + 1])), inv, neg);
+                            sum[c / 2 + q] = pass == 0 ? x : add2(sum[c / 2 + q], x);
+                        }
+                    }
+                }
+                fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive_cluster(in_cta(&ctl->tempty[buf], 0));
+                if (pass % kReduceEvery == kReduceEvery - 1) {
+#pragma unroll
+                    for (int q = 0; q < CPT / 2; ++q) sum[q] = reduce2(sum[q], inv, neg);
+                }
+            }
+            if (!ok) break;
+            const int m = w.m0 + row;
+            unsigned char* dst = p.planes + ((long long)(w.split * p.nm + w.l) * p.M + m) * p.pitch + w.n0 + col0;
+            if (m < p.M) {
+#pragma unroll
+                for (int c = 0; c < CPT; c += 16) {
+                    if (w.n0 + col0 + c >= p.pitch || col0 + c >= w.width) continue;
+                    uint32_t o[4];
+                    uint4 old = make_uint4(0, 0, 0, 0);
+                    if (p.accumulate) old = *reinterpret_cast<const uint4*>(dst + c);
+                    const uint32_t ov[4] = {old.x, old.y, old.z, old.w};
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        unsigned long long x[2];
+#pragma unroll
+                        for (int e = 0; e < 2; ++e) {
+                            x[e] = sum[c / 2 + 2 * q + e];
+                            if (p.accumulate)
+                                x[e] = add2(x[e], f2((float)((ov[q] >> (16 * e)) & 255u) - 128.0f,
+                                                     (float)((ov[q] >> (16 * e + 8)) & 255u) - 128.0f));
+                            // 2^23 + 128 + r: the low byte is 128 + r (r = 128, modulo 256 only, wraps to -128)
+                            x[e] = add2(reduce2(x[e], inv, neg), f2(8388736.0f, 8388736.0f));
+                        }
+                        o[q] = __byte_perm(__byte_perm((uint32_t)x[0], (uint32_t)(x[0] >> 32), 0x0040),
+                                           __byte_perm((uint32_t)x[1], (uint32_t)(x[1] >> 32), 0x0040), 0x5410);
+                    }
+                    *reinterpret_cast<uint4*>(dst + c) = make_uint4(o[0], o[1], o[2], o[3]);
+                }
+            }
+        }
+    }
+
+    fence_before();
+    __syncthreads();
+    cluster_sync();  // no CTA leaves while its peer may still read its shared memory or signal it
+    fence_after();
+    if (warp == WARP_MMA) {
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS));
+    }
+}
+
+PFN_cuTensorMapEncodeTiled_v12000 get_encode()
+{
+    static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
+    static std::once_flag once;
+    std::call_once(once, [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+            q == cudaDriverEntryPointSuccess)
+            fn = (PFN_cuTensorMapEncodeTiled_v12000)f;
+    });
+    return fn;
+}
+
+// 3-D map over a residue stack [nm][rows][pitch], extent K in the inner dimension; boxes of 64 x box_rows.
+bool make_map(CUtensorMap* m, const void* base, long long K, long long pitch, long long rows, int nm, int box_rows)
+{
+    auto enc = get_encode();
+    if (!enc) return false;
+    cuuint64_t dims[3] = {(cuuint64_t)K, (cuuint64_t)rows, (cuuint64_t)nm};
+    cuuint64_t strides[2] = {(cuuint64_t)(pitch * 2), (cuuint64_t)(pitch * 2 * rows)};
+    cuuint32_t box[3] = {(cuuint32_t)KSTEP, (cuuint32_t)box_rows, 1};
+    cuuint32_t estr[3] = {1, 1, 1};
+    return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+}  // namespace
+
+cudaError_t gemm_crt(const GemmCrt& g, cudaStream_t s)
+{
+    if (g.M <= 0 || g.N <= 0) return cudaSuccess;
+    if (g.K <= 0 || g.nm < 1 || g.nm > kCrtMax || g.pitch < g.N || g.pitch % 16 || g.tri < 0) return cudaErrorInvalidValue;
+    Params p{};
+    p.M = g.M; p.N = g.N; p.K = g.K; p.nm = g.nm;
+    p.rowA0 = g.rowA0; p.rowB0 = g.rowB0;
+    p.ksplit = g.ksplit > 1 ? g.ksplit : 1;
+    p.kper = (int)((((long long)g.K + p.ksplit - 1) / p.ksplit + KSTEP - 1) / KSTEP * KSTEP);
+    if ((long long)p.kper * (p.ksplit - 1) >= g.K || (p.ksplit > 1 && g.accumulate)) return cudaErrorInvalidValue;
+    p.tri = g.tri;
+    p.planes = g.planes;
+    p.pitch = g.pitch;
+    p.accumulate = g.accumulate;
+    for (int l = 0; l < g.nm; ++l) {
+        p.inv[l] = 1.0f / (float)crt_p(l);
+        p.neg[l] = -(float)crt_p(l);
+    }
+    p.status = g.status;
+    p.wait_ns = g.wait_ns;
+    p.tiles_m = (g.M + TM - 1) / TM;
+    p.tiles_n = (g.N + TN - 1) / TN;
+    const int units = (g.N + 31) / 32;
+    p.ubase = units / p.tiles_n;
+    p.urem = units % p.tiles_n;
+    p.group_m = p.tiles_m < 8 ? p.tiles_m : 8;
+    const long long nitems = (long long)p.tiles_m * p.tiles_n * p.ksplit * g.nm;
+    if (nitems > 0x7fffffffll - (1 << 20)) return cudaErrorInvalidConfiguration;
+    p.nitems = (int)nitems;
+
+    cudaLaunchConfig_t cfg{};
+    cfg.blockDim = dim3(THREADS);
+    cfg.dynamicSmemBytes = SMEM_BYTES;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    static std::once_flag once;
+    static cudaError_t attr_err = cudaSuccess;
+    static int max_pairs = 0;
+    std::call_once(once, [&cfg] {
+        attr_err = cudaFuncSetAttribute(gemm_crt_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
+        // persistent: as many pairs as are resident on the device at once
+        int n = 0;
+        cfg.gridDim = dim3(2 * 64);
+        if (attr_err != cudaSuccess || cudaOccupancyMaxActiveClusters(&n, gemm_crt_kernel, &cfg) != cudaSuccess || n <= 0) {
+            cudaGetLastError();
+            n = device_sm_count() / 2;
+        }
+        max_pairs = n;
+    });
+    if (attr_err != cudaSuccess) return attr_err;
+
+    // item counter: a slot of a small ring (launches in flight on other streams take other slots), zeroed in
+    // stream order before the launch
+    static std::atomic<unsigned> next_slot{0};
+    int* counters = nullptr;
+    cudaError_t err = cudaGetSymbolAddress((void**)&counters, g_crt_counter);
+    if (err != cudaSuccess) return err;
+    p.counter = counters + (next_slot.fetch_add(1) % kCounterSlots);
+    err = cudaMemsetAsync(p.counter, 0, sizeof(int), s);
+    if (err != cudaSuccess) return err;
+    CUtensorMap ma, mb;
+    // (narrow tiles, N <= 224, are bound by the copies: B's boxes hold only the rows a tile uses)
+    const int brows = 16 * (p.ubase + (p.urem > 0 ? 1 : 0));
+    p.step_bytes = 2u * (uint32_t)(TILE_BYTES + brows * 128);
+    if (!make_map(&ma, g.A, g.K, g.pitchA, g.rowsA, g.nm, BM) || !make_map(&mb, g.B, g.K, g.pitchB, g.rowsB, g.nm, brows))
+        return cudaErrorInvalidValue;
+    const int pairs = p.nitems < max_pairs ? p.nitems : max_pairs;
+    cfg.gridDim = dim3((unsigned)(2 * pairs));
+    err = cudaLaunchKernelEx(&cfg, gemm_crt_kernel, ma, mb, p);
+    if (err != cudaSuccess) return err;
+    count_launch();
+    return cudaGetLastError();
+}
+
+}  // namespace cc
