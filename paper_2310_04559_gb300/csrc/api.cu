@@ -76,7 +76,9 @@ struct Ctx {
     int mode, order, flags, s;
     bool sym, exch;
     long long pairs;  // GEMM rows for (i,j)
-    bool packed;      // pair-symmetric integral-first tensor-core path (R+ / R- over c <= d)
+    bool packed;      // integral-first on the c <-> d symmetric / antisymmetric parts (R+ / R- over c <= d)
+    bool gen = false; // packed without pair symmetry of t2: all o^2 pairs have a T+ and a T- row
+    bool part = false; // gen, a range of `a` only: integral rows (a, all b) instead of (a, b >= a)
     long long pp, pm; // packed path: pairs i <= j and i < j
     long long Kp, Km; // packed path: v(v+1)/2 and v(v-1)/2
     bool host;        // t2 and R are page-locked host memory, read and written over the host link
@@ -91,7 +93,7 @@ struct Ctx {
 };
 
 // Blocks of `a` values [a0, a0 + Ab) covering [alo, ahi).  Unpacked paths: Ab = P
-// for every block.  Packed path: a block holds the integrals (a, b >= a0), so its
+// for every block; packed without pair symmetry: Ab = P / v.  Packed path: a block holds the integrals (a, b >= a0), so its
 // size is Ab * (v - a0) rows; P bounds that product and blocks widen as a0 grows.
 std::vector<std::pair<int, int>> block_list(const Ctx& c, long long P, int alo, int ahi, int forced)
 {
@@ -99,6 +101,7 @@ std::vector<std::pair<int, int>> block_list(const Ctx& c, long long P, int alo, 
     for (int a0 = alo; a0 < ahi;) {
         int Ab;
         if (!c.packed) Ab = (int)std::min<long long>(P, ahi - a0);
+        else if (c.gen) Ab = (int)std::min<long long>(P / c.v, ahi - a0);
         else if (forced > 0) Ab = std::min(forced, ahi - a0);
         else Ab = (int)std::max(1ll, std::min<long long>(P / (c.v - a0), ahi - a0));
         out.emplace_back(a0, Ab);
@@ -341,11 +344,28 @@ long long pick_block_form(Ctx& c, size_t bytes, int requested, size_t* need)
     }
 }
 
+// Packed path for amplitudes without pair symmetry.  For any t2, T+-[ij] = t_ijcd +- t_ijdc over c <= d and the V+-
+// of b >= a give R_ijab = R+ + R- and R_ijba = R+ - R- ((ac|bd) = (bd|ac)), so half the integrals and half the ladder
+// GEMM of the unpacked product do.  A range of `a` (part) writes R[i,j,a,b] for all b, so it builds the rows (a, all b):
+// the unpacked product's work, and bit for bit the entries of the whole (residue form; FP64 ranges run unpacked).
+void set_gen(Ctx* c, bool on)
+{
+    c->gen = c->packed = on;
+    c->pp = on ? c->pairs : (long long)c->o * (c->o + 1) / 2;
+    c->pm = on ? c->pairs : (long long)c->o * (c->o - 1) / 2;
+    c->PB = c->pp;
+}
+
 // The residue form needs up to about twice the slices' memory (bf16 residues for 12 or 13 moduli instead of 6
 // digits): where it does not fit -- or, with host-resident amplitudes, would not hold all pairs at once next to
 // blocks of 4 `a` values, so that t2 would be split again for every block -- the digit slices run as before.
 long long pick_block(Ctx& c, size_t bytes, int requested, size_t* need)
 {
+    if (c.gen) {
+        const long long P = pick_block_form(c, bytes, requested, need);
+        if (P >= 0) return P;
+        set_gen(&c, false);
+    }
     if (c.crt) {
         Ctx t = c;
         const long long P = pick_block_form(t, bytes, requested, need);
@@ -392,6 +412,10 @@ long long pick_block_pb(const Ctx& c, size_t bytes, int requested, size_t* need)
         const long long nb = (c.v + lo - 1) / lo;
         P = (c.v + nb - 1) / nb;
     }
+    if (c.gen) {  // uniform blocks, evened out
+        const long long nb = (c.v + lo / c.v - 1) / (lo / c.v);
+        P = (c.v + nb - 1) / nb * c.v;
+    }
     *need = layout_fwd(c, P).total;
     return P;
 }
@@ -405,7 +429,8 @@ void set_crt(Ctx* c, long long K1, long long K2)
     c->crt = c->mode == CC_OZAKI_BF16 && c->s == kDefaultSlices && c->nm1 > 0 && c->nm2 > 0 && 4 * K2 < (1ll << 31);
 }
 
-int make_ctx(const cc_ladder_args* a, Ctx* c)
+// tuning: a partial range stands for the whole one (cc_ladder_autotune's trials)
+int make_ctx(const cc_ladder_args* a, Ctx* c, bool tuning = false)
 {
     if (!a) return CC_ERR_NULL;
     if (a->o < 1 || a->v < 1 || a->n_chol < 1) return CC_ERR_SHAPE;
@@ -436,10 +461,18 @@ int make_ctx(const cc_ladder_args* a, Ctx* c)
     // the order's cost model sees the packed flop count
     const bool can_pack = c->sym;
     c->packed = can_pack;
-    // host-resident amplitudes and streamed L run through the integral-first order only
+    const long long vv = (long long)a->v * a->v;
     const bool hostflags = (a->flags & (CC_FLAG_HOST_T2R | CC_FLAG_HOST_L)) != 0;
+    // without pair symmetry: FP64 and the residue form (the mixed modes' results would round differently)
+    set_crt(c, a->n_chol, vv);
+    const bool whole = a->a_hi == 0 || (a->a_lo == 0 && a->a_hi == a->v);
+    const bool can_gen = !c->sym && !hostflags && (a->mode == CC_FP64 ? whole || tuning : c->crt);
+    c->part = can_gen && !whole && !tuning;
+    if (can_gen) set_gen(c, true);
+    // host-resident amplitudes and streamed L run through the integral-first order only
     c->order = (hostflags && a->order == CC_ORDER_AUTO) ? (int)CC_ORDER_INTEGRAL_FIRST : pick_order(*c, a->order);
-    c->packed = can_pack && c->order == CC_ORDER_INTEGRAL_FIRST;
+    c->packed = (can_pack || can_gen) && c->order == CC_ORDER_INTEGRAL_FIRST;
+    if (can_gen) set_gen(c, c->packed);
     c->host = (a->flags & CC_FLAG_HOST_T2R) != 0;
     c->PB = c->pp;
     c->hostL = (a->flags & CC_FLAG_HOST_L) != 0;
@@ -449,7 +482,6 @@ int make_ctx(const cc_ladder_args* a, Ctx* c)
     if (c->hostL && !c->packed) return CC_ERR_UNSUPPORTED;
     // K of the two contractions
     const bool integral_first = c->order == CC_ORDER_INTEGRAL_FIRST;
-    const long long vv = (long long)a->v * a->v;
     set_crt(c, integral_first ? a->n_chol : a->v, integral_first ? vv : (long long)a->n_chol * a->v);
     return CC_OK;
 }
@@ -767,8 +799,10 @@ int fwd_packed(const Ctx& c, const cc_ladder_args* a, const double* Lsrc, const 
     long long* pairtab = at<long long>(ws, Lo.pairtab);
     long long* pairtab_m = at<long long>(ws, Lo.pairtab_m);
     long long* rtab = at<long long>(ws, Lo.rtab);
-    CC_CU(fill_pairs(c.o, c.v, 0, pairtab, st));
-    CC_CU(fill_pairs(c.o, c.v, 1, pairtab_m, st));
+    if (!c.gen) {
+        CC_CU(fill_pairs(c.o, c.v, 0, pairtab, st));
+        CC_CU(fill_pairs(c.o, c.v, 1, pairtab_m, st));
+    }
     const bool minus = c.pm > 0 && c.Km > 0;
 
     Operand Lw{}, Tp{}, Tm{}, Vp{}, Vm{};
@@ -840,6 +874,7 @@ int fwd_packed(const Ctx& c, const cc_ladder_args* a, const double* Lsrc, const 
     // enumeration (s(p) = p - i - [j > i] pairs i < j precede pair p = (i, j)).
     auto strict_before = [&](long long p) -> long long {
         if (p >= c.pp) return c.pm;
+        if (c.gen) return p;
         long long i = 0, rem = p;
         while (rem >= c.o - i) { rem -= c.o - i; ++i; }
         return p - i - (rem > 0 ? 1 : 0);
@@ -853,8 +888,14 @@ int fwd_packed(const Ctx& c, const cc_ladder_args* a, const double* Lsrc, const 
         Tp.rows = q1 - q0;
         Tm.rows = s1 - s0;
         if (c.crt)
-            return check_cuda(crt_pm_f64(t2, pairtab + q0, c.o, c.v, q0, q1 - q0, s0, minus ? s1 - s0 : 0, c.nm2, Tp.D, Tp.e,
+            return check_cuda(crt_pm_f64(t2, c.gen ? nullptr : pairtab + q0, c.o, c.v, q0, q1 - q0, s0, minus ? s1 - s0 : 0, c.nm2, Tp.D, Tp.e,
                                          Tm.D, Tm.e, Tp.pitch, c.status, st));
+        if (c.gen) {
+            CC_CU(pm_split_f64(t2, nullptr, vv, q1 - q0, c.v, +1, 1.0, kind, c.s, kBeta, Tp.D, Tp.pitch, Tp.e, c.status, st));
+            if (minus)
+                CC_CU(pm_split_f64(t2, nullptr, vv, q1 - q0, c.v, -1, 1.0, kind, c.s, kBeta, Tm.D, Tm.pitch, Tm.e, c.status, st));
+            return CC_OK;
+        }
         CC_CU(pm_split_f64(t2, pairtab + q0, 1, q1 - q0, c.v, +1, 1.0, kind, c.s, kBeta, Tp.D, Tp.pitch, Tp.e, c.status, st));
         if (minus && s1 > s0)
             CC_CU(pm_split_f64(t2, pairtab_m + s0, 1, s1 - s0, c.v, -1, 1.0, kind, c.s, kBeta, Tm.D, Tm.pitch, Tm.e,
@@ -867,8 +908,9 @@ int fwd_packed(const Ctx& c, const cc_ladder_args* a, const double* Lsrc, const 
     double* Rmc = at<double>(ws, Lo.Rmc);
     const int accum = (c.flags & CC_FLAG_ACCUMULATE) ? 1 : 0;
     for (const auto& blk : block_list(c, P, alo, ahi, a->a_block)) {
-        const int a0 = blk.first, Ab = blk.second, Nb = c.v - a0;
-        const long long nr = (long long)Ab * Nb - (long long)Ab * (Ab - 1) / 2;
+        const int a0 = blk.first, Ab = blk.second;
+        const int b0 = c.part ? 0 : a0, Nb = c.v - b0;
+        const long long nr = c.part ? (long long)Ab * Nb : (long long)Ab * Nb - (long long)Ab * (Ab - 1) / 2;
         // KG1: V[al][b'][c][d] = sum_P L[P, a0+al, c] L[P, a0+b', d], tiles with b < a skipped
         OutDesc o1{V, split_map(v, (long long)Nb * vv, v), split_map(v, vv, 1), 0};
         CrtPlanes vpl{};  // residue form: planes[l][(al, c)][(b', d)]
@@ -914,18 +956,19 @@ int fwd_packed(const Ctx& c, const cc_ladder_args* a, const double* Lsrc, const 
             g.tri = v;
             CC_TRY(run_f64("kg1_f64", g, st, tri_elems(g.M, g.N, v, 64, 64)));
         } else if (c.crt) {
-            CC_TRY(run_crt("kg1_tc", c, c.nm1, Ab * c.v, Nb * c.v, c.n, Lw, (long long)a0 * v, Lw, (long long)a0 * v,
-                           (unsigned char*)V, &vpl, st, v));
+            CC_TRY(run_crt("kg1_tc", c, c.nm1, Ab * c.v, Nb * c.v, c.n, Lw, (long long)a0 * v, Lw, (long long)b0 * v,
+                           (unsigned char*)V, &vpl, st, c.part ? 0 : v));
         } else {
             CC_TRY(run_tc("kg1_tc", c, Ab * c.v, Nb * c.v, c.n, Lw, (long long)a0 * v, Lw, (long long)a0 * v, o1,
                           status, st, true, v));
         }
-        CC_CU(fill_rtab(Ab, Nb, rtab, st));
+        if (!c.part) CC_CU(fill_rtab(Ab, Nb, rtab, st));
         Vp.rows = nr; Vm.rows = nr;
         {
             ProfScope ps("split", st);
             if (c.crt) {
-                CC_CU(crt_pm_planes(vpl, rtab, nr, Nb, c.v, Lw.e + (long long)a0 * v, c.nm2, Vp.D, Vp.e,
+                CC_CU(crt_pm_planes(vpl, c.part ? nullptr : rtab, nr, Nb, c.v, Lw.e + (long long)a0 * v,
+                                    Lw.e + (long long)b0 * v, a0 - b0, c.nm2, Vp.D, Vp.e,
                                     minus ? Vm.D : nullptr, minus ? Vm.e : nullptr, Vp.pitch, st));
             } else if (ozaki) {
                 // V[al][b'][c][d] = X * 2^(eL[(a0+al)v + c] + eL[(a0+b')v + d] + base)
@@ -964,17 +1007,19 @@ int fwd_packed(const Ctx& c, const cc_ladder_args* a, const double* Lsrc, const 
                 if (mb) CC_TRY(run_tc("kg2_tc", c, (int)(s1 - s0), (int)nr, (int)c.Km, Tm, 0, Vm, 0, om, status, st));
             }
             ProfScope ps("scatter", st);
-            CC_CU(pm_combine(c.o, c.v, a0, Ab, Nb, nr, q0, q1, s0, Rpc, mb ? Rmc : nullptr, a->R, accum, st));
+            if (c.part) CC_CU(pm_combine_rows(c.pp, c.v, a0, nr, Rpc, mb ? Rmc : nullptr, a->R, accum, st));
+            else if (c.gen) CC_CU(pm_combine_general(c.pp, c.v, a0, Ab, Nb, nr, Rpc, mb ? Rmc : nullptr, a->R, accum, st));
+            else CC_CU(pm_combine(c.o, c.v, a0, Ab, Nb, nr, q0, q1, s0, Rpc, mb ? Rmc : nullptr, a->R, accum, st));
         }
     }
     return CC_OK;
 }
 
-int fwd_impl(const cc_ladder_args* a, const double* Lsrc_override = nullptr)
+int fwd_impl(const cc_ladder_args* a, bool tuning = false)
 {
     Ctx c;
-    CC_TRY(make_ctx(a, &c));
-    const double* Lsrc = Lsrc_override ? Lsrc_override : a->L;
+    CC_TRY(make_ctx(a, &c, tuning));
+    const double* Lsrc = a->L;
     if (!Lsrc || !a->t2 || !a->R || !a->workspace) return CC_ERR_NULL;
     if (!aligned(Lsrc, 16) || !aligned(a->t2, 16) || !aligned(a->R, 16) || !aligned(a->workspace, 256) ||
         (a->energy && !aligned(a->energy, 8)))
@@ -1019,7 +1064,7 @@ int fwd_impl(const cc_ladder_args* a, const double* Lsrc_override = nullptr)
     const int alo = a->a_hi ? a->a_lo : 0, ahi = a->a_hi ? a->a_hi : c.v;
     // an a-range's share of the energy is defined where the range owns both R_ijab and R_ijba of
     // its terms: the packed path (entries with min(a, b) in the range)
-    if (a->energy && (alo != 0 || ahi != c.v) && !c.packed) return CC_ERR_UNSUPPORTED;
+    if (a->energy && (alo != 0 || ahi != c.v) && (!c.packed || c.gen)) return CC_ERR_UNSUPPORTED;
     CC_CU(cudaMemsetAsync(status, 0, 256, st));
 
     const double* t2 = a->t2;
@@ -1424,13 +1469,12 @@ int bwd_plan(int o, int v, int n, int mode, int flags, int slices, size_t bytes,
     // integral block and the M1 block) such that everything fits; in the residue form if one `a` fits
     // there, in digit slices otherwise (the nested forward then takes the same form: its own smallest plan
     // is at least the one counted here).
-    Ctx cf = c;  // the nested forward (K = n, then v^2)
+    Ctx cf = c;  // the nested forward (K = n, then v^2), without pair symmetry: packed where that fits
     set_crt(&c, (long long)o * o, (long long)v * v);
     c.crt = cf.crt = c.crt && cf.crt;
-    auto total_for = [&](int A) {
-        const size_t fb = layout_fwd(cf, A).total;
-        return layout_bwd(c, A, fb, sym).total;
-    };
+    auto fwd_bytes = [&](int A) { return layout_fwd(cf, cf.gen ? (long long)A * v : A).total; };
+    auto total_for = [&](int A) { return layout_bwd(c, A, fwd_bytes(A), sym).total; };
+    if (cf.gen && (!(c.crt || mode == CC_FP64) || total_for(1) > bytes)) set_gen(&cf, false);
     if (c.crt && total_for(1) > bytes) c.crt = cf.crt = false;
     if (total_for(1) > bytes) return for_query ? CC_ERR_BUDGET : CC_ERR_WORKSPACE;
     int lo = 1, hi = v;
@@ -1442,7 +1486,7 @@ int bwd_plan(int o, int v, int n, int mode, int flags, int slices, size_t bytes,
     const int A = (v + nb - 1) / nb;
     bp->c = c;
     bp->E = A;
-    bp->fwd_bytes = layout_fwd(cf, A).total;
+    bp->fwd_bytes = fwd_bytes(A);
     bp->L = layout_bwd(c, A, bp->fwd_bytes, sym);
     bp->fa = fa;
     bp->fa.a_block = A;
@@ -1677,7 +1721,8 @@ int cc_ladder_partition(const cc_ladder_args* args, int parts, int* bounds)
     // and the ladder columns of the same pairs, so its work is proportional to v - a; on the other
     // paths every `a` costs the same.
     const double v = c.v;
-    auto W = [&](int a) { return c.packed ? (double)a * v - (double)a * (a - 1) / 2.0 : (double)a; };
+    const bool tri = c.packed && !c.gen;  // (a range of one without pair symmetry runs unpacked)
+    auto W = [&](int a) { return tri ? (double)a * v - (double)a * (a - 1) / 2.0 : (double)a; };
     const double total = W(c.v);
     bounds[0] = 0;
     for (int g = 1; g < parts; ++g) {
@@ -1713,7 +1758,7 @@ int cc_ladder_autotune(const cc_ladder_args* args, cc_ladder_plan* plan, double*
         a.energy = nullptr;
         a.flags &= ~CC_FLAG_ACCUMULATE;
         Ctx cq;
-        make_ctx(&a, &cq);
+        make_ctx(&a, &cq, true);
         size_t need = 0;
         const long long P = pick_block(cq, a.ws_bytes, a.a_block, &need);
         if (P < 0) continue;  // this order does not fit the workspace
@@ -1726,10 +1771,10 @@ int cc_ladder_autotune(const cc_ladder_args* args, cc_ladder_plan* plan, double*
         for (int r = 0; r < reps && status == CC_OK; ++r) {
             a.a_lo = 0;
             a.a_hi = blocks[r].first + blocks[r].second;
-            status = fwd_impl(&a);  // warm (first use of the shape)
+            status = fwd_impl(&a, true);  // warm (first use of the shape)
             if (status != CC_OK) break;
             cudaEventRecord(e0, st);
-            status = fwd_impl(&a);
+            status = fwd_impl(&a, true);
             cudaEventRecord(e1, st);
             if (status != CC_OK) break;
             cudaEventSynchronize(e1);

@@ -168,6 +168,13 @@ cudaError_t fill_rtab(int Ab, int Nb, long long* rtab, cudaStream_t st);
 // Rp[p - q0][r]; Rm[s(p) - s0][r] for their pairs i < j (s = index among the pairs i < j).
 cudaError_t pm_combine(int o, int v, int a0, int Ab, int Nb, long long nr, long long q0, long long q1, long long s0,
                        const double* Rp, const double* Rm, double* R, int accumulate, cudaStream_t st);
+// R[p, a, b] (=|+=) R+ + R-, R[p, b, a] (=|+=) R+ - R- for the block a = a0 + al, b = a0 + b' >= a and the
+// `pairs` rows p = i o + j of Rp and Rm (amplitudes without pair symmetry).
+cudaError_t pm_combine_general(long long pairs, int v, int a0, int Ab, int Nb, long long nr, const double* Rp,
+                               const double* Rm, double* R, int accumulate, cudaStream_t st);
+// R[p, a, b] (=|+=) R+ + R- (b >= a), R+ - R- (b < a) for the rows r = al v + b, a = a0 + al, of Rp and Rm.
+cudaError_t pm_combine_rows(long long pairs, int v, int a0, long long nr, const double* Rp, const double* Rm, double* R,
+                            int accumulate, cudaStream_t st);
 // tab = (i*o + j) * v*v for the pairs i < j (strict = 1) or i <= j (strict = 0), i-major
 cudaError_t fill_pairs(int o, int v, int strict, long long* tab, cudaStream_t st);
 // Plain fp64 -> tf32 (stored as fp32) copies, K-major.
@@ -201,13 +208,15 @@ cudaError_t crt_rows(const RowSrc& src, int outer, int inner, long long ostride,
 cudaError_t crt_cols(const ColSrc& src, int nm, void* D, long long pitch, int* e, unsigned long long* scratch_max,
                      int* status, cudaStream_t st, bool premax = false);
 // T+ (rows_p pairs i <= j from pair q0, offsets rowtab) and T- (their rows_m pairs i < j from strict pair s0), packed
-// order crt_kq.
+// order crt_kq; rowtab NULL: the rows_p = rows_m pairs p, offsets p v^2.
 cudaError_t crt_pm_f64(const double* t2, const long long* rowtab, int o, int v, long long q0, long long rows_p, long long s0,
                        long long rows_m, int nm, void* Dp, int* ep, void* Dm, int* em, long long pitch, int* status,
                        cudaStream_t st);
-// V+ and (Dm not NULL) V- of the rows (al, b') = rtab[r] = al * Nb + b' from planes[l][(al, c)][(b', d)], packed order.
-cudaError_t crt_pm_planes(const CrtPlanes& src, const long long* rtab, long long rows, int Nb, int v, const int* eL,
-                          int nm, void* Dp, int* ep, void* Dm, int* em, long long pitch, cudaStream_t st);
+// V+ and (Dm not NULL) V- of the rows (al, b') = rtab[r] = al * Nb + b' (rtab NULL: r) from planes[l][(al, c)][(b', d)],
+// packed order, exponents eA[al v + c] + eB[b' v + d].  Rows with b' < al + diag get the V- of (b, a) instead (V-_ba =
+// -V-_ab up to the rounding of ties: this way a pair's row is the same bits wherever it is built).
+cudaError_t crt_pm_planes(const CrtPlanes& src, const long long* rtab, long long rows, int Nb, int v, const int* eA,
+                          const int* eB, int diag, int nm, void* Dp, int* ep, void* Dm, int* em, long long pitch, cudaStream_t st);
 // Rows (al, q) of K = (o, i) from planes[l][(al, o)][(q, i)]; row index al * nq + q, or q * nal + al (q_major).
 cudaError_t crt_rows_planes(const CrtPlanes& src, int nal, int nq, bool q_major, int outer, int inner, const int* eA,
                             const int* eB, int nm, void* D, long long pitch, int* e, cudaStream_t st);

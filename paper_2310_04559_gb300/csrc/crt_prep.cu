@@ -351,7 +351,7 @@ struct TilePair {
     __device__ bool ok() const { return tc < nt; }
 };
 
-// T+ and T- of the pairs i <= j: row p of D+ holds t_cd + t_dc (the diagonal t_cc), row p - (i + 1) - s0 of D-
+// T+ and T- of the pairs i <= j (rowtab NULL: of all pairs, each with both rows): row p of D+ holds t_cd + t_dc (the diagonal t_cc), row p - (i + 1) - s0 of D-
 // (pairs i < j) holds t_cd - t_dc; each with its own row exponent.
 struct PmRows {
     const double* X;
@@ -370,12 +370,12 @@ __global__ void __launch_bounds__(NT) crt_pm_f64_kernel(const PmRows a, int nm, 
     const uint32_t cs = cluster_size(), rank = cluster_rank();
     const long long r = blockIdx.x / cs;
     const int v = a.v, v4 = (v + 3) & ~3;
-    const long long off = a.rowtab[r];
+    const long long off = a.rowtab ? a.rowtab[r] : r * (long long)v * v;
     const double* X = a.X + off;
     const long long ij = off / ((long long)v * v);
     const int i = (int)(ij / a.o), j = (int)(ij % a.o);
-    const bool minus = i < j && Dm != nullptr;
-    const long long rm = a.q0 + r - (i + 1) - a.s0;
+    const bool minus = (i < j || !a.rowtab) && Dm != nullptr;
+    const long long rm = a.rowtab ? a.q0 + r - (i + 1) - a.s0 : r;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const int qy = threadIdx.x >> 3, qx = (threadIdx.x & 7) * 4;
     const int nt = (v + TT - 1) / TT;
@@ -436,15 +436,16 @@ __global__ void __launch_bounds__(NT) crt_pm_f64_kernel(const PmRows a, int nm, 
 }
 
 // V+ and V- of the integral rows (a, b >= a) of one block from the byte planes of the integral GEMM,
-// planes[l][(al, c)][(b', d)], each element's fraction y scaled by 2^(eL[al v + c] + eL[b' v + d]) (eL of the block's
-// first row; the factor CrtRec::frac is left to the result).  Both halves share the row exponent E of the largest |V|,
+// planes[l][(al, c)][(b', d)], each element's fraction y scaled by 2^(eA[al v + c] + eB[b' v + d]) (the factor CrtRec::frac is left to the result).  Both halves share the row exponent E of the largest |V|,
 // as Y = round(V 2^(43 - E)) (one guard bit), V+- = (Y1 +- Y2) / 4.
 struct PmPlanes {
     const unsigned char* planes;
     long long plane, pitch_in;  // bytes between planes, per GEMM row
-    const long long* rtab;      // packed row -> al * Nb + b'
+    const long long* rtab;      // packed row -> al * Nb + b' (NULL: itself)
     int Nb, v;
-    const int* eL;
+    const int* eA;
+    const int* eB;
+    int diag;                   // b' < al + diag: V- of (b, a)
 };
 
 template <bool AL, bool WIDE>
@@ -459,15 +460,16 @@ __global__ void __launch_bounds__(NT, 4) crt_pm_planes_kernel(const PmPlanes a, 
     const uint32_t cs = cluster_size(), rank = cluster_rank();
     const long long r = blockIdx.x / cs;
     const int v = a.v, v4 = (v + 3) & ~3;
-    const long long ru = a.rtab[r];
+    const long long ru = a.rtab ? a.rtab[r] : r;
     const long long al = ru / a.Nb, bq = ru % a.Nb;
+    const bool flip = bq < al + a.diag;
     int* eo = esm;
     int* ei = esm + v4;
     int* co = esm + 2 * v4;
     int* ci = esm + 3 * v4;
     int m1 = INT_MIN, m2 = INT_MIN;
     for (int q = threadIdx.x; q < v4; q += NT) {
-        const int e1 = q < v ? a.eL[al * v + q] : 0, e2 = q < v ? a.eL[bq * v + q] : 0;
+        const int e1 = q < v ? a.eA[al * v + q] : 0, e2 = q < v ? a.eB[bq * v + q] : 0;
         eo[q] = e1;
         ei[q] = e2;
         if (q < v) { m1 = max(m1, e1); m2 = max(m2, e2); }
@@ -564,7 +566,7 @@ __global__ void __launch_bounds__(NT, 4) crt_pm_planes_kernel(const PmPlanes a, 
             const long long Y1 = S1[qy][qx + j], Y2 = S2[qx + j][qy];
             // Y is rounded down, by half a unit on average: the sum of two makes up for it with 1 more
             u[0][j] = (unsigned long long)((Y1 + Y2 + (long long)(4 * kCrtBias + 3)) >> 2);
-            u[1][j] = (unsigned long long)((Y1 - Y2 + (long long)(4 * kCrtBias + 2)) >> 2);
+            u[1][j] = (unsigned long long)(((flip ? Y2 - Y1 : Y1 - Y2) + (long long)(4 * kCrtBias + 2)) >> 2);
             const int d = d0 + j;
             if (t.tc == t.td && d <= c) {
                 u[0][j] = d == c ? (unsigned long long)((Y1 + (long long)(2 * kCrtBias + 1)) >> 1) : kCrtBias;
@@ -825,13 +827,13 @@ cudaError_t crt_pm_f64(const double* t2, const long long* rowtab, int o, int v, 
                        ep, rows_p, rows_m > 0 ? (unsigned short*)Dm : nullptr, em, rows_m, pitch, status);
 }
 
-cudaError_t crt_pm_planes(const CrtPlanes& src, const long long* rtab, long long rows, int Nb, int v, const int* eL,
-                          int nm, void* Dp, int* ep, void* Dm, int* em, long long pitch, cudaStream_t st)
+cudaError_t crt_pm_planes(const CrtPlanes& src, const long long* rtab, long long rows, int Nb, int v, const int* eA,
+                          const int* eB, int diag, int nm, void* Dp, int* ep, void* Dm, int* em, long long pitch, cudaStream_t st)
 {
     if (rows <= 0) return cudaSuccess;
     const size_t smem = sizeof(int) * 4 * (size_t)((v + 3) & ~3);  // v up to about 12800
     if (smem > 200 * 1024) return cudaErrorInvalidValue;
-    const PmPlanes a{src.planes, src.plane, src.pitch, rtab, Nb, v, eL};
+    const PmPlanes a{src.planes, src.plane, src.pitch, rtab, Nb, v, eA, eB, diag};
     const CrtRec rec = crt_rec(src.nm);
     const long long elems = (long long)v * v;
     const int cs = cluster_for(rows, elems, src.nm * elems);

@@ -316,38 +316,73 @@ __device__ __forceinline__ void pair_ij(int o, int p, int& i, int& j)
 }
 
 // R from R+ (rows: pairs q0 <= p < q1, i <= j) and R- (rows: their pairs i < j, from strict index
-// s0) of one block; columns are packed rows r (al, b' >= al).  Grid: x = pair p - q0, y = al.
-__global__ void pm_combine_kernel(int o, int v, int a0, int Nb, long long nr, long long q0, long long s0,
-                                  const double* __restrict__ Rp, const double* __restrict__ Rm,
+// s0) of one block; columns are packed rows r (al, b' >= al).  Grid: x = tile (al, b'), y + z gridDim.y = pair p - q0.
+// GEN: amplitudes without pair symmetry, every pair p = i o + j has its own R+ and R- row and writes R[p] only.
+// A 32 x 32 tile (al, b') is written as it is and, through shared memory, transposed, so that both halves of R are
+// written along the last index (entry by entry, the transposed half took host-resident R 4.3 ms of 19 at o=30, v=150,
+// 8 bytes per write over the host link).
+template <bool GEN>
+__global__ void pm_combine_kernel(int o, int v, int a0, int Ab, int Nb, long long nr, long long np, long long q0,
+                                  long long s0, const double* __restrict__ Rp, const double* __restrict__ Rm,
                                   double* __restrict__ R, int accumulate)
 {
-    const long long pl = blockIdx.x;
-    const int p = (int)(q0 + pl), al = blockIdx.y;
-    int i, j;
-    pair_ij(o, p, i, j);
-    const long long q = p - (i + 1) - s0;  // row among this block's pairs i < j
+    __shared__ double E1[TT][TT + 1], E2[TT][TT + 1];
+    const long long pl = (long long)blockIdx.y + (long long)blockIdx.z * gridDim.y;
+    if (pl >= np) return;  // uniform over the block
+    const int ntb = (Nb + TT - 1) / TT;
+    const int ta = (int)(blockIdx.x / ntb) * TT, tb = (int)(blockIdx.x % ntb) * TT;
+    if (tb + TT - 1 < ta) return;  // b' < al throughout
+    int i = 0, j = 1;
+    if (!GEN) pair_ij(o, (int)(q0 + pl), i, j);
     const long long vv = (long long)v * v;
-    const long long base = (long long)al * Nb - (long long)al * (al - 1) / 2;
-    const int a = a0 + al;
-    double* Rij = R + ((long long)i * o + j) * vv;
-    double* Rji = R + ((long long)j * o + i) * vv;
-    const double* rp = Rp + pl * nr + base - al;
-    const double* rm = (i < j && Rm) ? Rm + q * nr + base - al : nullptr;
-    for (int bq = al + threadIdx.x; bq < Nb; bq += blockDim.x) {
-        const int b = a0 + bq;
-        const double plus = rp[bq];
-        const double minus = (rm && b != a) ? rm[bq] : 0.0;
+    double* Rij = R + (GEN ? pl : (long long)i * o + j) * vv;
+    double* Rji = GEN ? Rij : R + ((long long)j * o + i) * vv;
+    const double* rp = Rp + pl * nr;
+    const double* rm = GEN ? (Rm ? Rm + pl * nr : nullptr)
+                           : ((i < j && Rm) ? Rm + (q0 + pl - (i + 1) - s0) * nr : nullptr);  // row among the pairs i < j
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    auto put = [&](double* p, double x) { *p = accumulate ? *p + x : x; };
+#pragma unroll
+    for (int y = ty; y < TT; y += TY) {
+        const int al = ta + y, bq = tb + tx;
+        if (al >= Ab || bq >= Nb || bq < al) continue;
+        const long long r = (long long)al * Nb - (long long)al * (al - 1) / 2 + (bq - al);
+        const double plus = rp[r];
+        const double minus = (rm && bq != al) ? rm[r] : 0.0;
         const double e1 = plus + minus, e2 = plus - minus;
-        const long long ab = (long long)a * v + b, ba = (long long)b * v + a;
-        if (accumulate) {
-            Rij[ab] += e1;
-            if (!(i == j && a == b)) Rji[ba] += e1;
-            if (i != j && a != b) { Rji[ab] += e2; Rij[ba] += e2; }
+        E1[y][tx] = e1;
+        E2[y][tx] = e2;
+        const long long ab = (long long)(a0 + al) * v + a0 + bq;
+        put(Rij + ab, e1);
+        if (!GEN && i != j && al != bq) put(Rji + ab, e2);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int y = ty; y < TT; y += TY) {
+        const int bq = tb + y, al = ta + tx;
+        if (al >= Ab || bq >= Nb || bq < al) continue;
+        const long long ba = (long long)(a0 + bq) * v + a0 + al;
+        if (GEN) {
+            if (al != bq) put(Rij + ba, E2[tx][y]);
         } else {
-            Rij[ab] = e1;
-            if (!(i == j && a == b)) Rji[ba] = e1;
-            if (i != j && a != b) { Rji[ab] = e2; Rij[ba] = e2; }
+            if (i != j || al != bq) put(Rji + ba, E1[tx][y]);
+            if (i != j && al != bq) put(Rij + ba, E2[tx][y]);
         }
+    }
+}
+
+// Rows (al, all b) of a range of `a`: see pm_combine_rows.
+__global__ void pm_combine_rows_kernel(long long np, int v, int a0, long long nr, const double* __restrict__ Rp,
+                                       const double* __restrict__ Rm, double* __restrict__ R, int accumulate)
+{
+    const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (r >= nr) return;
+    const int a = a0 + (int)(r / v), b = (int)(r % v);
+    for (long long p = blockIdx.y; p < np; p += gridDim.y) {
+        const double plus = Rp[p * nr + r], minus = Rm && a != b ? Rm[p * nr + r] : 0.0;
+        double* dst = R + p * ((long long)v * v) + (long long)a0 * v + r;
+        const double e = b < a ? plus - minus : plus + minus;
+        *dst = accumulate ? *dst + e : e;
     }
 }
 
@@ -405,14 +440,42 @@ cudaError_t fill_rtab(int Ab, int Nb, long long* rtab, cudaStream_t st)
     return cudaGetLastError();
 }
 
+namespace {
+// Tiles of a block by the pairs, within the grid limits for any number of pairs.
+dim3 combine_grid(int Ab, int Nb, long long np)
+{
+    const long long gz = (np + 65534) / 65535, gy = (np + gz - 1) / gz;
+    return dim3((unsigned)(((Ab + TT - 1) / TT) * ((Nb + TT - 1) / TT)), (unsigned)gy, (unsigned)gz);
+}
+}  // namespace
+
 cudaError_t pm_combine(int o, int v, int a0, int Ab, int Nb, long long nr, long long q0, long long q1, long long s0,
                        const double* Rp, const double* Rm, double* R, int accumulate, cudaStream_t st)
 {
     const long long np = q1 - q0;
     if (Ab <= 0 || np <= 0) return cudaSuccess;
     if (Ab > 65535 || np > 0x7fffffffll || q0 < 0 || q1 > (long long)o * (o + 1) / 2) return cudaErrorInvalidValue;
-    pm_combine_kernel<<<dim3((unsigned)np, (unsigned)Ab), 256, 0, st>>>(o, v, a0, Nb, nr, q0, s0, Rp, Rm, R,
-                                                                        accumulate);
+    pm_combine_kernel<false><<<combine_grid(Ab, Nb, np), TT * TY, 0, st>>>(o, v, a0, Ab, Nb, nr, np, q0, s0, Rp, Rm, R, accumulate);
+    count_launch();
+    return cudaGetLastError();
+}
+
+cudaError_t pm_combine_general(long long pairs, int v, int a0, int Ab, int Nb, long long nr, const double* Rp,
+                               const double* Rm, double* R, int accumulate, cudaStream_t st)
+{
+    if (Ab <= 0 || pairs <= 0) return cudaSuccess;
+    if (Ab > 65535 || pairs > 0x7fffffffll) return cudaErrorInvalidValue;
+    pm_combine_kernel<true><<<combine_grid(Ab, Nb, pairs), TT * TY, 0, st>>>(0, v, a0, Ab, Nb, nr, pairs, 0, 0, Rp, Rm, R, accumulate);
+    count_launch();
+    return cudaGetLastError();
+}
+
+cudaError_t pm_combine_rows(long long pairs, int v, int a0, long long nr, const double* Rp, const double* Rm, double* R,
+                            int accumulate, cudaStream_t st)
+{
+    if (nr <= 0 || pairs <= 0) return cudaSuccess;
+    pm_combine_rows_kernel<<<dim3((unsigned)((nr + 255) / 256), (unsigned)(pairs < 65535 ? pairs : 65535)), 256, 0, st>>>(
+        pairs, v, a0, nr, Rp, Rm, R, accumulate);
     count_launch();
     return cudaGetLastError();
 }
