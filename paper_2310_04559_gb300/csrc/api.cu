@@ -755,6 +755,32 @@ int run_crt_out(const char* name, const Ctx& c, int nm, int M, int N, int K, con
     return check_cuda(crt_to_f64(M, N, pl, g.ksplit, o, base, factor, swap, Ao.e, Bo.e, st));
 }
 
+// Mixed modes: C = A B^T with FP32 sums over kMixedChunk elements of K, as FP32 rows (f32, one chunk) or as FP64 through
+// `out`, there in the orientation whose tiles waste less.
+int run_mix(const char* name, const Ctx& c, int M, int N, int K, const Operand& A, long long rowA0, const Operand& B,
+            long long rowB0, float* f32, long long pitch, const OutDesc& out, cudaStream_t st, long long tri = 0)
+{
+    const bool swap = !f32 && tri == 0 && crt_tile_area(N, M) < crt_tile_area(M, N);
+    GemmMix g{};
+    g.kind = c.mode == CC_TF32 ? TC_TF32 : TC_BF16;
+    g.M = M; g.N = N; g.K = K; g.chunk = kMixedChunk;
+    g.A = A.D; g.pitchA = A.pitch; g.rowsA = A.rows; g.rowA0 = rowA0;
+    g.B = B.D; g.pitchB = B.pitch; g.rowsB = B.rows; g.rowB0 = rowB0;
+    g.f32 = f32; g.pitch = pitch;
+    g.out = out;
+    if (swap) {
+        std::swap(g.M, g.N);
+        std::swap(g.A, g.B); std::swap(g.pitchA, g.pitchB); std::swap(g.rowsA, g.rowsB); std::swap(g.rowA0, g.rowB0);
+        std::swap(g.out.rmap, g.out.cmap);
+    }
+    g.tri = tri;
+    g.status = c.status;
+    g.wait_ns = g_wait_ns.load();
+    const double el = tri_elems(g.M, g.N, tri, 256, 256);
+    ProfScope ps(name, st, 2.0 * el * K, (double)esz_of(c.mode) * ((double)M + N) * K + el * (f32 ? 4 : 8));
+    return check_cuda(gemm_mix(g, st));
+}
+
 // Rows of K = (o, i) from FP64 (ostride between outer indices).
 int prep_crt_rows(const Ctx& c, const RowSrc& src, int outer, int inner, long long ostride, int nm, Operand& op,
                   cudaStream_t st)
@@ -815,6 +841,9 @@ int fwd_packed(const Ctx& c, const cc_ladder_args* a, const double* Lsrc, const 
     Vm.D = at<void>(ws, Lo.Vm); Vm.e = at<int>(ws, Lo.eVm); Vm.pitch = Tm.pitch;
     unsigned char* Rw = c.crt ? at<unsigned char>(ws, Lo.Rw) : nullptr;
     unsigned long long* colmax = at<unsigned long long>(ws, Lo.colmax);
+    // mixed modes whose integrals are one FP32 sum over the Cholesky vectors keep the block in FP32
+    const bool mix32 = !f64 && !ozaki && !c.hostL && n <= kMixedChunk;
+    auto ldx32 = [&](int Nb) { return ((long long)Nb * v + 3) & ~3ll; };
     // Streamed L (CC_FLAG_HOST_L): chunks of PC Cholesky vectors are copied from page-locked host
     // memory into two device buffers on a second stream, so that chunk q + 1 arrives while chunk q
     // is split and contracted (the batches of Cholesky vectors of Section 5, overlapped); events
@@ -958,6 +987,10 @@ int fwd_packed(const Ctx& c, const cc_ladder_args* a, const double* Lsrc, const 
         } else if (c.crt) {
             CC_TRY(run_crt("kg1_tc", c, c.nm1, Ab * c.v, Nb * c.v, c.n, Lw, (long long)a0 * v, Lw, (long long)b0 * v,
                            (unsigned char*)V, &vpl, st, c.part ? 0 : v));
+        } else if (mix32) {
+            // the integral GEMM's FP32 sums as they are: X[(al, c)][(b', d)]
+            CC_TRY(run_mix("kg1_tc", c, Ab * c.v, Nb * c.v, c.n, Lw, (long long)a0 * v, Lw, (long long)a0 * v, (float*)V,
+                           ldx32(Nb), OutDesc{}, st, v));
         } else {
             CC_TRY(run_tc("kg1_tc", c, Ab * c.v, Nb * c.v, c.n, Lw, (long long)a0 * v, Lw, (long long)a0 * v, o1,
                           status, st, true, v));
@@ -975,6 +1008,9 @@ int fwd_packed(const Ctx& c, const cc_ladder_args* a, const double* Lsrc, const 
                 PmFixedSrc fs{(const long long*)V, rtab, nr, vv, c.v, Lw.e, split_map(Nb, v, 0, (long long)a0 * v),
                               Lw.e, split_map(Nb, 0, v, (long long)a0 * v), kFixedBase};
                 CC_CU(pm_split_fixed(fs, c.s, kBeta, Vp.D, Vp.pitch, Vp.e, minus ? Vm.D : nullptr, Vm.pitch, Vm.e, st));
+            } else if (mix32) {
+                CC_CU(pm_split_f32((const float*)V, ldx32(Nb), rtab, nr, Nb, c.v, kind, Vp.D, Vp.pitch, Vp.e,
+                                   minus ? Vm.D : nullptr, Vm.pitch, minus ? Vm.e : nullptr, st));
             } else {
                 CC_CU(pm_split_f64(V, rtab, vv, nr, c.v, +1, 0.5, kind, c.s, kBeta, Vp.D, Vp.pitch, Vp.e, nullptr, st));
                 if (minus)
@@ -1002,6 +1038,9 @@ int fwd_packed(const Ctx& c, const cc_ladder_args* a, const double* Lsrc, const 
             } else if (c.crt) {
                 CC_TRY(run_crt_out("kg2_tc", c, c.nm2, (int)(q1 - q0), (int)nr, kq, Tp, Vp, op, Rw, Lo.Rw_bytes, st, c.nm1));
                 if (mb) CC_TRY(run_crt_out("kg2_tc", c, c.nm2, (int)(s1 - s0), (int)nr, kq, Tm, Vm, om, Rw, Lo.Rw_bytes, st, c.nm1));
+            } else if (!ozaki) {
+                CC_TRY(run_mix("kg2_tc", c, (int)(q1 - q0), (int)nr, (int)c.Kp, Tp, 0, Vp, 0, nullptr, 0, op, st));
+                if (mb) CC_TRY(run_mix("kg2_tc", c, (int)(s1 - s0), (int)nr, (int)c.Km, Tm, 0, Vm, 0, nullptr, 0, om, st));
             } else {
                 CC_TRY(run_tc("kg2_tc", c, (int)(q1 - q0), (int)nr, (int)c.Kp, Tp, 0, Vp, 0, op, status, st));
                 if (mb) CC_TRY(run_tc("kg2_tc", c, (int)(s1 - s0), (int)nr, (int)c.Km, Tm, 0, Vm, 0, om, status, st));

@@ -197,6 +197,24 @@ struct GemmCrt {
     unsigned long long wait_ns;
 };
 cudaError_t gemm_crt(const GemmCrt& g, cudaStream_t s);
+// Mixed modes on the same tiles: one bf16 / tf32 stack each, FP32 sums over `chunk` elements of K.  f32 not NULL (K <=
+// chunk): [M][pitch] FP32 sums (pitch a multiple of 4); else out = (or +=) the FP64 sum of the chunks.
+struct GemmMix {
+    int kind;  // TcKind
+    int M, N, K, chunk;
+    const void* A; long long pitchA, rowsA, rowA0;
+    const void* B; long long pitchB, rowsB, rowB0;
+    float* f32; long long pitch;
+    OutDesc out;
+    long long tri;
+    int* status;
+    unsigned long long wait_ns;
+};
+cudaError_t gemm_mix(const GemmMix& g, cudaStream_t s);
+// V+ and (Dm not NULL) V- of the rows rtab[r] = al * Nb + b' from FP32 X[(al, c)][(b', d)] (pitch floats per row), in the
+// packed orders of pm_split_f64: (x1 +- x2) / 2, rounded once to bf16 (kind 1) or through FP32 to tf32 (kind 2).
+cudaError_t pm_split_f32(const float* X, long long ldx, const long long* rtab, long long rows, int Nb, int v, int kind,
+                         void* Dp, long long pitchp, int* ep, void* Dm, long long pitchm, int* em, cudaStream_t st);
 struct CrtPlanes {
     const unsigned char* planes;
     long long plane, pitch;  // bytes between planes, bytes per GEMM row

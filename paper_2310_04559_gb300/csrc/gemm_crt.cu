@@ -20,6 +20,10 @@
 // (r = x - p rint(x / p), exact), 1.5 instructions per element and pass: converting to integers instead took 8000
 // clocks per tile, as long as the MMAs of K = 1000 (8192 x 8192 x 1024, 12 moduli: 1518 TFLOP/s then, see below).
 //
+// The same kernel runs the mixed modes' GEMMs (one bf16 or tf32 operand each, passes of 16384 elements in FP32, FP64
+// across passes), storing the FP32 sums or FP64: on 128 x 128 tiles of single SMs they had no operand reuse and were
+// bound by the copies (integral build of o=27/v=301/n=1501 in BF16: 37.2 ms, see below).
+//
 // Bound: tensor pipe (power-capped).  o=40/v=400/n=2000 integral blocks: see the table in the design notes.
 //
 // Roles (384 threads): warp 0 issues the A copies and fetches items (leader CTA), warp 3 the B copies,
@@ -45,7 +49,6 @@ namespace {
 constexpr int BM = 128;                        // tile rows per CTA (256 per pair)
 constexpr int TM = 2 * BM;                     // tile rows per pair
 constexpr int TN = 256;                        // widest tile
-constexpr int KSTEP = 64;                      // bf16 elements per 128-byte swizzle atom
 constexpr int TILE_BYTES = 128 * 128;          // 128 rows x 128 bytes
 constexpr int NS = 6;                          // ring slots (one K-step of A and B each)
 constexpr int RING_BYTES = NS * 2 * TILE_BYTES;  // 192 KB
@@ -63,7 +66,7 @@ constexpr unsigned long long kSettleNs = 5000000ull;      // abort path: copies 
 constexpr unsigned long long kDrainLimitNs = 1000000000ull;  // abort path: bound on the MMA drain
 constexpr int WARP_A = 0, WARP_MMA = 2, WARP_B = 3;
 
-__device__ int g_crt_counter[kCounterSlots];
+__device__ int g_crt_counter[6 * kCounterSlots];  // a ring for each kernel
 
 struct SmemCtl {
     unsigned long long full[NS], empty[NS];
@@ -77,8 +80,12 @@ struct SmemCtl {
 constexpr size_t SMEM_BYTES = 1024 + RING_BYTES + sizeof(SmemCtl);
 static_assert(SMEM_BYTES <= 227 * 1024, "shared memory");
 
+// What a kernel stores: residue bytes, the FP32 sums themselves (one pass), or FP64 through an index map.
+enum OutKind { OUT_RES = 0, OUT_F32 = 1, OUT_F64 = 2 };
+
 struct Params {
     int M, N, K, nm;
+    int chunk;                       // K elements per pass
     long long rowA0, rowB0;
     int ksplit, kper;                // K split s owns [s*kper, min(K, (s+1)*kper))
     long long tri;                   // triangular tile skip (0 = off): b(n) = n / tri < a(m) = m / tri
@@ -89,6 +96,8 @@ struct Params {
     long long pitch;
     int accumulate;                  // add to the residues that are there (modulo p_l)
     float inv[kCrtMax], neg[kCrtMax];  // 1 / p_l, -p_l
+    float* f32;                      // OUT_F32: [M][pitch]
+    OutDesc out;                     // OUT_F64
     int* counter;                    // items handed out beyond the first of each pair (zero at launch)
     int* status;
     unsigned long long wait_ns;
@@ -214,18 +223,27 @@ __device__ __forceinline__ unsigned long long smem_desc(const void* p)
     return ((addr >> 4) & 0x3fffull) | (1ull << 16) | ((unsigned long long)(1024 >> 4) << 32) | (1ull << 46) | (2ull << 61);
 }
 
-// FP32 accumulate, bf16 x bf16, both K-major, M = 256, N = width.
+// FP32 accumulate, A and B bf16 (1) or tf32 (2), both K-major, M = 256, N = width.
+template <int KIND>
 __device__ __forceinline__ uint32_t instr_desc(int width)
 {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(width >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
+    const uint32_t fmt = KIND == TC_BF16 ? 1u : 2u;
+    return (1u << 4) | (fmt << 7) | (fmt << 10) | ((uint32_t)(width >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
 }
 
+template <int KIND>
 __device__ __forceinline__ void mma(uint32_t d, unsigned long long a, unsigned long long b, uint32_t idesc, uint32_t acc)
 {
-    asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-        " tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n"
-        ::"r"(d), "l"(a), "l"(b), "r"(idesc), "r"(acc));
+    if (KIND == TC_BF16)
+        asm volatile(
+            "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+            " tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n"
+            ::"r"(d), "l"(a), "l"(b), "r"(idesc), "r"(acc));
+    else
+        asm volatile(
+            "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+            " tcgen05.mma.cta_group::2.kind::tf32 [%0], %1, %2, %3, p;\n}\n"
+            ::"r"(d), "l"(a), "l"(b), "r"(idesc), "r"(acc));
 }
 
 // Arrive on `bar` (same offset) in both CTAs once this thread's prior MMAs complete.
@@ -250,6 +268,16 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32])
           "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
           "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
           "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        : "r"(taddr));
+}
+
+// 32 lanes x 8 columns, waited for.
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8])
+{
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
         : "r"(taddr));
 }
 
@@ -305,6 +333,7 @@ __device__ __forceinline__ int publish_item(SmemCtl* ctl, const Params& p, uint3
     return item;
 }
 
+template <int KIND, int OUT>
 __global__ void __launch_bounds__(THREADS, 1)
 gemm_crt_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const Params p)
 {
@@ -313,6 +342,7 @@ gemm_crt_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     unsigned char* aring = base;
     unsigned char* bring = base + NS * TILE_BYTES;
     SmemCtl* ctl = (SmemCtl*)(base + RING_BYTES);
+    constexpr int KSTEP = KIND == TC_BF16 ? 64 : 32;  // K elements per 128-byte swizzle atom
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_rank();
@@ -401,14 +431,14 @@ gemm_crt_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                 const int item = item_at(ctl, k, rank, p);
                 if (item < 0) break;
                 const Item w = item_of(p, item);
-                const uint32_t idesc = instr_desc(w.width);
+                const uint32_t idesc = instr_desc<KIND>(w.width);
                 const int kbeg = w.split * p.kper, kend = min(p.K, kbeg + p.kper);
-                for (int k0 = kbeg; k0 < kend && ok; k0 += kCrtChunk) {
+                for (int k0 = kbeg; k0 < kend && ok; k0 += p.chunk) {
                     const int buf = (int)(npass & 1);
                     if (!mbar_wait(&ctl->tempty[buf], ((npass >> 1) & 1) ^ 1, ctl, rank, p)) { ok = false; break; }
                     fence_after();
                     const uint32_t d = tmem + (uint32_t)(buf * TN);
-                    const int k1 = min(kend, k0 + kCrtChunk);
+                    const int k1 = min(kend, k0 + p.chunk);
                     uint32_t acc = 0;
                     for (int kb = k0; kb < k1; kb += KSTEP, ++u) {
                         const uint32_t s = u % NS;
@@ -418,10 +448,10 @@ gemm_crt_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                         const unsigned long long bd = bdesc0 + (unsigned long long)(s * (TILE_BYTES >> 4));
                         any = true;
                         // four MMAs per 128-byte row: advance the start address by 32 bytes each
-                        mma(d, ad, bd, idesc, acc);
-                        mma(d, ad + 2, bd + 2, idesc, 1u);
-                        mma(d, ad + 4, bd + 4, idesc, 1u);
-                        mma(d, ad + 6, bd + 6, idesc, 1u);
+                        mma<KIND>(d, ad, bd, idesc, acc);
+                        mma<KIND>(d, ad + 2, bd + 2, idesc, 1u);
+                        mma<KIND>(d, ad + 4, bd + 4, idesc, 1u);
+                        mma<KIND>(d, ad + 6, bd + 6, idesc, 1u);
                         acc = 1;
                         commit_both(&ctl->empty[s]);
                     }
@@ -460,38 +490,68 @@ gemm_crt_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             item = __shfl_sync(0xffffffffu, item, 0);
             if (item < 0) break;
             const Item w = item_of(p, item);
+            const int m = w.m0 + row;
             const unsigned long long inv = f2(p.inv[w.l], p.inv[w.l]), neg = f2(p.neg[w.l], p.neg[w.l]);
             const int kbeg = w.split * p.kper, kend = min(p.K, kbeg + p.kper);
             int pass = 0;
-            for (int k0 = kbeg; k0 < kend; k0 += kCrtChunk, ++pass, ++npass) {
+            for (int k0 = kbeg; k0 < kend; k0 += p.chunk, ++pass, ++npass) {
                 const int buf = (int)(npass & 1);
                 if (lane == 0) ok = mbar_wait(&ctl->tfull[buf], (npass >> 1) & 1, ctl, rank, p);
                 ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
                 if (!ok) break;
                 fence_after();
+                if (OUT == OUT_F64) {
+                    // FP64 across the passes, in the output: first pass = (or +=), later ones +=
+                    double* Crow = p.out.C + (m < p.M ? map2(p.out.rmap, m) : 0);
+                    const bool add = pass > 0 || p.out.accumulate;
+#pragma unroll 1
+                    for (int c = 0; c < CPT && col0 + c < w.width; c += 8) {  // (uniform over the warp)
+                        uint32_t r[8];
+                        __syncwarp();
+                        tmem_ld8(tl + (uint32_t)(buf * TN + c), r);
 #pragma unroll
-                for (int c = 0; c < CPT; c += 32) {
-                    if (col0 + c < w.width) {  // (uniform over the warp)
+                        for (int q = 0; q < 8; ++q) {
+                            const int n = w.n0 + col0 + c + q;
+                            if (m >= p.M || n >= p.N) continue;
+                            double* dst = Crow + map2(p.out.cmap, n);
+                            const double x = (double)__uint_as_float(r[q]);
+                            *dst = add ? *dst + x : x;
+                        }
+                    }
+                } else {
+#pragma unroll
+                    for (int c = 0; c < CPT; c += 32) {
+                        if (col0 + c >= w.width) continue;  // (uniform over the warp; widths are multiples of 32)
                         uint32_t r[32];
+                        __syncwarp();
                         tmem_ld32(tl + (uint32_t)(buf * TN + c), r);
+                        if (OUT == OUT_F32) {
+                            float* dst = p.f32 + (long long)m * p.pitch + w.n0 + col0 + c;
+                            if (m >= p.M) continue;
 #pragma unroll
-                        for (int q = 0; q < 16; ++q) {
-                            const unsigned long long x =
-                                reduce2(f2(__uint_as_float(r[2 * q]), __uint_as_float(r[2 * q + 1])), inv, neg);
-                            sum[c / 2 + q] = pass == 0 ? x : add2(sum[c / 2 + q], x);
+                            for (int q = 0; q < 32; q += 4)
+                                if (w.n0 + col0 + c + q < p.pitch)
+                                    *reinterpret_cast<uint4*>(dst + q) = make_uint4(r[q], r[q + 1], r[q + 2], r[q + 3]);
+                        } else {
+#pragma unroll
+                            for (int q = 0; q < 16; ++q) {
+                                const unsigned long long x =
+                                    reduce2(f2(__uint_as_float(r[2 * q]), __uint_as_float(r[2 * q + 1])), inv, neg);
+                                sum[c / 2 + q] = pass == 0 ? x : add2(sum[c / 2 + q], x);
+                            }
                         }
                     }
                 }
                 fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive_cluster(in_cta(&ctl->tempty[buf], 0));
-                if (pass % kReduceEvery == kReduceEvery - 1) {
+                if (OUT == OUT_RES && pass % kReduceEvery == kReduceEvery - 1) {
 #pragma unroll
                     for (int q = 0; q < CPT / 2; ++q) sum[q] = reduce2(sum[q], inv, neg);
                 }
             }
             if (!ok) break;
-            const int m = w.m0 + row;
+            if (OUT != OUT_RES) continue;
             unsigned char* dst = p.planes + ((long long)(w.split * p.nm + w.l) * p.M + m) * p.pitch + w.n0 + col0;
             if (m < p.M) {
 #pragma unroll
@@ -545,49 +605,37 @@ PFN_cuTensorMapEncodeTiled_v12000 get_encode()
     return fn;
 }
 
-// 3-D map over a residue stack [nm][rows][pitch], extent K in the inner dimension; boxes of 64 x box_rows.
-bool make_map(CUtensorMap* m, const void* base, long long K, long long pitch, long long rows, int nm, int box_rows)
+// 3-D map over a stack [nm][rows][pitch] of bf16 or tf32, extent K in the inner dimension; boxes of 128 bytes x box_rows.
+bool make_map(CUtensorMap* m, const void* base, int kind, long long K, long long pitch, long long rows, int nm, int box_rows)
 {
     auto enc = get_encode();
     if (!enc) return false;
+    const int es = kind == TC_BF16 ? 2 : 4;
     cuuint64_t dims[3] = {(cuuint64_t)K, (cuuint64_t)rows, (cuuint64_t)nm};
-    cuuint64_t strides[2] = {(cuuint64_t)(pitch * 2), (cuuint64_t)(pitch * 2 * rows)};
-    cuuint32_t box[3] = {(cuuint32_t)KSTEP, (cuuint32_t)box_rows, 1};
+    cuuint64_t strides[2] = {(cuuint64_t)(pitch * es), (cuuint64_t)(pitch * es * rows)};
+    cuuint32_t box[3] = {(cuuint32_t)(128 / es), (cuuint32_t)box_rows, 1};
     cuuint32_t estr[3] = {1, 1, 1};
-    return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    return enc(m, kind == TC_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3,
+               const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-}  // namespace
+struct Sides {  // operands of a launch
+    const void* A; long long pitchA, rowsA;
+    const void* B; long long pitchB, rowsB;
+};
 
-cudaError_t gemm_crt(const GemmCrt& g, cudaStream_t s)
+// Tiles, items, counter and launch; p holds everything else.
+template <int KIND, int OUT>
+cudaError_t launch(const Sides& g, Params& p, cudaStream_t s)
 {
-    if (g.M <= 0 || g.N <= 0) return cudaSuccess;
-    if (g.K <= 0 || g.nm < 1 || g.nm > kCrtMax || g.pitch < g.N || g.pitch % 16 || g.tri < 0) return cudaErrorInvalidValue;
-    Params p{};
-    p.M = g.M; p.N = g.N; p.K = g.K; p.nm = g.nm;
-    p.rowA0 = g.rowA0; p.rowB0 = g.rowB0;
-    p.ksplit = g.ksplit > 1 ? g.ksplit : 1;
-    p.kper = (int)((((long long)g.K + p.ksplit - 1) / p.ksplit + KSTEP - 1) / KSTEP * KSTEP);
-    if ((long long)p.kper * (p.ksplit - 1) >= g.K || (p.ksplit > 1 && g.accumulate)) return cudaErrorInvalidValue;
-    p.tri = g.tri;
-    p.planes = g.planes;
-    p.pitch = g.pitch;
-    p.accumulate = g.accumulate;
-    for (int l = 0; l < g.nm; ++l) {
-        p.inv[l] = 1.0f / (float)crt_p(l);
-        p.neg[l] = -(float)crt_p(l);
-    }
-    p.status = g.status;
-    p.wait_ns = g.wait_ns;
-    p.tiles_m = (g.M + TM - 1) / TM;
-    p.tiles_n = (g.N + TN - 1) / TN;
-    const int units = (g.N + 31) / 32;
+    p.tiles_m = (p.M + TM - 1) / TM;
+    p.tiles_n = (p.N + TN - 1) / TN;
+    const int units = (p.N + 31) / 32;
     p.ubase = units / p.tiles_n;
     p.urem = units % p.tiles_n;
     p.group_m = p.tiles_m < 8 ? p.tiles_m : 8;
-    const long long nitems = (long long)p.tiles_m * p.tiles_n * p.ksplit * g.nm;
+    const long long nitems = (long long)p.tiles_m * p.tiles_n * p.ksplit * p.nm;
     if (nitems > 0x7fffffffll - (1 << 20)) return cudaErrorInvalidConfiguration;
     p.nitems = (int)nitems;
 
@@ -606,11 +654,11 @@ cudaError_t gemm_crt(const GemmCrt& g, cudaStream_t s)
     static cudaError_t attr_err = cudaSuccess;
     static int max_pairs = 0;
     std::call_once(once, [&cfg] {
-        attr_err = cudaFuncSetAttribute(gemm_crt_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
+        attr_err = cudaFuncSetAttribute(gemm_crt_kernel<KIND, OUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
         // persistent: as many pairs as are resident on the device at once
         int n = 0;
         cfg.gridDim = dim3(2 * 64);
-        if (attr_err != cudaSuccess || cudaOccupancyMaxActiveClusters(&n, gemm_crt_kernel, &cfg) != cudaSuccess || n <= 0) {
+        if (attr_err != cudaSuccess || cudaOccupancyMaxActiveClusters(&n, gemm_crt_kernel<KIND, OUT>, &cfg) != cudaSuccess || n <= 0) {
             cudaGetLastError();
             n = device_sm_count() / 2;
         }
@@ -624,21 +672,71 @@ cudaError_t gemm_crt(const GemmCrt& g, cudaStream_t s)
     int* counters = nullptr;
     cudaError_t err = cudaGetSymbolAddress((void**)&counters, g_crt_counter);
     if (err != cudaSuccess) return err;
-    p.counter = counters + (next_slot.fetch_add(1) % kCounterSlots);
+    p.counter = counters + (OUT * 2 + KIND) * kCounterSlots + (next_slot.fetch_add(1) % kCounterSlots);
     err = cudaMemsetAsync(p.counter, 0, sizeof(int), s);
     if (err != cudaSuccess) return err;
     CUtensorMap ma, mb;
     // (narrow tiles, N <= 224, are bound by the copies: B's boxes hold only the rows a tile uses)
     const int brows = 16 * (p.ubase + (p.urem > 0 ? 1 : 0));
     p.step_bytes = 2u * (uint32_t)(TILE_BYTES + brows * 128);
-    if (!make_map(&ma, g.A, g.K, g.pitchA, g.rowsA, g.nm, BM) || !make_map(&mb, g.B, g.K, g.pitchB, g.rowsB, g.nm, brows))
+    if (!make_map(&ma, g.A, KIND, p.K, g.pitchA, g.rowsA, p.nm, BM) ||
+        !make_map(&mb, g.B, KIND, p.K, g.pitchB, g.rowsB, p.nm, brows))
         return cudaErrorInvalidValue;
     const int pairs = p.nitems < max_pairs ? p.nitems : max_pairs;
     cfg.gridDim = dim3((unsigned)(2 * pairs));
-    err = cudaLaunchKernelEx(&cfg, gemm_crt_kernel, ma, mb, p);
+    err = cudaLaunchKernelEx(&cfg, gemm_crt_kernel<KIND, OUT>, ma, mb, p);
     if (err != cudaSuccess) return err;
     count_launch();
     return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t gemm_crt(const GemmCrt& g, cudaStream_t s)
+{
+    if (g.M <= 0 || g.N <= 0) return cudaSuccess;
+    if (g.K <= 0 || g.nm < 1 || g.nm > kCrtMax || g.pitch < g.N || g.pitch % 16 || g.tri < 0) return cudaErrorInvalidValue;
+    Params p{};
+    p.M = g.M; p.N = g.N; p.K = g.K; p.nm = g.nm;
+    p.chunk = kCrtChunk;
+    p.rowA0 = g.rowA0; p.rowB0 = g.rowB0;
+    p.ksplit = g.ksplit > 1 ? g.ksplit : 1;
+    p.kper = (int)((((long long)g.K + p.ksplit - 1) / p.ksplit + 63) / 64 * 64);
+    if ((long long)p.kper * (p.ksplit - 1) >= g.K || (p.ksplit > 1 && g.accumulate)) return cudaErrorInvalidValue;
+    p.tri = g.tri;
+    p.planes = g.planes;
+    p.pitch = g.pitch;
+    p.accumulate = g.accumulate;
+    for (int l = 0; l < g.nm; ++l) {
+        p.inv[l] = 1.0f / (float)crt_p(l);
+        p.neg[l] = -(float)crt_p(l);
+    }
+    p.status = g.status;
+    p.wait_ns = g.wait_ns;
+    return launch<TC_BF16, OUT_RES>(Sides{g.A, g.pitchA, g.rowsA, g.B, g.pitchB, g.rowsB}, p, s);
+}
+
+cudaError_t gemm_mix(const GemmMix& g, cudaStream_t s)
+{
+    if (g.M <= 0 || g.N <= 0) return cudaSuccess;
+    const int kstep = g.kind == TC_BF16 ? 64 : 32;
+    if (g.K <= 0 || g.chunk <= 0 || g.chunk % kstep || g.tri < 0) return cudaErrorInvalidValue;
+    if (g.f32 && (g.K > g.chunk || g.pitch < g.N || g.pitch % 4)) return cudaErrorInvalidValue;
+    Params p{};
+    p.M = g.M; p.N = g.N; p.K = g.K; p.nm = 1;
+    p.chunk = g.chunk;
+    p.rowA0 = g.rowA0; p.rowB0 = g.rowB0;
+    p.ksplit = 1;
+    p.kper = (g.K + 63) / 64 * 64;
+    p.tri = g.tri;
+    p.f32 = g.f32;
+    p.pitch = g.pitch;
+    p.out = g.out;
+    p.status = g.status;
+    p.wait_ns = g.wait_ns;
+    const Sides sd{g.A, g.pitchA, g.rowsA, g.B, g.pitchB, g.rowsB};
+    if (g.kind == TC_BF16) return g.f32 ? launch<TC_BF16, OUT_F32>(sd, p, s) : launch<TC_BF16, OUT_F64>(sd, p, s);
+    return g.f32 ? launch<TC_TF32, OUT_F32>(sd, p, s) : launch<TC_TF32, OUT_F64>(sd, p, s);
 }
 
 }  // namespace cc

@@ -111,13 +111,13 @@ __device__ __forceinline__ int exp_of_maxbits(unsigned long long b)
     return ex == 0 ? -1022 : ex - 1022;
 }
 
-__device__ __forceinline__ float tf32_of(double x)
+__device__ __forceinline__ float tf32_round(float f)
 {
-    const float f = (float)x;
     unsigned int u;
     asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(u) : "f"(f));
     return __uint_as_float(u);
 }
+__device__ __forceinline__ float tf32_of(double x) { return tf32_round((float)x); }
 
 __device__ __forceinline__ unsigned long long block_max_u64(unsigned long long m, unsigned long long* red)
 {
@@ -299,6 +299,78 @@ __global__ void pm_fixed_kernel(const PmFixedSrc src, int s, int beta, __nv_bflo
     }
 }
 
+// (x1 + x2) / 2 rounded once to bf16, as from the exact sum: the FP32 sum is made odd where it is not exact
+// (its last bit then stands for all that follows), which the 16 bits to be dropped keep for the second rounding.
+__device__ __forceinline__ unsigned short half_sum_bf16(float x1, float x2)
+{
+    const float s = __fadd_rn(x1, x2);
+    const float t = __fsub_rn(s, x1);
+    const float err = __fadd_rn(__fsub_rn(x1, __fsub_rn(s, t)), __fsub_rn(x2, t));  // x1 + x2 = s + err
+    uint32_t b = __float_as_uint(s);
+    if (err != 0.0f && !(b & 1u)) b += ((__float_as_uint(err) ^ b) >> 31) ? 0xffffffffu : 1u;
+    const __nv_bfloat16 h = __float2bfloat16_rn(0.5f * __uint_as_float(b));
+    return *reinterpret_cast<const unsigned short*>(&h);
+}
+
+// Integral block of the mixed modes in FP32 (the integral GEMM's own sums): V+ and V- of one row in one walk over its
+// tile pairs, 4 bytes read and 2 (4) written per element.  Bound: HBM.  From an FP64 block, one kernel per sign, the
+// same split took 38 ms of the 80 at o=27/v=301/n=1501 in BF16, most of it FP64 arithmetic.
+template <bool BF16>
+__global__ void __launch_bounds__(TT * TY) pm_f32_kernel(const float* __restrict__ X0, long long ldx,
+                                                         const long long* __restrict__ rtab, int Nb, int v,
+                                                         void* __restrict__ Dp, long long pitchp, int* __restrict__ ep,
+                                                         void* __restrict__ Dm, long long pitchm, int* __restrict__ em)
+{
+    __shared__ float S[2][2][TT][TT + 1];  // two buffers: one barrier per tile pair
+    const long long r = blockIdx.x;
+    const long long ru = rtab[r];
+    const float* X = X0 + (ru / Nb) * v * ldx + (ru % Nb) * v;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int nt = (v + TT - 1) / TT;
+    int buf = 0;
+    for (int tc = 0; tc < nt; ++tc) {
+        for (int td = tc; td < nt; ++td, buf ^= 1) {
+            float (&S1)[TT][TT + 1] = S[buf][0];
+            float (&S2)[TT][TT + 1] = S[buf][1];
+            float q1[TT / TY], q2[TT / TY];
+#pragma unroll
+            for (int u = 0; u < TT / TY; ++u) {
+                const int y = ty + u * TY;
+                const int c = tc * TT + y, d = td * TT + tx, d2 = td * TT + y, c2 = tc * TT + tx;
+                q1[u] = (c < v && d < v) ? __ldcs(X + c * ldx + d) : 0.0f;
+                q2[u] = (d2 < v && c2 < v) ? __ldcs(X + d2 * ldx + c2) : 0.0f;
+            }
+#pragma unroll
+            for (int u = 0; u < TT / TY; ++u) {
+                S1[ty + u * TY][tx] = q1[u];
+                S2[ty + u * TY][tx] = q2[u];
+            }
+            __syncthreads();
+#pragma unroll
+            for (int u = 0; u < TT / TY; ++u) {
+                const int y = ty + u * TY;
+                const int c = tc * TT + y, d = td * TT + tx;
+                if (c >= v || d >= v || d < c) continue;
+                const float x1 = S1[y][tx], x2 = S2[tx][y];
+                const long long kp = r * pitchp + kp_of(c, d, v);
+                if (BF16) {
+                    const __nv_bfloat16 h = __float2bfloat16_rn(x1);
+                    ((unsigned short*)Dp)[kp] = c == d ? *reinterpret_cast<const unsigned short*>(&h) : half_sum_bf16(x1, x2);
+                    if (Dm && c != d) ((unsigned short*)Dm)[r * pitchm + km_of(c, d, v)] = half_sum_bf16(x1, -x2);
+                } else {
+                    // (FP64 sums of two FP32 values round to the same FP32 as the FP32 sum)
+                    ((float*)Dp)[kp] = tf32_round(c == d ? x1 : 0.5f * __fadd_rn(x1, x2));
+                    if (Dm && c != d) ((float*)Dm)[r * pitchm + km_of(c, d, v)] = tf32_round(0.5f * __fsub_rn(x1, x2));
+                }
+            }
+        }
+    }
+    if (threadIdx.x == 0) {
+        if (ep) ep[r] = 0;
+        if (em) em[r] = 0;
+    }
+}
+
 // rtab[rowbase(al) + b' - al] = al * Nb + b' for b' in [al, Nb)
 __global__ void fill_rtab_kernel(int Ab, int Nb, long long* __restrict__ rtab)
 {
@@ -428,6 +500,17 @@ cudaError_t pm_split_fixed(const PmFixedSrc& src, int s, int beta, void* Dp, lon
     }
     pm_fixed_kernel<<<(unsigned)src.rows, 256, smem, st>>>(src, s, beta, (__nv_bfloat16*)Dp, pitchp, ep,
                                                            (__nv_bfloat16*)Dm, pitchm, em);
+    count_launch();
+    return cudaGetLastError();
+}
+
+cudaError_t pm_split_f32(const float* X, long long ldx, const long long* rtab, long long rows, int Nb, int v, int kind,
+                         void* Dp, long long pitchp, int* ep, void* Dm, long long pitchm, int* em, cudaStream_t st)
+{
+    if (rows <= 0) return cudaSuccess;
+    if (v < 1 || (kind != 1 && kind != 2) || rows > 0x7fffffffll) return cudaErrorInvalidValue;
+    if (kind == 1) pm_f32_kernel<true><<<(unsigned)rows, TT * TY, 0, st>>>(X, ldx, rtab, Nb, v, Dp, pitchp, ep, Dm, pitchm, em);
+    else pm_f32_kernel<false><<<(unsigned)rows, TT * TY, 0, st>>>(X, ldx, rtab, Nb, v, Dp, pitchp, ep, Dm, pitchm, em);
     count_launch();
     return cudaGetLastError();
 }
