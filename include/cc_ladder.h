@@ -65,7 +65,7 @@ enum cc_status {
 
 /* Arithmetic used for the two contractions (integral build and ladder GEMM). */
 enum cc_precision {
-    CC_FP64 = 0,       /* FP64 tensor-core MMA (DMMA), FP64 accumulation              */
+    CC_FP64 = 0,       /* FP64 fused multiply-adds, FP64 accumulation                 */
     CC_OZAKI_BF16 = 1, /* FP64 emulated by integers on tcgen05 BF16 tensor cores (Ozaki scheme): each
                           operand row is scaled by a power of two and rounded once to 42-bit integers.
                           Default precision (slices = 0 or 6): the integers' residues modulo 12 or 13
@@ -287,7 +287,7 @@ void cc_ladder_set_wait_limit_ns(unsigned long long ns);
 
 /* Building block used by every contraction above, exposed for direct use and testing:
  *   C[m*ldc + n] (= or +=) sum_k A[m*lda + k] * B[n*ldb + k]     (row-major, K-contiguous FP64)
- * in the arithmetic of `mode` (CC_FP64: DMMA; CC_OZAKI_BF16: split BF16 slices on tcgen05 with
+ * in the arithmetic of `mode` (CC_FP64: FP64 FMAs; CC_OZAKI_BF16: split BF16 slices on tcgen05 with
  * FP64 recombination; CC_TF32 / CC_BF16: one rounded copy, FP32 accumulation per K-chunk).
  * accumulate != 0 adds into C.  Workspace from cc_ladder_gemm_workspace_size.
  * CC_OZAKI_BF16 is exact in its FP32 sums for any K and any input (see cc_precision). */
@@ -319,8 +319,8 @@ long long cc_ladder_launch_count(void);
  * mode's throughput can be set against the rate of the unit it runs on, measured on the same GPU).
  * Launches one microbenchmark kernel twice (warm-up, then timed with CUDA events on `stream`,
  * synchronised) and writes the whole GPU's rate in TFLOP/s to *tflops (host pointer).
- *   CC_PROBE_DMMA     mma.sync.m8n8k4.f64 from registers (the FP64 mode's GEMM instruction)
- *   CC_PROBE_DFMA     scalar FP64 fma from registers
+ *   CC_PROBE_DMMA     mma.sync.m8n8k4.f64 from registers (the FP64 tensor-core form)
+ *   CC_PROBE_DFMA     scalar FP64 fma from registers (the FP64 mode's GEMM instruction)
  *   CC_PROBE_TC_BF16  tcgen05.mma kind::f16, BF16 operands in shared memory, M=128 N=256 K=16,
  *                     one issuing thread per SM (the emulated-FP64 and BF16 modes)
  *   CC_PROBE_TC_TF32  tcgen05.mma kind::tf32, M=128 N=256 K=8 (the TF32 mode)

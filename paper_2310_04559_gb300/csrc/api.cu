@@ -22,7 +22,7 @@
 // which issues about (n + o^2/2) v^4 multiply-adds instead of 2 (n + o(o+1)/2) v^4.
 // In the emulated-FP64 and mixed modes every GEMM operand is first turned into
 // a slice stack (split.cu, pm.cu) and the GEMM runs on the tensor cores (gemm_tc.cu);
-// in the FP64 mode the GEMMs run on DMMA (gemm_f64.cu) straight from FP64.
+// in the FP64 mode the GEMMs run on FP64 FMAs (gemm_f64.cu) straight from FP64.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -149,7 +149,7 @@ FwdLayout layout_packed(const Ctx& c, long long P)
     FwdLayout L{};
     Carve cv;
     const long long o = c.o, v = c.v, n = c.n, vv = v * v;
-    const bool f64 = c.mode == CC_FP64;  // packed operands stay FP64 (DMMA), no slices
+    const bool f64 = c.mode == CC_FP64;  // packed operands stay FP64, no slices
     const int es = f64 ? 8 : esz_of(c.mode);
     const long long s = f64 ? 1 : c.s;
     L.status = cv.take(256);
@@ -560,7 +560,7 @@ double tc_products(const Ctx& c) { return c.mode == CC_OZAKI_BF16 ? c.s * (c.s +
 
 // Output elements of an M x N slice GEMM that lie in tiles the triangular skip keeps
 // (a(m) = m / tri, b(n) = n / tri; a tile goes when b < a for all its elements).
-// Tile edges TM x TN: 128 x 128 in gemm_tc.cu, 64 x 64 in gemm_f64.cu.
+// Tile edges TM x TN: 128 x 128 in gemm_tc.cu, 256 x 256 in gemm_crt.cu; 64 x 64 stands for gemm_f64.cu's.
 double tri_elems(long long M, long long N, long long tri, long long TM = 128, long long TN = 128)
 {
     if (tri <= 0) return (double)M * N;

@@ -49,7 +49,7 @@ struct OutDesc {
     int accumulate;  // 1: C += ..., 0: C = ...
 };
 
-// ---------------------------------------------------------------- FP64 DMMA GEMM
+// ---------------------------------------------------------------- FP64 GEMM
 // A(m,k) = A[am(m) + ak(k)], B(n,k) = B[bm(n) + bk(k)].  An operand whose k map is
 // the unit stride is loaded k-contiguously, any other one row-contiguously.
 struct GemmF64 {

@@ -2,7 +2,7 @@
 // modes run on, so that every mode's throughput has a roofline measured on the
 // same GPU in the same run:
 //
-//   CC_PROBE_DMMA        FP64 tensor-core MMA (mma.sync.m8n8k4.f64), the FP64 mode's GEMMs
+//   CC_PROBE_DMMA        FP64 tensor-core MMA (mma.sync.m8n8k4.f64)
 //   CC_PROBE_DFMA        scalar FP64 fused multiply-add
 //   CC_PROBE_TC_BF16     tcgen05.mma kind::f16 with BF16 operands, M=128 N=256 K=16 (emulated
 //                        FP64 slices and the BF16 mode)
