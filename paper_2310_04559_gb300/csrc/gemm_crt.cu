@@ -72,12 +72,12 @@ struct SmemCtl {
     unsigned long long full[NS], empty[NS];
     unsigned long long tfull[2], tempty[2];
     unsigned long long drain;
-    int item_q[QN];                            // this pair's items in order (-1: no work left)
-    unsigned int items_pub;                    // items written to item_q
+    unsigned long long item_q[QN];             // slot k % QN: k + 1 above this pair's item k (-1: no work left)
     unsigned int tmem_base;
     volatile int abort;
 };
-constexpr size_t SMEM_BYTES = 1024 + RING_BYTES + sizeof(SmemCtl);
+constexpr int STAGE_BYTES = 32 * CPT;          // residues of one epilogue warp: 32 rows x 128 columns
+constexpr size_t SMEM_BYTES = 1024 + RING_BYTES + EPI_WARPS * STAGE_BYTES + sizeof(SmemCtl);
 static_assert(SMEM_BYTES <= 227 * 1024, "shared memory");
 
 // What a kernel stores: residue bytes, the FP32 sums themselves (one pass), or FP64 through an index map.
@@ -181,9 +181,9 @@ __device__ __forceinline__ int item_at(SmemCtl* ctl, uint32_t k, uint32_t rank, 
 {
     unsigned long long t0 = 0;
     for (unsigned it = 0;; ++it) {
-        uint32_t n;
-        asm volatile("ld.acquire.cluster.shared::cta.u32 %0, [%1];" : "=r"(n) : "r"(smem_u32(&ctl->items_pub)) : "memory");
-        if ((int)(n - k) > 0) return *(volatile int*)&ctl->item_q[k % QN];
+        unsigned long long q;
+        asm volatile("ld.relaxed.cluster.shared::cta.u64 %0, [%1];" : "=l"(q) : "r"(smem_u32(&ctl->item_q[k % QN])) : "memory");
+        if ((uint32_t)(q >> 32) == k + 1) return (int)(uint32_t)q;
         if (it == 0) t0 = gtime();
         __nanosleep(32);
         if ((it & 15) == 15) {
@@ -316,7 +316,8 @@ __device__ __forceinline__ Item item_of(const Params& p, int i)
     return it;
 }
 
-// Leader: publishes the pair's item k to both CTAs, `item` being the counter's answer (the first one the pair's own
+// Number and index travel in one word: a count published with release semantics waited for the counter's answer, about
+// 2 us per item.  Leader: publishes the pair's item k to both CTAs, `item` being the counter's answer (the first one the pair's own
 // index), moved on past skipped tiles.  Slot k % QN is free: when item k is published, every copy of item k - 2 has
 // been issued, so the MMAs of item k - 8 have completed (a ring of 6 slots, at least one per item), so both epilogues
 // have drained item k - 10 and read its queue slot before.
@@ -324,24 +325,24 @@ __device__ __forceinline__ int publish_item(SmemCtl* ctl, const Params& p, uint3
 {
     while (item < p.nitems && item_of(p, item).skip) item = npairs + atomicAdd(p.counter, 1);
     if (item >= p.nitems || ctl->abort) item = -1;
-    for (uint32_t r = 0; r < 2; ++r) {
-        asm volatile("st.relaxed.cluster.shared::cluster.u32 [%0], %1;" ::"r"(in_cta(&ctl->item_q[k % QN], r)), "r"(item)
+    const unsigned long long q = ((unsigned long long)(k + 1) << 32) | (uint32_t)item;
+    for (uint32_t r = 0; r < 2; ++r)
+        asm volatile("st.relaxed.cluster.shared::cluster.u64 [%0], %1;" ::"r"(in_cta(&ctl->item_q[k % QN], r)), "l"(q)
                      : "memory");
-        asm volatile("st.release.cluster.shared::cluster.u32 [%0], %1;" ::"r"(in_cta(&ctl->items_pub, r)), "r"(k + 1)
-                     : "memory");
-    }
     return item;
 }
 
 template <int KIND, int OUT>
 __global__ void __launch_bounds__(THREADS, 1)
-gemm_crt_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const Params p)
+gemm_crt_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+                const __grid_constant__ CUtensorMap tmC, const Params p)
 {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* base = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     unsigned char* aring = base;
     unsigned char* bring = base + NS * TILE_BYTES;
-    SmemCtl* ctl = (SmemCtl*)(base + RING_BYTES);
+    unsigned char* stage = base + RING_BYTES;
+    SmemCtl* ctl = (SmemCtl*)(base + RING_BYTES + EPI_WARPS * STAGE_BYTES);
     constexpr int KSTEP = KIND == TC_BF16 ? 64 : 32;  // K elements per 128-byte swizzle atom
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -358,7 +359,7 @@ gemm_crt_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             mbar_init(&ctl->tempty[b], 2 * EPI_WARPS);
         }
         mbar_init(&ctl->drain, 1);
-        ctl->items_pub = 0;
+        for (int q = 0; q < QN; ++q) ctl->item_q[q] = 0;
         ctl->abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -518,27 +519,31 @@ gemm_crt_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                             *dst = add ? *dst + x : x;
                         }
                     }
-                } else {
+                } else if (OUT == OUT_F32) {
 #pragma unroll
                     for (int c = 0; c < CPT; c += 32) {
                         if (col0 + c >= w.width) continue;  // (uniform over the warp; widths are multiples of 32)
                         uint32_t r[32];
                         __syncwarp();
                         tmem_ld32(tl + (uint32_t)(buf * TN + c), r);
-                        if (OUT == OUT_F32) {
-                            float* dst = p.f32 + (long long)m * p.pitch + w.n0 + col0 + c;
-                            if (m >= p.M) continue;
+                        float* dst = p.f32 + (long long)m * p.pitch + w.n0 + col0 + c;
+                        if (m >= p.M) continue;
 #pragma unroll
-                            for (int q = 0; q < 32; q += 4)
-                                if (w.n0 + col0 + c + q < p.pitch)
-                                    *reinterpret_cast<uint4*>(dst + q) = make_uint4(r[q], r[q + 1], r[q + 2], r[q + 3]);
-                        } else {
+                        for (int q = 0; q < 32; q += 4)
+                            if (w.n0 + col0 + c + q < p.pitch)
+                                *reinterpret_cast<uint4*>(dst + q) = make_uint4(r[q], r[q + 1], r[q + 2], r[q + 3]);
+                    }
+                } else if (col0 < w.width) {
+                    // (columns beyond the width are read as well and never stored)
 #pragma unroll
-                            for (int q = 0; q < 16; ++q) {
-                                const unsigned long long x =
-                                    reduce2(f2(__uint_as_float(r[2 * q]), __uint_as_float(r[2 * q + 1])), inv, neg);
-                                sum[c / 2 + q] = pass == 0 ? x : add2(sum[c / 2 + q], x);
-                            }
+                    for (int c = 0; c < CPT; c += 32) {
+                        uint32_t r[32];
+                        tmem_ld32(tl + (uint32_t)(buf * TN + c), r);
+#pragma unroll
+                        for (int q = 0; q < 16; ++q) {
+                            const unsigned long long x =
+                                reduce2(f2(__uint_as_float(r[2 * q]), __uint_as_float(r[2 * q + 1])), inv, neg);
+                            sum[c / 2 + q] = pass == 0 ? x : add2(sum[c / 2 + q], x);
                         }
                     }
                 }
@@ -551,35 +556,62 @@ gemm_crt_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                 }
             }
             if (!ok) break;
-            if (OUT != OUT_RES) continue;
-            unsigned char* dst = p.planes + ((long long)(w.split * p.nm + w.l) * p.M + m) * p.pitch + w.n0 + col0;
-            if (m < p.M) {
+            if (OUT != OUT_RES || col0 >= w.width) continue;
+            // The bytes 128 + r, four columns to a word.  One pass leaves |r| <= (p + 1) / 2, which fits but for p = 255;
+            // sums of passes (and that modulus) are reduced once more.
+            const int plane = w.split * p.nm + w.l;
+            unsigned char* dst = p.planes + ((long long)plane * p.M + m) * p.pitch + w.n0 + col0;
+            if (p.accumulate && m < p.M) {
 #pragma unroll
-                for (int c = 0; c < CPT; c += 16) {
-                    if (w.n0 + col0 + c >= p.pitch || col0 + c >= w.width) continue;
-                    uint32_t o[4];
-                    uint4 old = make_uint4(0, 0, 0, 0);
-                    if (p.accumulate) old = *reinterpret_cast<const uint4*>(dst + c);
-                    const uint32_t ov[4] = {old.x, old.y, old.z, old.w};
+                for (int q = 0; q < CPT / 4; ++q) {
+                    if (w.n0 + col0 + 4 * q >= p.pitch) continue;
+                    const uint32_t old = *reinterpret_cast<const uint32_t*>(dst + 4 * q);
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        unsigned long long x[2];
-#pragma unroll
-                        for (int e = 0; e < 2; ++e) {
-                            x[e] = sum[c / 2 + 2 * q + e];
-                            if (p.accumulate)
-                                x[e] = add2(x[e], f2((float)((ov[q] >> (16 * e)) & 255u) - 128.0f,
-                                                     (float)((ov[q] >> (16 * e + 8)) & 255u) - 128.0f));
-                            // 2^23 + 128 + r: the low byte is 128 + r (r = 128, modulo 256 only, wraps to -128)
-                            x[e] = add2(reduce2(x[e], inv, neg), f2(8388736.0f, 8388736.0f));
-                        }
-                        o[q] = __byte_perm(__byte_perm((uint32_t)x[0], (uint32_t)(x[0] >> 32), 0x0040),
-                                           __byte_perm((uint32_t)x[1], (uint32_t)(x[1] >> 32), 0x0040), 0x5410);
-                    }
-                    *reinterpret_cast<uint4*>(dst + c) = make_uint4(o[0], o[1], o[2], o[3]);
+                    for (int e = 0; e < 2; ++e)
+                        sum[2 * q + e] = add2(sum[2 * q + e], f2((float)((old >> (16 * e)) & 255u) - 128.0f,
+                                                                 (float)((old >> (16 * e + 8)) & 255u) - 128.0f));
                 }
             }
+            if (pass > 1 || w.l == 1 || p.accumulate) {
+#pragma unroll
+                for (int q = 0; q < CPT / 2; ++q) sum[q] = reduce2(sum[q], inv, neg);
+            }
+            // 2^23 + 128 + r: the low byte is 128 + r (r = 128, modulo 256 only, wraps to -128)
+            auto word = [&](int q) {
+                const unsigned long long off = f2(8388736.0f, 8388736.0f);
+                const unsigned long long a = add2(sum[2 * q], off), b = add2(sum[2 * q + 1], off);
+                return __byte_perm(__byte_perm((uint32_t)a, (uint32_t)(a >> 32), 0x0040),
+                                   __byte_perm((uint32_t)b, (uint32_t)(b >> 32), 0x0040), 0x5410);
+            };
+            if (col0 + CPT <= w.width) {
+                // a whole half tile leaves as one TMA store per warp, 128-byte rows (16 bytes per lane and row straight
+                // to memory are half sectors in 32 different lines per instruction): 32 rows x 128 bytes, 128-byte swizzle
+                unsigned char* buf = stage + (warp - 4) * STAGE_BYTES;
+                if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+                __syncwarp();
+#pragma unroll
+                for (int c = 0; c < CPT / 16; ++c)
+                    *reinterpret_cast<uint4*>(buf + lane * CPT + ((c ^ (lane & 7)) * 16)) =
+                        make_uint4(word(4 * c), word(4 * c + 1), word(4 * c + 2), word(4 * c + 3));
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                __syncwarp();
+                const int mw = w.m0 + (int)rank * BM + q4 * 32;
+                if (lane == 0 && mw < p.M) {
+                    asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%2, %3, %4}], [%1];"
+                                 ::"l"((unsigned long long)&tmC), "r"(smem_u32(buf)), "r"(w.n0 + col0), "r"(mw), "r"(plane)
+                                 : "memory");
+                    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                }
+            } else if (m < p.M) {
+#pragma unroll
+                for (int c = 0; c < CPT / 16; ++c)
+                    if (w.n0 + col0 + 16 * c < p.pitch && col0 + 16 * c < w.width)
+                        *reinterpret_cast<uint4*>(dst + 16 * c) =
+                            make_uint4(word(4 * c), word(4 * c + 1), word(4 * c + 2), word(4 * c + 3));
+            }
         }
+        // this warp's stores have left shared memory and are complete before the CTA exits
+        if (OUT == OUT_RES && lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     }
 
     fence_before();
@@ -675,7 +707,17 @@ cudaError_t launch(const Sides& g, Params& p, cudaStream_t s)
     p.counter = counters + (OUT * 2 + KIND) * kCounterSlots + (next_slot.fetch_add(1) % kCounterSlots);
     err = cudaMemsetAsync(p.counter, 0, sizeof(int), s);
     if (err != cudaSuccess) return err;
-    CUtensorMap ma, mb;
+    CUtensorMap ma, mb, mc{};
+    if (OUT == OUT_RES) {
+        // output planes: 128 bytes x 32 rows per store
+        auto enc = get_encode();
+        cuuint64_t dims[3] = {(cuuint64_t)p.pitch, (cuuint64_t)p.M, (cuuint64_t)p.nm * p.ksplit};
+        cuuint64_t strides[2] = {(cuuint64_t)p.pitch, (cuuint64_t)p.pitch * p.M};
+        cuuint32_t box[3] = {(cuuint32_t)CPT, 32, 1}, estr[3] = {1, 1, 1};
+        if (!enc || enc(&mc, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, p.planes, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                        CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return cudaErrorInvalidValue;
+    }
     // (narrow tiles, N <= 224, are bound by the copies: B's boxes hold only the rows a tile uses)
     const int brows = 16 * (p.ubase + (p.urem > 0 ? 1 : 0));
     p.step_bytes = 2u * (uint32_t)(TILE_BYTES + brows * 128);
@@ -684,7 +726,7 @@ cudaError_t launch(const Sides& g, Params& p, cudaStream_t s)
         return cudaErrorInvalidValue;
     const int pairs = p.nitems < max_pairs ? p.nitems : max_pairs;
     cfg.gridDim = dim3((unsigned)(2 * pairs));
-    err = cudaLaunchKernelEx(&cfg, gemm_crt_kernel<KIND, OUT>, ma, mb, p);
+    err = cudaLaunchKernelEx(&cfg, gemm_crt_kernel<KIND, OUT>, ma, mb, mc, p);
     if (err != cudaSuccess) return err;
     count_launch();
     return cudaGetLastError();
