@@ -226,7 +226,7 @@ cudaError_t crt_rows(const RowSrc& src, int outer, int inner, long long ostride,
 cudaError_t crt_cols(const ColSrc& src, int nm, void* D, long long pitch, int* e, unsigned long long* scratch_max,
                      int* status, cudaStream_t st, bool premax = false);
 // T+ (rows_p pairs i <= j from pair q0, offsets rowtab) and T- (their rows_m pairs i < j from strict pair s0), packed
-// order crt_kq; rowtab NULL: the rows_p = rows_m pairs p, offsets p v^2.
+// order (crt.cuh); rowtab NULL: the rows_p = rows_m pairs p, offsets p v^2.
 cudaError_t crt_pm_f64(const double* t2, const long long* rowtab, int o, int v, long long q0, long long rows_p, long long s0,
                        long long rows_m, int nm, void* Dp, int* ep, void* Dm, int* em, long long pitch, int* status,
                        cudaStream_t st);

@@ -110,18 +110,22 @@ inline CrtRec crt_rec(int nm)
 // counts 2^(e - (bits - 1)).
 inline int crt_base(const CrtRec& c, int bits_a, int bits_b) { return c.unit - (bits_a - 1) - (bits_b - 1); }
 
-// Packed order of the entries c <= d of a v x v matrix (v4 = v rounded up to four): row c holds d = c rounded
-// down to four .. v4 - 1, entries outside c <= d < v zero, so that four consecutive d share one aligned store.
-// (v = 400: 80800 entries for v(v+1)/2 = 80200.)
-__host__ __device__ inline long long crt_kq(long long c, long long d, long long v4)
-{
-    const long long g = c / 4, s = c % 4;
-    return 4 * g * v4 - 8 * g * (g - 1) + s * (v4 - 4 * g) + (d - 4 * g);
-}
+// Packed order of the entries c <= d of a v x v matrix: 8 x 8 blocks (bc <= bd, 64 entries row by row, zero outside
+// c <= d < v), one 128-byte line of bf16 each, the blocks of a 32 x 32 tile together, tiles (tc <= td) in order.  What a
+// CTA makes of one tile pair is then one run of up to 2 KB in every residue's row, in whole lines (row by row in c it was
+// 32 segments of 64 bytes, none aligned).  v = 400: 81600 entries for v(v+1)/2 = 80200.
+__host__ __device__ inline int crt_blocks(int v) { return (v + 7) / 8; }
 inline long long crt_kq_total(long long v)
 {
-    const long long v4 = (v + 3) / 4 * 4, c = v - 1;
-    return crt_kq(c, v4 - 1, v4) + 1;
+    const long long nb = (v + 7) / 8;
+    return nb * (nb + 1) / 2 * 64;
+}
+// Blocks before tile (tc, td) of nb x nb blocks.
+__host__ __device__ inline int crt_tile_off(int tc, int td, int nb)
+{
+    const int b0 = 4 * tc, n = nb - b0 < 4 ? nb - b0 : 4;
+    const int base = b0 * nb - b0 * (b0 - 1) / 2;
+    return td == tc ? base : base + n * (n + 1) / 2 + n * 4 * (td - tc - 1);
 }
 
 #ifdef __CUDACC__

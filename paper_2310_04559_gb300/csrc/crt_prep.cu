@@ -11,7 +11,7 @@
 // per modulus.  Quads must not straddle the segments a row consists of, so segments are padded to
 // multiples of four with zeros (both operands of a GEMM use the same padded order, and zeros add nothing):
 //   plain rows of K = (o, i):    k = o inner4 + i, inner4 = inner rounded up to four
-//   packed c <= d rows (crt_kq): row c of the triangle starts at d = c rounded down to four
+//   packed c <= d rows: blocks of 8 x 8 entries (crt.cuh)
 #include <climits>
 #include <type_traits>
 
@@ -116,11 +116,12 @@ __device__ __forceinline__ long long fixed_of(double x, int e)
 // y 2^-s rounded down
 __device__ __forceinline__ long long shr_floor(long long y, int s) { return s >= 0 ? y >> min(s, 63) : y << -s; }
 
-// Residues of N quads (u = X + kCrtBias): 8 bytes per modulus and quad at out[] + l * stride (elements).  Streaming
-// stores: the rows in flight keep the L2.
+// Residues of N quads (u = X + kCrtBias): 8 bytes per modulus and quad at out[] + l * stride + k (elements).  out and
+// stride are the same for the whole CTA, only the 32-bit k differs between threads.  Streaming stores: the rows in
+// flight keep the L2.
 template <int N>
 __device__ __forceinline__ void put_quads(const unsigned long long (&u)[N][4], int nm, unsigned short* const (&out)[N],
-                                          const long long (&stride)[N])
+                                          const long long (&stride)[N], uint32_t k)
 {
     CrtPieces2 h[N][2] = {};
 #pragma unroll
@@ -135,31 +136,34 @@ __device__ __forceinline__ void put_quads(const unsigned long long (&u)[N][4], i
 #pragma unroll
         for (int i = 0; i < N; ++i) {
             const uint2 v = make_uint2(crt_residues2(h[i][0], p), crt_residues2(h[i][1], p));
-            __stcs(reinterpret_cast<uint2*>(out[i] + l * stride[i]), v);
+            unsigned short* row = out[i] + l * stride[i];
+            __stcs(reinterpret_cast<uint2*>(row + k), v);
         }
     }
 }
 
-__device__ __forceinline__ void put_quad(const long long (&X)[4], int nm, unsigned short* out, long long stride)
+__device__ __forceinline__ void put_quad(const long long (&X)[4], int nm, unsigned short* out, long long stride, uint32_t k)
 {
     const unsigned long long x[1][4] = {{X[0] + kCrtBias, X[1] + kCrtBias, X[2] + kCrtBias, X[3] + kCrtBias}};
     unsigned short* const o[1] = {out};
     const long long st[1] = {stride};
-    put_quads<1>(x, nm, o, st);
+    put_quads<1>(x, nm, o, st, k);
 }
 
-// One byte of each of four consecutive elements from every plane; `ps` bytes between planes.
+// One byte of each of four consecutive elements from every plane, at base + off in plane 0, `ps` bytes between planes
+// (a multiple of 16).  base is the same for the whole CTA where that matters.
 template <bool AL>
 struct RawQuad {
     uint32_t w[kCrtMax];
-    __device__ __forceinline__ void load(const unsigned char* p, long long ps, int nm)
+    __device__ __forceinline__ void load(const unsigned char* base, uint32_t off, long long ps, int nm)
     {
-        const uint32_t sh = AL ? 0u : (uint32_t)((uintptr_t)p & 3) * 8;
-        const unsigned char* q = AL ? p : p - ((uintptr_t)p & 3);
+        const uint32_t mis = AL ? 0u : (uint32_t)((uintptr_t)base & 3);
+        const unsigned char* q = base - mis;
+        const uint32_t o = off + mis, sh = AL ? 0u : (o & 3) * 8, oa = AL ? o : o & ~3u;
 #pragma unroll
         for (int l = 0; l < kCrtMax; ++l) {
             if (l >= kCrtMin && l >= nm) break;
-            const uint32_t* s = reinterpret_cast<const uint32_t*>(q + l * ps);
+            const uint32_t* s = reinterpret_cast<const uint32_t*>(q + l * ps + oa);
             w[l] = AL ? __ldg(s) : __funnelshift_r(__ldg(s), __ldg(s + 1), sh);
         }
     }
@@ -238,12 +242,12 @@ __device__ __forceinline__ void walk_quads(QuadIter t, uint32_t outer, const uns
                                            long long plane, int nm, F&& use)
 {
     RawQuad<AL> w;
-    if (t.o < outer) w.load(X + (long long)t.o * pitch + t.i * 4, plane, nm);
+    if (t.o < outer) w.load(X + (long long)t.o * pitch + t.i * 4, 0u, plane, nm);
     while (t.o < outer) {
         const RawQuad<AL> now = w;
         const uint32_t o = t.o, i = t.i;
         t.next();
-        if (t.o < outer) w.load(X + (long long)t.o * pitch + t.i * 4, plane, nm);
+        if (t.o < outer) w.load(X + (long long)t.o * pitch + t.i * 4, 0u, plane, nm);
         use(o, i, now);
     }
 }
@@ -290,7 +294,7 @@ __global__ void __launch_bounds__(NT) crt_rows_kernel(const RowsArg a, int nm, u
         long long v[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) v[j] = (int)i0 + j < a.inner ? fixed_of(x[j], e) : 0;
-        put_quad(v, nm, Dr + ((long long)t.o * qi + t.i) * 4, stride);
+        put_quad(v, nm, Dr, stride, (t.o * qi + t.i) * 4);
     }
 }
 
@@ -331,7 +335,7 @@ __global__ void __launch_bounds__(NT) crt_cols_kernel(const ColSrc src, int nm, 
             long long v[4];
 #pragma unroll
             for (int j = 0; j < 4; ++j) v[j] = fixed_of(S[4 * q + j][y], e);
-            put_quad(v, nm, D + r * pitch + k, stride);
+            put_quad(v, nm, D + r * pitch, stride, (uint32_t)k);
         }
     }
 }
@@ -349,6 +353,25 @@ struct TilePair {
         while (tc < nt && td >= nt) { td = td - nt + tc + 1; ++tc; }
     }
     __device__ bool ok() const { return tc < nt; }
+};
+
+// This thread's quad of a tile pair's output: entries (c, d .. d + 3) of tile (tc, td), local coordinates cl, dl, position k
+// in the packed order.  16 threads make one 8 x 8 block, so every 16 lanes write one whole line per residue.
+struct QuadPos {
+    int cl, dl;
+    uint32_t k;
+    bool live;
+    __device__ __forceinline__ QuadPos(const TilePair& t, int nb)
+    {
+        const int blk = (int)threadIdx.x >> 4, bi = blk >> 2, bj = blk & 3;
+        const int n = min(4, nb - 4 * t.tc), m = min(4, nb - 4 * t.td);
+        const bool diag = t.tc == t.td;
+        live = bi < n && bj < m && (!diag || bj >= bi);
+        cl = bi * 8 + (((int)threadIdx.x & 15) >> 1);
+        dl = bj * 8 + ((int)threadIdx.x & 1) * 4;
+        const int idx = diag ? bi * n - bi * (bi - 1) / 2 + (bj - bi) : bi * m + bj;
+        k = (uint32_t)((crt_tile_off(t.tc, t.td, nb) + idx) * 64 + (cl & 7) * 8 + (dl & 7));
+    }
 };
 
 // T+ and T- of the pairs i <= j (rowtab NULL: of all pairs, each with both rows): row p of D+ holds t_cd + t_dc (the diagonal t_cc), row p - (i + 1) - s0 of D-
@@ -369,7 +392,7 @@ __global__ void __launch_bounds__(NT) crt_pm_f64_kernel(const PmRows a, int nm, 
     __shared__ unsigned long long red[NT / 32 + 1];
     const uint32_t cs = cluster_size(), rank = cluster_rank();
     const long long r = blockIdx.x / cs;
-    const int v = a.v, v4 = (v + 3) & ~3;
+    const int v = a.v;
     const long long off = a.rowtab ? a.rowtab[r] : r * (long long)v * v;
     const double* X = a.X + off;
     const long long ij = off / ((long long)v * v);
@@ -377,8 +400,7 @@ __global__ void __launch_bounds__(NT) crt_pm_f64_kernel(const PmRows a, int nm, 
     const bool minus = (i < j || !a.rowtab) && Dm != nullptr;
     const long long rm = a.rowtab ? a.q0 + r - (i + 1) - a.s0 : r;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    const int qy = threadIdx.x >> 3, qx = (threadIdx.x & 7) * 4;
-    const int nt = (v + TT - 1) / TT;
+    const int nt = (v + TT - 1) / TT, nb = crt_blocks(v);
     int e1 = 0, e2 = 0;
     for (int pass = 0; pass < 2; ++pass) {
         unsigned long long m1 = 0, m2 = 0;
@@ -392,14 +414,15 @@ __global__ void __launch_bounds__(NT) crt_pm_f64_kernel(const PmRows a, int nm, 
                 S2[y + ty][tx] = (d2 < v && c2 < v) ? X[(long long)d2 * v + c2] : 0.0;
             }
             __syncthreads();
-            const int c = t.tc * TT + qy, d0 = t.td * TT + qx;
-            if (c >= v || d0 >= v4 || d0 + 3 < (c & ~3)) continue;
+            const QuadPos pos(t, nb);
+            if (!pos.live) continue;
+            const int c = t.tc * TT + pos.cl, d0 = t.td * TT + pos.dl;
             long long xp[4], xm[4];
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const int d = d0 + q;
                 const bool in = d >= c && d < v;
-                const double x1 = S1[qy][qx + q], x2 = S2[qx + q][qy];
+                const double x1 = S1[pos.cl][pos.dl + q], x2 = S2[pos.dl + q][pos.cl];
                 const double zp = !in ? 0.0 : (d == c ? x1 : x1 + x2);
                 const double zm = (!in || d == c || !minus) ? 0.0 : x1 - x2;
                 if (pass == 0) {
@@ -413,9 +436,8 @@ __global__ void __launch_bounds__(NT) crt_pm_f64_kernel(const PmRows a, int nm, 
                 }
             }
             if (pass == 1) {
-                const long long k = crt_kq(c, d0, v4);
-                put_quad(xp, nm, Dp + r * pitch + k, rows_p * pitch);
-                if (minus) put_quad(xm, nm, Dm + rm * pitch + k, rows_m * pitch);
+                put_quad(xp, nm, Dp + r * pitch, rows_p * pitch, pos.k);
+                if (minus) put_quad(xm, nm, Dm + rm * pitch, rows_m * pitch, pos.k);
             }
         }
         if (pass == 0) {
@@ -484,7 +506,7 @@ __global__ void __launch_bounds__(NT, 4) crt_pm_planes_kernel(const PmPlanes a, 
     const int emax = m1 + m2;
     const unsigned char* X = a.planes + al * v * a.pitch_in + bq * v;
     const int qy = threadIdx.x >> 3, qx = (threadIdx.x & 7) * 4;
-    const int nt = (v + TT - 1) / TT;
+    const int nt = (v + TT - 1) / TT, nb = crt_blocks(v);
     // walk 1: the row exponent
     const uint32_t qi = (uint32_t)v4 / 4, step = cs * NT, first = rank * NT + threadIdx.x;
     int code = INT_MIN;
@@ -508,7 +530,7 @@ __global__ void __launch_bounds__(NT, 4) crt_pm_planes_kernel(const PmPlanes a, 
         for (QuadIter t(first, step, qi); t.o < (uint32_t)v; t.next()) {
             const int d0 = (int)t.i * 4;
             RawQuad<AL> w;
-            w.load(X + (long long)t.o * a.pitch_in + d0, a.plane, rec.nm);
+            w.load(X + (long long)t.o * a.pitch_in + d0, 0u, a.plane, rec.nm);
             long long y[4];
             w.template fractions<WIDE>(rec, y);
 #pragma unroll
@@ -535,7 +557,8 @@ __global__ void __launch_bounds__(NT, 4) crt_pm_planes_kernel(const PmPlanes a, 
         long long y[4] = {0, 0, 0, 0};
         if (!zero && c < v && d0 < v) {
             RawQuad<AL> w;
-            w.load(X + (long long)c * a.pitch_in + d0, a.plane, rec.nm);
+            // (one tile's rows span less than 4 GB)
+            w.load(X + (long long)row0 * a.pitch_in + col0, (uint32_t)qy * (uint32_t)a.pitch_in + (uint32_t)qx, a.plane, rec.nm);
             w.template fractions<WIDE>(rec, y);
             const int sc = s0 - eo[c];
             const int4 e4 = *reinterpret_cast<const int4*>(ei + d0);
@@ -558,32 +581,31 @@ __global__ void __launch_bounds__(NT, 4) crt_pm_planes_kernel(const PmPlanes a, 
         tile(S1, t.tc * TT, t.td * TT);
         if (t.tc != t.td) tile(S2, t.td * TT, t.tc * TT);
         __syncthreads();
-        const int c = t.tc * TT + qy, d0 = t.td * TT + qx;
-        if (c >= v || d0 >= v4 || d0 + 3 < (c & ~3)) continue;
+        const QuadPos pos(t, nb);
+        if (!pos.live) continue;
         unsigned long long u[2][4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const long long Y1 = S1[qy][qx + j], Y2 = S2[qx + j][qy];
+            // (entries beyond v are zero in the tiles)
+            const long long Y1 = S1[pos.cl][pos.dl + j], Y2 = S2[pos.dl + j][pos.cl];
             // Y is rounded down, by half a unit on average: the sum of two makes up for it with 1 more
             u[0][j] = (unsigned long long)((Y1 + Y2 + (long long)(4 * kCrtBias + 3)) >> 2);
             u[1][j] = (unsigned long long)(((flip ? Y2 - Y1 : Y1 - Y2) + (long long)(4 * kCrtBias + 2)) >> 2);
-            const int d = d0 + j;
+            const int c = t.tc * TT + pos.cl, d = t.td * TT + pos.dl + j;
             if (t.tc == t.td && d <= c) {
                 u[0][j] = d == c ? (unsigned long long)((Y1 + (long long)(2 * kCrtBias + 1)) >> 1) : kCrtBias;
                 u[1][j] = kCrtBias;
             }
-            if (!AL && d >= v) u[0][j] = u[1][j] = kCrtBias;
         }
-        const long long k = crt_kq(c, d0, v4);
         if (Mr) {
-            unsigned short* const o[2] = {Pr + k, Mr + k};
+            unsigned short* const o[2] = {Pr, Mr};
             const long long st[2] = {stride, stride};
-            put_quads<2>(u, nm, o, st);
+            put_quads<2>(u, nm, o, st, pos.k);
         } else {
             const unsigned long long u1[1][4] = {{u[0][0], u[0][1], u[0][2], u[0][3]}};
-            unsigned short* const o[1] = {Pr + k};
+            unsigned short* const o[1] = {Pr};
             const long long st[1] = {stride};
-            put_quads<1>(u1, nm, o, st);
+            put_quads<1>(u1, nm, o, st, pos.k);
         }
     }
     cluster_done();
@@ -641,7 +663,7 @@ __global__ void __launch_bounds__(NT) crt_rows_planes_kernel(const PlaneRows a, 
         for (QuadIter t(first, step, qi); t.o < (uint32_t)a.outer; t.next()) {
             const int i0 = (int)t.i * 4;
             RawQuad<AL> w;
-            w.load(X + (long long)t.o * a.pitch_in + i0, a.plane, rec.nm);
+            w.load(X + (long long)t.o * a.pitch_in + i0, 0u, a.plane, rec.nm);
             long long y[4];
             w.template fractions<WIDE>(rec, y);
 #pragma unroll
@@ -672,9 +694,9 @@ __global__ void __launch_bounds__(NT) crt_rows_planes_kernel(const PlaneRows a, 
             u[0][j] = (zero || !(AL || i0 + j < a.inner)) ? kCrtBias
                                                           : (unsigned long long)((Y + (long long)(2 * kCrtBias + 1)) >> 1);
         }
-        unsigned short* const o[1] = {Dr + ((long long)oo * qi + i) * 4};
+        unsigned short* const o[1] = {Dr};
         const long long st[1] = {stride};
-        put_quads<1>(u, nm, o, st);
+        put_quads<1>(u, nm, o, st, (oo * qi + i) * 4);
     });
     cluster_done();
 }
