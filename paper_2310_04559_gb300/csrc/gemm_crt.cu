@@ -281,6 +281,15 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8])
         : "r"(taddr));
 }
 
+// One warp's staged 32-row box to the output at (x, y, z), unless all its rows lie beyond M.
+__device__ __forceinline__ void store_box(const CUtensorMap* map, const void* src, int x, int y, int z, int M, int lane)
+{
+    if (lane != 0 || y >= M) return;
+    asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%2, %3, %4}], [%1];"
+                 ::"l"((unsigned long long)map), "r"(smem_u32(src)), "r"(x), "r"(y), "r"(z) : "memory");
+    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+}
+
 // x - p rint(x / p) of two integers |x| <= 2^24 at once: exact, and at most p / 2 + 1 in magnitude (the quotient is
 // within 2^-8 of x / p, so it is off by one at most next to a tie); at most p / 2 for |x| < 2^16.
 __device__ __forceinline__ unsigned long long reduce2(unsigned long long x, unsigned long long inv, unsigned long long neg)
@@ -526,12 +535,17 @@ gemm_crt_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                         uint32_t r[32];
                         __syncwarp();
                         tmem_ld32(tl + (uint32_t)(buf * TN + c), r);
-                        float* dst = p.f32 + (long long)m * p.pitch + w.n0 + col0 + c;
-                        if (m >= p.M) continue;
+                        // 32 rows x 32 columns (128 bytes) per TMA store, 128-byte swizzle; the map clips what lies outside
+                        unsigned char* sb = stage + (warp - 4) * STAGE_BYTES;
+                        if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+                        __syncwarp();
 #pragma unroll
-                        for (int q = 0; q < 32; q += 4)
-                            if (w.n0 + col0 + c + q < p.pitch)
-                                *reinterpret_cast<uint4*>(dst + q) = make_uint4(r[q], r[q + 1], r[q + 2], r[q + 3]);
+                        for (int q = 0; q < 8; ++q)
+                            *reinterpret_cast<uint4*>(sb + lane * 128 + ((q ^ (lane & 7)) * 16)) =
+                                make_uint4(r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
+                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                        __syncwarp();
+                        store_box(&tmC, sb, w.n0 + col0 + c, w.m0 + (int)rank * BM + q4 * 32, 0, p.M, lane);
                     }
                 } else if (col0 < w.width) {
                     // (columns beyond the width are read as well and never stored)
@@ -595,13 +609,7 @@ gemm_crt_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                         make_uint4(word(4 * c), word(4 * c + 1), word(4 * c + 2), word(4 * c + 3));
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 __syncwarp();
-                const int mw = w.m0 + (int)rank * BM + q4 * 32;
-                if (lane == 0 && mw < p.M) {
-                    asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%2, %3, %4}], [%1];"
-                                 ::"l"((unsigned long long)&tmC), "r"(smem_u32(buf)), "r"(w.n0 + col0), "r"(mw), "r"(plane)
-                                 : "memory");
-                    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-                }
+                store_box(&tmC, buf, w.n0 + col0, w.m0 + (int)rank * BM + q4 * 32, plane, p.M, lane);
             } else if (m < p.M) {
 #pragma unroll
                 for (int c = 0; c < CPT / 16; ++c)
@@ -611,7 +619,7 @@ gemm_crt_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             }
         }
         // this warp's stores have left shared memory and are complete before the CTA exits
-        if (OUT == OUT_RES && lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+        if (OUT != OUT_F64 && lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     }
 
     fence_before();
@@ -708,13 +716,15 @@ cudaError_t launch(const Sides& g, Params& p, cudaStream_t s)
     err = cudaMemsetAsync(p.counter, 0, sizeof(int), s);
     if (err != cudaSuccess) return err;
     CUtensorMap ma, mb, mc{};
-    if (OUT == OUT_RES) {
-        // output planes: 128 bytes x 32 rows per store
+    if (OUT != OUT_F64) {
+        // output planes, or the FP32 rows: 128 bytes x 32 rows per store
+        const cuuint64_t es = OUT == OUT_RES ? 1 : 4, planes = OUT == OUT_RES ? (cuuint64_t)p.nm * p.ksplit : 1;
         auto enc = get_encode();
-        cuuint64_t dims[3] = {(cuuint64_t)p.pitch, (cuuint64_t)p.M, (cuuint64_t)p.nm * p.ksplit};
-        cuuint64_t strides[2] = {(cuuint64_t)p.pitch, (cuuint64_t)p.pitch * p.M};
-        cuuint32_t box[3] = {(cuuint32_t)CPT, 32, 1}, estr[3] = {1, 1, 1};
-        if (!enc || enc(&mc, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, p.planes, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+        cuuint64_t dims[3] = {(cuuint64_t)p.pitch, (cuuint64_t)p.M, planes};
+        cuuint64_t strides[2] = {(cuuint64_t)p.pitch * es, (cuuint64_t)p.pitch * es * p.M};
+        cuuint32_t box[3] = {(cuuint32_t)(128 / es), 32, 1}, estr[3] = {1, 1, 1};
+        if (!enc || enc(&mc, OUT == OUT_RES ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3,
+                        OUT == OUT_RES ? (void*)p.planes : (void*)p.f32, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                         CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return cudaErrorInvalidValue;
     }

@@ -31,6 +31,7 @@
 #include <cuda_bf16.h>
 
 #include <climits>
+#include <type_traits>
 
 #include "cc_internal.cuh"
 
@@ -299,17 +300,18 @@ __global__ void pm_fixed_kernel(const PmFixedSrc src, int s, int beta, __nv_bflo
     }
 }
 
-// (x1 + x2) / 2 rounded once to bf16, as from the exact sum: the FP32 sum is made odd where it is not exact
-// (its last bit then stands for all that follows), which the 16 bits to be dropped keep for the second rounding.
-__device__ __forceinline__ unsigned short half_sum_bf16(float x1, float x2)
+// s = x1 + x2 in FP32, to be rounded on to bf16: only where s sits exactly between two bf16 numbers does the part that
+// s left out decide, and there the sum is moved by one unit towards it (about one sum in 65536).
+__device__ __forceinline__ float sum_for_bf16(float x1, float x2)
 {
     const float s = __fadd_rn(x1, x2);
-    const float t = __fsub_rn(s, x1);
-    const float err = __fadd_rn(__fsub_rn(x1, __fsub_rn(s, t)), __fsub_rn(x2, t));  // x1 + x2 = s + err
     uint32_t b = __float_as_uint(s);
-    if (err != 0.0f && !(b & 1u)) b += ((__float_as_uint(err) ^ b) >> 31) ? 0xffffffffu : 1u;
-    const __nv_bfloat16 h = __float2bfloat16_rn(0.5f * __uint_as_float(b));
-    return *reinterpret_cast<const unsigned short*>(&h);
+    if ((b & 0xffffu) == 0x8000u) {
+        const float t = __fsub_rn(s, x1);
+        const float err = __fadd_rn(__fsub_rn(x1, __fsub_rn(s, t)), __fsub_rn(x2, t));  // x1 + x2 = s + err
+        if (err != 0.0f) b += ((__float_as_uint(err) ^ b) >> 31) ? 0xffffffffu : 1u;
+    }
+    return __uint_as_float(b);
 }
 
 // Integral block of the mixed modes in FP32 (the integral GEMM's own sums): V+ and V- of one row in one walk over its
@@ -321,24 +323,37 @@ __global__ void __launch_bounds__(TT * TY) pm_f32_kernel(const float* __restrict
                                                          void* __restrict__ Dp, long long pitchp, int* __restrict__ ep,
                                                          void* __restrict__ Dm, long long pitchm, int* __restrict__ em)
 {
+    typedef typename std::conditional<BF16, unsigned short, float>::type out_t;
     __shared__ float S[2][2][TT][TT + 1];  // two buffers: one barrier per tile pair
     const long long r = blockIdx.x;
     const long long ru = rtab[r];
     const float* X = X0 + (ru / Nb) * v * ldx + (ru % Nb) * v;
+    out_t* P = (out_t*)Dp + r * pitchp;
+    out_t* M = Dm ? (out_t*)Dm + r * pitchm : nullptr;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const int nt = (v + TT - 1) / TT;
+    const uint32_t ld = (uint32_t)ldx;  // (a tile's rows span less than 2^32 elements)
     int buf = 0;
     for (int tc = 0; tc < nt; ++tc) {
+        // packed positions of (c, d): kp_of = op[u] + d, km_of = op[u] - c - 1 + d, for this thread's rows c
+        uint32_t op[TT / TY];
+#pragma unroll
+        for (int u = 0; u < TT / TY; ++u) {
+            const uint32_t c = (uint32_t)(tc * TT + ty + u * TY);
+            op[u] = c * (uint32_t)v - c * (c - 1) / 2 - c;
+        }
         for (int td = tc; td < nt; ++td, buf ^= 1) {
             float (&S1)[TT][TT + 1] = S[buf][0];
             float (&S2)[TT][TT + 1] = S[buf][1];
+            const float* X1 = X + (long long)tc * TT * ldx + td * TT;
+            const float* X2 = X + (long long)td * TT * ldx + tc * TT;
             float q1[TT / TY], q2[TT / TY];
 #pragma unroll
             for (int u = 0; u < TT / TY; ++u) {
                 const int y = ty + u * TY;
-                const int c = tc * TT + y, d = td * TT + tx, d2 = td * TT + y, c2 = tc * TT + tx;
-                q1[u] = (c < v && d < v) ? __ldcs(X + c * ldx + d) : 0.0f;
-                q2[u] = (d2 < v && c2 < v) ? __ldcs(X + d2 * ldx + c2) : 0.0f;
+                const uint32_t o = (uint32_t)y * ld + (uint32_t)tx;
+                q1[u] = (tc * TT + y < v && td * TT + tx < v) ? __ldcs(X1 + o) : 0.0f;
+                q2[u] = (td * TT + y < v && tc * TT + tx < v) ? __ldcs(X2 + o) : 0.0f;
             }
 #pragma unroll
             for (int u = 0; u < TT / TY; ++u) {
@@ -352,15 +367,18 @@ __global__ void __launch_bounds__(TT * TY) pm_f32_kernel(const float* __restrict
                 const int c = tc * TT + y, d = td * TT + tx;
                 if (c >= v || d >= v || d < c) continue;
                 const float x1 = S1[y][tx], x2 = S2[tx][y];
-                const long long kp = r * pitchp + kp_of(c, d, v);
+                const uint32_t kp = op[u] + (uint32_t)d, km = kp - (uint32_t)c - 1;
                 if (BF16) {
-                    const __nv_bfloat16 h = __float2bfloat16_rn(x1);
-                    ((unsigned short*)Dp)[kp] = c == d ? *reinterpret_cast<const unsigned short*>(&h) : half_sum_bf16(x1, x2);
-                    if (Dm && c != d) ((unsigned short*)Dm)[r * pitchm + km_of(c, d, v)] = half_sum_bf16(x1, -x2);
+                    // (2 x1 for the diagonal: the halves are exact)
+                    const float sp = c == d ? x1 + x1 : sum_for_bf16(x1, x2), sm = sum_for_bf16(x1, -x2);
+                    const __nv_bfloat162 h = __floats2bfloat162_rn(0.5f * sp, 0.5f * sm);
+                    const uint32_t w = *reinterpret_cast<const uint32_t*>(&h);
+                    P[kp] = (out_t)(w & 0xffffu);
+                    if (M && c != d) M[km] = (out_t)(w >> 16);
                 } else {
                     // (FP64 sums of two FP32 values round to the same FP32 as the FP32 sum)
-                    ((float*)Dp)[kp] = tf32_round(c == d ? x1 : 0.5f * __fadd_rn(x1, x2));
-                    if (Dm && c != d) ((float*)Dm)[r * pitchm + km_of(c, d, v)] = tf32_round(0.5f * __fsub_rn(x1, x2));
+                    P[kp] = (out_t)tf32_round(c == d ? x1 : 0.5f * __fadd_rn(x1, x2));
+                    if (M && c != d) M[km] = (out_t)tf32_round(0.5f * __fsub_rn(x1, x2));
                 }
             }
         }
