@@ -51,6 +51,7 @@ constexpr int kMixedChunk = 16384;       // K elements per FP32 accumulation in 
 constexpr int kFixF = 26;                // fixed-point fraction bits (of a level-0 unit) in the Ozaki epilogue
 constexpr int kFixedBase = 2 - 2 * kBeta - kFixF;  // exponent of one fixed-point unit, before row/col exponents
 constexpr size_t kDefaultBudget = 150ull << 30;
+constexpr int kCounterInt = 16;          // item counters of the SM-pair GEMMs, in the status block of the workspace
 
 std::atomic<unsigned long long> g_wait_ns{2000000000ull};
 
@@ -511,14 +512,41 @@ int status_of(int h)
     return CC_OK;
 }
 
+// Two ints of page-locked host memory per host thread, freed with it: the status word comes back with the work it
+// reports on, instead of in a copy of its own after the stream has drained (10 us of a 130 us call).
+struct HostWords {
+    int* p = nullptr;
+    HostWords()
+    {
+        if (cudaHostAlloc((void**)&p, 2 * sizeof(int), cudaHostAllocPortable) != cudaSuccess) {
+            cudaGetLastError();
+            p = nullptr;
+        }
+    }
+    ~HostWords() { if (p) cudaFreeHost(p); }
+};
+
+// The stream's work, then the first `n` (1 or 2) words of the status block.
+int read_status(const void* ws_status, int n, cudaStream_t s)
+{
+    static thread_local HostWords hw;
+    int h[2] = {0, 0};
+    if (hw.p) {
+        CC_CU(cudaMemcpyAsync(hw.p, ws_status, n * sizeof(int), cudaMemcpyDeviceToHost, s));
+        CC_CU(cudaStreamSynchronize(s));
+        for (int i = 0; i < n; ++i) h[i] = hw.p[i];
+    } else {
+        CC_CU(cudaStreamSynchronize(s));
+        CC_CU(cudaMemcpy(h, ws_status, n * sizeof(int), cudaMemcpyDeviceToHost));
+    }
+    return status_of(h[0] | h[1]);
+}
+
 int finish(void* ws_status, int flags, cudaStream_t s)
 {
     CC_CU(cudaGetLastError());
     if (flags & CC_FLAG_NO_STATUS_SYNC) return CC_OK;
-    CC_CU(cudaStreamSynchronize(s));
-    int h = 0;
-    CC_CU(cudaMemcpy(&h, ws_status, sizeof(int), cudaMemcpyDeviceToHost));
-    return status_of(h);
+    return read_status(ws_status, 1, s);
 }
 
 // ---------------------------------------------------- tensor-core operand prep
@@ -715,6 +743,7 @@ int run_crt(const char* name, const Ctx& c, int nm, int M, int N, int K, const O
     g.accumulate = accumulate ? 1 : 0;
     g.tri = tri;
     g.status = c.status;
+    g.counter = c.status + kCounterInt;
     g.wait_ns = g_wait_ns.load();
     *out = CrtPlanes{planes, (long long)M * g.pitch, g.pitch, nm};
     return crt_gemm(name, g, st);
@@ -740,6 +769,7 @@ int run_crt_out(const char* name, const Ctx& c, int nm, int M, int N, int K, con
     g.B = Bo.D; g.pitchB = Bo.pitch; g.rowsB = Bo.rows;
     g.planes = planes; g.pitch = pitch16(N);
     g.status = c.status;
+    g.counter = c.status + kCounterInt;
     g.wait_ns = g_wait_ns.load();
     const long long items = (long long)nm * ((M + 255) / 256) * ((N + 255) / 256);
     const int pairs = std::max(1, device_sm_count() / 2);
@@ -775,6 +805,7 @@ int run_mix(const char* name, const Ctx& c, int M, int N, int K, const Operand& 
     }
     g.tri = tri;
     g.status = c.status;
+    g.counter = c.status + kCounterInt;
     g.wait_ns = g_wait_ns.load();
     const double el = tri_elems(g.M, g.N, tri, 256, 256);
     ProfScope ps(name, st, 2.0 * el * K, (double)esz_of(c.mode) * ((double)M + N) * K + el * (f32 ? 4 : 8));
@@ -791,13 +822,13 @@ int prep_crt_rows(const Ctx& c, const RowSrc& src, int outer, int inner, long lo
     return check_cuda(crt_rows(src, outer, inner, ostride, nm, op.D, op.pitch, op.e, c.status, st));
 }
 
-int prep_crt_cols(const Ctx& c, const ColSrc& src, int nm, Operand& op, unsigned long long* colmax, cudaStream_t st,
-                  bool premax = false)
+int prep_crt_cols(const Ctx& c, const ColSrc& src, int nm, Operand& op, cudaStream_t st,
+                  const unsigned long long* premax = nullptr)
 {
     ProfScope ps("split", st);
     op.rows = src.rows;
     op.pitch = pitch_crt(src.K);
-    return check_cuda(crt_cols(src, nm, op.D, op.pitch, op.e, colmax, c.status, st, premax));
+    return check_cuda(crt_cols(src, nm, op.D, op.pitch, op.e, premax, c.status, st));
 }
 
 int prep_crt_planes(const CrtPlanes& src, int nal, int nq, bool q_major, int outer, int inner, const int* eA, const int* eB,
@@ -825,7 +856,7 @@ int fwd_packed(const Ctx& c, const cc_ladder_args* a, const double* Lsrc, const 
     long long* pairtab = at<long long>(ws, Lo.pairtab);
     long long* pairtab_m = at<long long>(ws, Lo.pairtab_m);
     long long* rtab = at<long long>(ws, Lo.rtab);
-    if (!c.gen) {
+    if (!c.gen && !c.crt) {
         CC_CU(fill_pairs(c.o, c.v, 0, pairtab, st));
         CC_CU(fill_pairs(c.o, c.v, 1, pairtab_m, st));
     }
@@ -889,7 +920,7 @@ int fwd_packed(const Ctx& c, const cc_ladder_args* a, const double* Lsrc, const 
     if (!f64 && !c.hostL) {
         // L rows (a,c) are contiguous in L[P][a][c]; K = P is strided
         ColSrc ls{Lsrc, vv, vv, n, 0, plain_map(0)};
-        if (c.crt) CC_TRY(prep_crt_cols(c, ls, c.nm1, Lw, colmax, st));
+        if (c.crt) CC_TRY(prep_crt_cols(c, ls, c.nm1, Lw, st));
         else CC_TRY(prep_cols(c, ls, Lw, colmax, st));
     } else if (ozaki && c.hostL) {
         // row scales of the Ozaki split need every Cholesky vector: one streaming pass for the maxima
@@ -917,7 +948,7 @@ int fwd_packed(const Ctx& c, const cc_ladder_args* a, const double* Lsrc, const 
         Tp.rows = q1 - q0;
         Tm.rows = s1 - s0;
         if (c.crt)
-            return check_cuda(crt_pm_f64(t2, c.gen ? nullptr : pairtab + q0, c.o, c.v, q0, q1 - q0, s0, minus ? s1 - s0 : 0, c.nm2, Tp.D, Tp.e,
+            return check_cuda(crt_pm_f64(t2, c.gen, c.o, c.v, q0, q1 - q0, s0, minus ? s1 - s0 : 0, c.nm2, Tp.D, Tp.e,
                                          Tm.D, Tm.e, Tp.pitch, c.status, st));
         if (c.gen) {
             CC_CU(pm_split_f64(t2, nullptr, vv, q1 - q0, c.v, +1, 1.0, kind, c.s, kBeta, Tp.D, Tp.pitch, Tp.e, c.status, st));
@@ -949,7 +980,7 @@ int fwd_packed(const Ctx& c, const cc_ladder_args* a, const double* Lsrc, const 
                 OutDesc oq = o1;
                 if (c.crt) {
                     const ColSrc lq{buf, vv, vv, Pq, 0, plain_map(0)};
-                    CC_TRY(prep_crt_cols(c, lq, c.nm1, Lw, colmax, st, true));
+                    CC_TRY(prep_crt_cols(c, lq, c.nm1, Lw, st, colmax));
                     return run_crt("kg1_tc", c, c.nm1, Ab * c.v, Nb * c.v, (int)Pq, Lw, (long long)a0 * v, Lw,
                                    (long long)a0 * v, (unsigned char*)V, &vpl, st, v, P0 > 0);
                 }
@@ -995,12 +1026,12 @@ int fwd_packed(const Ctx& c, const cc_ladder_args* a, const double* Lsrc, const 
             CC_TRY(run_tc("kg1_tc", c, Ab * c.v, Nb * c.v, c.n, Lw, (long long)a0 * v, Lw, (long long)a0 * v, o1,
                           status, st, true, v));
         }
-        if (!c.part) CC_CU(fill_rtab(Ab, Nb, rtab, st));
+        if (!c.crt) CC_CU(fill_rtab(Ab, Nb, rtab, st));
         Vp.rows = nr; Vm.rows = nr;
         {
             ProfScope ps("split", st);
             if (c.crt) {
-                CC_CU(crt_pm_planes(vpl, c.part ? nullptr : rtab, nr, Nb, c.v, Lw.e + (long long)a0 * v,
+                CC_CU(crt_pm_planes(vpl, c.part, nr, Nb, c.v, Lw.e + (long long)a0 * v,
                                     Lw.e + (long long)b0 * v, a0 - b0, c.nm2, Vp.D, Vp.e,
                                     minus ? Vm.D : nullptr, minus ? Vm.e : nullptr, Vp.pitch, st));
             } else if (ozaki) {
@@ -1139,7 +1170,7 @@ int fwd_impl(const cc_ladder_args* a, bool tuning = false)
             ColSrc ls{Lsrc, vv, vv, n, 0, plain_map(0)};
             RowSrc ts{t2, trows, plain_map(1), c.pairs, vv};
             if (c.crt) {
-                CC_TRY(prep_crt_cols(c, ls, c.nm1, Lw, at<unsigned long long>(ws, Lo.colmax), st));
+                CC_TRY(prep_crt_cols(c, ls, c.nm1, Lw, st));
                 CC_TRY(prep_crt_rows(c, ts, c.v, c.v, v, c.nm2, tw, st));
             } else {
                 CC_TRY(prep_cols(c, ls, Lw, at<unsigned long long>(ws, Lo.colmax), st));
@@ -1208,7 +1239,7 @@ int fwd_impl(const cc_ladder_args* a, bool tuning = false)
             RowSrc lb{Lsrc, plain_map(v), split_map(v, vv, 1), v, n * v};
             if (c.crt) {
                 CC_TRY(prep_crt_rows(c, la, 1, c.v, 0, c.nm1, LwA, st));
-                CC_TRY(prep_crt_cols(c, tb, c.nm1, twB, at<unsigned long long>(ws, Lo.colmax), st));
+                CC_TRY(prep_crt_cols(c, tb, c.nm1, twB, st));
                 CC_TRY(prep_crt_rows(c, lb, c.n, c.v, vv, c.nm2, LwB, st));
             } else {
                 CC_TRY(prep_rows(c, la, LwA, st));
@@ -1389,14 +1420,14 @@ int term_impl(int which, int o, int v, int n, const double* Lov, const double* L
         // rows (p, c) of A[P][p][c] are contiguous; K = P is strided
         ColSrc as{A, np_ * v_, np_ * v_, n, 0, plain_map(0)};
         unsigned long long* colmax = at<unsigned long long>(ws, Lo.colmax);
-        if (c.crt) CC_TRY(prep_crt_cols(c, as, c.nm1, Aw, colmax, st));
+        if (c.crt) CC_TRY(prep_crt_cols(c, as, c.nm1, Aw, st));
         else CC_TRY(prep_cols(c, as, Aw, colmax, st));
         if (tc.same) {
             Bw = Aw;
         } else {
             Bw.D = at<void>(ws, Lo.Bw); Bw.e = at<int>(ws, Lo.eB);
             ColSrc bs{Bm, nq * v_, nq * v_, n, 0, plain_map(0)};
-            if (c.crt) CC_TRY(prep_crt_cols(c, bs, c.nm1, Bw, colmax, st));
+            if (c.crt) CC_TRY(prep_crt_cols(c, bs, c.nm1, Bw, st));
             else CC_TRY(prep_cols(c, bs, Bw, colmax, st));
         }
         RowSrc ts{t2, plain_map(vv), plain_map(1), (long long)o * o, vv};
@@ -1601,7 +1632,7 @@ int bwd_impl(int o, int v, int n, const double* L, const double* t2, const doubl
             if (is_tc(mode)) {
                 ColSrc ts{tt[pass], vv, vv, P, 0, plain_map(0)};  // M1 B: rows (f,d), K = ij
                 unsigned long long* colmax = at<unsigned long long>(ws, Lo.colmax);
-                if (c.crt) CC_TRY(prep_crt_cols(c, ts, c.nm1, tw, colmax, st));
+                if (c.crt) CC_TRY(prep_crt_cols(c, ts, c.nm1, tw, st));
                 else CC_TRY(prep_cols(c, ts, tw, colmax, st));
             }
             for (int e0 = 0; e0 < v; e0 += E) {
@@ -1618,7 +1649,7 @@ int bwd_impl(int o, int v, int n, const double* L, const double* t2, const doubl
                 } else if (c.crt) {
                     // planes[l][(el, b)][(f, d)], then rows (el, f) of K = (b, d)
                     ColSrc wc{Xs[pass] + (long long)e0 * v, vv, (long long)Eb * v, P, 0, plain_map(0)};
-                    CC_TRY(prep_crt_cols(c, wc, c.nm1, Ww, at<unsigned long long>(ws, Lo.colmax), st));
+                    CC_TRY(prep_crt_cols(c, wc, c.nm1, Ww, st));
                     CrtPlanes pl;
                     CC_TRY(run_crt("m1_tc", c, c.nm1, Eb * v, (int)vv, (int)P, Ww, 0, tw, 0, (unsigned char*)M1, &pl, st));
                     CC_TRY(prep_crt_planes(pl, Eb, v, false, v, v, Ww.e, tw.e, c.nm2, M1w, st));
@@ -1656,10 +1687,7 @@ int bwd_impl(int o, int v, int n, const double* L, const double* t2, const doubl
     }
     CC_CU(cudaGetLastError());
     if (flags & CC_FLAG_NO_STATUS_SYNC) return CC_OK;
-    CC_CU(cudaStreamSynchronize(st));
-    int h[2] = {0, 0};
-    CC_CU(cudaMemcpy(h, status, sizeof(h), cudaMemcpyDeviceToHost));
-    return status_of(h[0] | h[1]);
+    return read_status(status, 2, st);
 }
 
 }  // namespace

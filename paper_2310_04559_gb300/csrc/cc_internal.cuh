@@ -194,6 +194,7 @@ struct GemmCrt {
     int accumulate;    // add to the residues in the planes
     long long tri;     // triangular tile skip, a(m) = m / tri, b(n) = n / tri (0 = off)
     int* status;
+    int* counter;      // two ints, zero at launch and zero again when it ends; launches that share them run one by one
     unsigned long long wait_ns;
 };
 cudaError_t gemm_crt(const GemmCrt& g, cudaStream_t s);
@@ -208,6 +209,7 @@ struct GemmMix {
     OutDesc out;
     long long tri;
     int* status;
+    int* counter;  // as GemmCrt
     unsigned long long wait_ns;
 };
 cudaError_t gemm_mix(const GemmMix& g, cudaStream_t s);
@@ -223,17 +225,18 @@ struct CrtPlanes {
 // Rows r at src.X + rm(r), K = (o, i) at o * ostride + i, padded order o * inner4 + i.
 cudaError_t crt_rows(const RowSrc& src, int outer, int inner, long long ostride, int nm, void* D, long long pitch, int* e,
                      int* status, cudaStream_t st);
-cudaError_t crt_cols(const ColSrc& src, int nm, void* D, long long pitch, int* e, unsigned long long* scratch_max,
-                     int* status, cudaStream_t st, bool premax = false);
-// T+ (rows_p pairs i <= j from pair q0, offsets rowtab) and T- (their rows_m pairs i < j from strict pair s0), packed
-// order (crt.cuh); rowtab NULL: the rows_p = rows_m pairs p, offsets p v^2.
-cudaError_t crt_pm_f64(const double* t2, const long long* rowtab, int o, int v, long long q0, long long rows_p, long long s0,
+// premax (nullable): every row's max |x| bit pattern over a K range that may be longer than this call's.
+cudaError_t crt_cols(const ColSrc& src, int nm, void* D, long long pitch, int* e, const unsigned long long* premax,
+                     int* status, cudaStream_t st);
+// T+ (rows_p pairs i <= j from pair q0) and T- (their rows_m pairs i < j from strict pair s0), packed order (crt.cuh);
+// all_pairs: the rows_p = rows_m = o^2 pairs instead.
+cudaError_t crt_pm_f64(const double* t2, bool all_pairs, int o, int v, long long q0, long long rows_p, long long s0,
                        long long rows_m, int nm, void* Dp, int* ep, void* Dm, int* em, long long pitch, int* status,
                        cudaStream_t st);
-// V+ and (Dm not NULL) V- of the rows (al, b') = rtab[r] = al * Nb + b' (rtab NULL: r) from planes[l][(al, c)][(b', d)],
+// V+ and (Dm not NULL) V- of the rows (al, b' >= al) in order (all_b: all b') from planes[l][(al, c)][(b', d)],
 // packed order, exponents eA[al v + c] + eB[b' v + d].  Rows with b' < al + diag get the V- of (b, a) instead (V-_ba =
 // -V-_ab up to the rounding of ties: this way a pair's row is the same bits wherever it is built).
-cudaError_t crt_pm_planes(const CrtPlanes& src, const long long* rtab, long long rows, int Nb, int v, const int* eA,
+cudaError_t crt_pm_planes(const CrtPlanes& src, bool all_b, long long rows, int Nb, int v, const int* eA,
                           const int* eB, int diag, int nm, void* Dp, int* ep, void* Dm, int* em, long long pitch, cudaStream_t st);
 // Rows (al, q) of K = (o, i) from planes[l][(al, o)][(q, i)]; row index al * nq + q, or q * nal + al (q_major).
 cudaError_t crt_rows_planes(const CrtPlanes& src, int nal, int nq, bool q_major, int outer, int inner, const int* eA,

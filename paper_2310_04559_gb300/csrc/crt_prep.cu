@@ -198,6 +198,17 @@ struct RawQuad {
     }
 };
 
+// (i, j) of place p in the enumeration i-major of 0 <= i <= j < n: i n - i (i - 1) / 2 places lie before row i.
+__device__ __forceinline__ void tri_index(long long p, long long n, long long& i, long long& j)
+{
+    const double b = 2.0 * (double)n + 1.0;
+    i = (long long)(0.5 * (b - sqrt(fmax(b * b - 8.0 * (double)p, 0.0))));
+    auto before = [&](long long q) { return q * n - q * (q - 1) / 2; };
+    while (i > 0 && before(i) > p) --i;  // (the square root may be off by one)
+    while (before(i + 1) <= p) ++i;
+    j = i + (p - before(i));
+}
+
 // Row exponent of fractions y_k 2^(e_k): E with max |y_k| 2^(e_k) < 2^E, from one walk over the top words t_k of y_k.
 // With e'_k = e_k - emax <= 0 and F = max |t_k| 2^(e'_k), max |y_k| 2^(e_k) is within (F +- slack) 2^(32 + emax),
 // slack = nm * 128 + the rounding of F's float.  Where both ends give bit lengths at most one apart, the upper one
@@ -307,16 +318,63 @@ __device__ __forceinline__ long long col_off(const ColSrc& s, long long r)
 
 constexpr int CR = 32, CK = 64;  // transpose tile: 32 rows x 64 k
 
+// PREMAX: mx holds every row's largest |x| (over a K range longer than this call's); else it is found first, over the
+// whole K by the cluster's CTAs, each taking every cs-th tile of k in both walks.
+template <bool PREMAX>
 __global__ void __launch_bounds__(NT) crt_cols_kernel(const ColSrc src, int nm, const unsigned long long* __restrict__ mx,
                                                       unsigned short* __restrict__ D, long long pitch,
-                                                      int* __restrict__ e_out)
+                                                      int* __restrict__ e_out, int* __restrict__ status)
 {
     __shared__ double S[CK][CR + 1];
-    const long long r0 = (long long)blockIdx.x * CR;
+    __shared__ unsigned long long part[NT / 32][CR], top[CR];
+    __shared__ int ex[CR];
+    const uint32_t cs = cluster_size(), rank = cluster_rank();
+    const long long r0 = (long long)(blockIdx.x / cs) * CR;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const long long stride = src.rows * pitch;
     const long long roff = r0 + tx < src.rows ? col_off(src, r0 + tx) : -1;
-    for (long long k0 = (long long)blockIdx.y * CK; k0 < src.K; k0 += (long long)gridDim.y * CK) {
+    unsigned long long m = 0;
+    if (PREMAX) {
+        if (roff >= 0 && ty == 0) m = mx[r0 + tx];
+    } else {
+        if (roff >= 0)
+            for (long long k0 = (long long)rank * CK; k0 < src.K; k0 += (long long)cs * CK)
+#pragma unroll
+                for (int y = 0; y < CK; y += NT / 32) {
+                    const long long k = k0 + y + ty;
+                    if (k >= src.K) break;
+                    const unsigned long long b = (unsigned long long)__double_as_longlong(src.X[roff + k * src.ldk]) & kAbs;
+                    m = b > m ? b : m;
+                }
+        part[ty][tx] = m;
+        __syncthreads();
+        if (ty == 0) {
+            for (int w = 1; w < NT / 32; ++w) m = part[w][tx] > m ? part[w][tx] : m;
+            top[tx] = m;
+        }
+        if (cs > 1) {
+            asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+            if (ty == 0) {
+                const uint32_t mine = (uint32_t)__cvta_generic_to_shared(&top[tx]);
+                for (uint32_t r = 0; r < cs; ++r) {
+                    uint32_t a;
+                    unsigned long long o;
+                    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(mine), "r"(r));
+                    asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(o) : "r"(a) : "memory");
+                    m = o > m ? o : m;
+                }
+            }
+            asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");  // (waited for at the end)
+        }
+    }
+    if (ty == 0) {
+        ex[tx] = exp_of_maxbits(m);
+        if (rank == 0 && roff >= 0) {
+            e_out[r0 + tx] = ex[tx];
+            if (status && m >= kInf) atomicOr(status, kStatusNonfinite);
+        }
+    }
+    for (long long k0 = (long long)rank * CK; k0 < src.K; k0 += (long long)cs * CK) {
         __syncthreads();
 #pragma unroll
         for (int y = 0; y < CK; y += NT / 32) {
@@ -330,14 +388,14 @@ __global__ void __launch_bounds__(NT) crt_cols_kernel(const ColSrc src, int nm, 
         for (int y = threadIdx.x >> 4; y < CR; y += NT / 16) {
             const long long r = r0 + y, k = k0 + 4 * q;
             if (r >= src.rows || k >= src.K) continue;
-            const int e = exp_of_maxbits(mx[r]);
-            if (k == 0) e_out[r] = e;
+            const int e = ex[y];
             long long v[4];
 #pragma unroll
             for (int j = 0; j < 4; ++j) v[j] = fixed_of(S[4 * q + j][y], e);
             put_quad(v, nm, D + r * pitch, stride, (uint32_t)k);
         }
     }
+    if (!PREMAX) cluster_done();
 }
 
 // ------------------------------------------------ symmetric / antisymmetric packing
@@ -374,11 +432,11 @@ struct QuadPos {
     }
 };
 
-// T+ and T- of the pairs i <= j (rowtab NULL: of all pairs, each with both rows): row p of D+ holds t_cd + t_dc (the diagonal t_cc), row p - (i + 1) - s0 of D-
+// T+ and T- of the pairs i <= j (or of all pairs, each with both rows): row p of D+ holds t_cd + t_dc (the diagonal t_cc), row p - (i + 1) - s0 of D-
 // (pairs i < j) holds t_cd - t_dc; each with its own row exponent.
 struct PmRows {
     const double* X;
-    const long long* rowtab;  // offsets (i o + j) v^2 of the pairs of this call
+    int all_pairs;            // every pair (i, j) has both rows, in the order i o + j
     int o, v;
     long long q0, s0;         // first pair of this call in the enumeration, first strict pair
 };
@@ -393,12 +451,11 @@ __global__ void __launch_bounds__(NT) crt_pm_f64_kernel(const PmRows a, int nm, 
     const uint32_t cs = cluster_size(), rank = cluster_rank();
     const long long r = blockIdx.x / cs;
     const int v = a.v;
-    const long long off = a.rowtab ? a.rowtab[r] : r * (long long)v * v;
-    const double* X = a.X + off;
-    const long long ij = off / ((long long)v * v);
-    const int i = (int)(ij / a.o), j = (int)(ij % a.o);
-    const bool minus = (i < j || !a.rowtab) && Dm != nullptr;
-    const long long rm = a.rowtab ? a.q0 + r - (i + 1) - a.s0 : r;
+    long long i = 0, j = 1;
+    if (!a.all_pairs) tri_index(a.q0 + r, a.o, i, j);
+    const double* X = a.X + (a.all_pairs ? r : i * a.o + j) * v * v;
+    const bool minus = i < j && Dm != nullptr;
+    const long long rm = a.all_pairs ? r : a.q0 + r - (i + 1) - a.s0;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const int nt = (v + TT - 1) / TT, nb = crt_blocks(v);
     int e1 = 0, e2 = 0;
@@ -463,7 +520,7 @@ __global__ void __launch_bounds__(NT) crt_pm_f64_kernel(const PmRows a, int nm, 
 struct PmPlanes {
     const unsigned char* planes;
     long long plane, pitch_in;  // bytes between planes, per GEMM row
-    const long long* rtab;      // packed row -> al * Nb + b' (NULL: itself)
+    int all_b;                  // rows (al, all b'), else (al, b' >= al)
     int Nb, v;
     const int* eA;
     const int* eB;
@@ -482,8 +539,8 @@ __global__ void __launch_bounds__(NT, 4) crt_pm_planes_kernel(const PmPlanes a, 
     const uint32_t cs = cluster_size(), rank = cluster_rank();
     const long long r = blockIdx.x / cs;
     const int v = a.v, v4 = (v + 3) & ~3;
-    const long long ru = a.rtab ? a.rtab[r] : r;
-    const long long al = ru / a.Nb, bq = ru % a.Nb;
+    long long al = r / a.Nb, bq = r % a.Nb;
+    if (!a.all_b) tri_index(r, a.Nb, al, bq);
     const bool flip = bq < al + a.diag;
     int* eo = esm;
     int* ei = esm + v4;
@@ -821,41 +878,38 @@ cudaError_t crt_rows(const RowSrc& src, int outer, int inner, long long ostride,
                        (unsigned short*)D, pitch, e, status);
 }
 
-cudaError_t crt_cols(const ColSrc& src, int nm, void* D, long long pitch, int* e, unsigned long long* scratch_max,
-                     int* status, cudaStream_t st, bool premax)
+cudaError_t crt_cols(const ColSrc& src, int nm, void* D, long long pitch, int* e, const unsigned long long* premax,
+                     int* status, cudaStream_t st)
 {
     if (src.rows <= 0) return cudaSuccess;
-    if (!premax) {
-        cudaError_t err = cudaMemsetAsync(scratch_max, 0, sizeof(unsigned long long) * src.rows, st);
-        if (err != cudaSuccess) return err;
-        err = cols_max(src, scratch_max, status, st);
-        if (err != cudaSuccess) return err;
-    }
-    const long long ky = (src.K + CK - 1) / CK;
-    crt_cols_kernel<<<dim3((unsigned)((src.rows + CR - 1) / CR), (unsigned)(ky < 65535 ? ky : 65535)), NT, 0, st>>>(
-        src, nm, scratch_max, (unsigned short*)D, pitch, e);
-    count_launch();
-    return cudaGetLastError();
+    const long long blocks = (src.rows + CR - 1) / CR;
+    // few blocks of rows: K is spread over a cluster
+    int cs = 1;
+    while (cs < 8 && blocks * cs < 4ll * device_sm_count() && src.K > 2ll * CK * cs) cs *= 2;
+    if (premax)
+        return launch_rows(crt_cols_kernel<true>, blocks, cs, 0, st, src, nm, premax, (unsigned short*)D, pitch, e, status);
+    return launch_rows(crt_cols_kernel<false>, blocks, cs, 0, st, src, nm, (const unsigned long long*)nullptr,
+                       (unsigned short*)D, pitch, e, status);
 }
 
-cudaError_t crt_pm_f64(const double* t2, const long long* rowtab, int o, int v, long long q0, long long rows_p, long long s0,
+cudaError_t crt_pm_f64(const double* t2, bool all_pairs, int o, int v, long long q0, long long rows_p, long long s0,
                        long long rows_m, int nm, void* Dp, int* ep, void* Dm, int* em, long long pitch, int* status,
                        cudaStream_t st)
 {
     if (rows_p <= 0) return cudaSuccess;
-    const PmRows a{t2, rowtab, o, v, q0, s0};
+    const PmRows a{t2, all_pairs ? 1 : 0, o, v, q0, s0};
     const long long elems = (long long)v * v;
     return launch_rows(crt_pm_f64_kernel, rows_p, cluster_for(rows_p, elems, 8 * elems), 0, st, a, nm, (unsigned short*)Dp,
                        ep, rows_p, rows_m > 0 ? (unsigned short*)Dm : nullptr, em, rows_m, pitch, status);
 }
 
-cudaError_t crt_pm_planes(const CrtPlanes& src, const long long* rtab, long long rows, int Nb, int v, const int* eA,
+cudaError_t crt_pm_planes(const CrtPlanes& src, bool all_b, long long rows, int Nb, int v, const int* eA,
                           const int* eB, int diag, int nm, void* Dp, int* ep, void* Dm, int* em, long long pitch, cudaStream_t st)
 {
     if (rows <= 0) return cudaSuccess;
     const size_t smem = sizeof(int) * 4 * (size_t)((v + 3) & ~3);  // v up to about 12800
     if (smem > 200 * 1024) return cudaErrorInvalidValue;
-    const PmPlanes a{src.planes, src.plane, src.pitch, rtab, Nb, v, eA, eB, diag};
+    const PmPlanes a{src.planes, src.plane, src.pitch, all_b ? 1 : 0, Nb, v, eA, eB, diag};
     const CrtRec rec = crt_rec(src.nm);
     const long long elems = (long long)v * v;
     const int cs = cluster_for(rows, elems, src.nm * elems);

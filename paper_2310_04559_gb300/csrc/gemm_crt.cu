@@ -37,7 +37,6 @@
 #include <cudaTypedefs.h>
 #include <cuda_runtime.h>
 
-#include <atomic>
 #include <mutex>
 
 #include "cc_internal.cuh"
@@ -53,7 +52,6 @@ constexpr int TILE_BYTES = 128 * 128;          // 128 rows x 128 bytes
 constexpr int NS = 6;                          // ring slots (one K-step of A and B each)
 constexpr int RING_BYTES = NS * 2 * TILE_BYTES;  // 192 KB
 constexpr int QN = 16;                         // item queue slots
-constexpr int kCounterSlots = 64;              // item counters, one per launch in flight
 constexpr int EPI_WARPS = 8;
 constexpr int THREADS = 128 + 32 * EPI_WARPS;  // 384
 constexpr int TMEM_COLS = 512;                 // two accumulators of 256 columns
@@ -65,8 +63,6 @@ static_assert(128 * REG_LOW + 256 * REG_HIGH <= THREADS * 168, "register split e
 constexpr unsigned long long kSettleNs = 5000000ull;      // abort path: copies in flight land within this
 constexpr unsigned long long kDrainLimitNs = 1000000000ull;  // abort path: bound on the MMA drain
 constexpr int WARP_A = 0, WARP_MMA = 2, WARP_B = 3;
-
-__device__ int g_crt_counter[6 * kCounterSlots];  // a ring for each kernel
 
 struct SmemCtl {
     unsigned long long full[NS], empty[NS];
@@ -98,7 +94,7 @@ struct Params {
     float inv[kCrtMax], neg[kCrtMax];  // 1 / p_l, -p_l
     float* f32;                      // OUT_F32: [M][pitch]
     OutDesc out;                     // OUT_F64
-    int* counter;                    // items handed out beyond the first of each pair (zero at launch)
+    int* counter;                    // [0] items handed out beyond the first of each pair, [1] pairs done (both zero)
     int* status;
     unsigned long long wait_ns;
 };
@@ -426,6 +422,15 @@ gemm_crt_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                 const uint32_t v = u - q;
                 ok = mbar_wait(&ctl->empty[v % NS], (v / NS) & 1, ctl, rank, p);
             }
+            if (fetcher) {
+                // the last pair to finish leaves the counters zero for the next launch on them
+                __threadfence();
+                if (atomicAdd(p.counter + 1, 1) == npairs - 1) {
+                    __threadfence();
+                    p.counter[0] = 0;
+                    p.counter[1] = 0;
+                }
+            }
             if (!ok) {
                 // abort: copies into this CTA's ring may still be in flight, and the two CTAs may have stopped at
                 // different K-steps, so the leader's barriers need not complete: give the copies time to land
@@ -706,15 +711,6 @@ cudaError_t launch(const Sides& g, Params& p, cudaStream_t s)
     });
     if (attr_err != cudaSuccess) return attr_err;
 
-    // item counter: a slot of a small ring (launches in flight on other streams take other slots), zeroed in
-    // stream order before the launch
-    static std::atomic<unsigned> next_slot{0};
-    int* counters = nullptr;
-    cudaError_t err = cudaGetSymbolAddress((void**)&counters, g_crt_counter);
-    if (err != cudaSuccess) return err;
-    p.counter = counters + (OUT * 2 + KIND) * kCounterSlots + (next_slot.fetch_add(1) % kCounterSlots);
-    err = cudaMemsetAsync(p.counter, 0, sizeof(int), s);
-    if (err != cudaSuccess) return err;
     CUtensorMap ma, mb, mc{};
     if (OUT != OUT_F64) {
         // output planes, or the FP32 rows: 128 bytes x 32 rows per store
@@ -736,7 +732,7 @@ cudaError_t launch(const Sides& g, Params& p, cudaStream_t s)
         return cudaErrorInvalidValue;
     const int pairs = p.nitems < max_pairs ? p.nitems : max_pairs;
     cfg.gridDim = dim3((unsigned)(2 * pairs));
-    err = cudaLaunchKernelEx(&cfg, gemm_crt_kernel<KIND, OUT>, ma, mb, mc, p);
+    const cudaError_t err = cudaLaunchKernelEx(&cfg, gemm_crt_kernel<KIND, OUT>, ma, mb, mc, p);
     if (err != cudaSuccess) return err;
     count_launch();
     return cudaGetLastError();
@@ -765,6 +761,7 @@ cudaError_t gemm_crt(const GemmCrt& g, cudaStream_t s)
     }
     p.status = g.status;
     p.wait_ns = g.wait_ns;
+    p.counter = g.counter;
     return launch<TC_BF16, OUT_RES>(Sides{g.A, g.pitchA, g.rowsA, g.B, g.pitchB, g.rowsB}, p, s);
 }
 
@@ -786,6 +783,7 @@ cudaError_t gemm_mix(const GemmMix& g, cudaStream_t s)
     p.out = g.out;
     p.status = g.status;
     p.wait_ns = g.wait_ns;
+    p.counter = g.counter;
     const Sides sd{g.A, g.pitchA, g.rowsA, g.B, g.pitchB, g.rowsB};
     if (g.kind == TC_BF16) return g.f32 ? launch<TC_BF16, OUT_F32>(sd, p, s) : launch<TC_BF16, OUT_F64>(sd, p, s);
     return g.f32 ? launch<TC_TF32, OUT_F32>(sd, p, s) : launch<TC_TF32, OUT_F64>(sd, p, s);
