@@ -315,17 +315,21 @@ __device__ __forceinline__ float sum_for_bf16(float x1, float x2)
 }
 
 // Integral block of the mixed modes in FP32 (the integral GEMM's own sums): V+ and V- of one row in one walk over its
-// tile pairs, 4 bytes read and 2 (4) written per element.  Bound: HBM.  From an FP64 block, one kernel per sign, the
-// same split took 38 ms of the 80 at o=27/v=301/n=1501 in BF16, most of it FP64 arithmetic.
+// tile pairs, 4 bytes read and 2 (4) written per element.  Bound: HBM.  A row's tile pairs are shared by `share` CTAs,
+// so that few rows are in flight: the 128-byte pieces of a tile start anywhere, and the sectors that two
+// neighbouring tiles share are read once only if they are still in L2 when the second tile comes.  With one CTA per
+// row and streaming loads 1.7 times the block was read; o=27/v=301/n=1501 in BF16 took 9.09 ms for the split, plain loads
+// 7.66, 2 / 4 / 8 / 16 CTAs per row 6.74 / 6.16 / 5.96 / 6.23 (o=20/v=200/n=1000 in TF32: 2.38, 1.99, 1.86 / 1.73 / 1.61 / 1.71).
 template <bool BF16>
 __global__ void __launch_bounds__(TT * TY) pm_f32_kernel(const float* __restrict__ X0, long long ldx,
                                                          const long long* __restrict__ rtab, int Nb, int v,
                                                          void* __restrict__ Dp, long long pitchp, int* __restrict__ ep,
-                                                         void* __restrict__ Dm, long long pitchm, int* __restrict__ em)
+                                                         void* __restrict__ Dm, long long pitchm, int* __restrict__ em,
+                                                         int share)
 {
     typedef typename std::conditional<BF16, unsigned short, float>::type out_t;
     __shared__ float S[2][2][TT][TT + 1];  // two buffers: one barrier per tile pair
-    const long long r = blockIdx.x;
+    const long long r = blockIdx.x / share;
     const long long ru = rtab[r];
     const float* X = X0 + (ru / Nb) * v * ldx + (ru % Nb) * v;
     out_t* P = (out_t*)Dp + r * pitchp;
@@ -333,57 +337,80 @@ __global__ void __launch_bounds__(TT * TY) pm_f32_kernel(const float* __restrict
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const int nt = (v + TT - 1) / TT;
     const uint32_t ld = (uint32_t)ldx;  // (a tile's rows span less than 2^32 elements)
-    int buf = 0;
-    for (int tc = 0; tc < nt; ++tc) {
-        // packed positions of (c, d): kp_of = op[u] + d, km_of = op[u] - c - 1 + d, for this thread's rows c
-        uint32_t op[TT / TY];
+    // tile pairs (tc, td >= tc) in order, every share-th one
+    int buf = 0, tc = 0, td = (int)(blockIdx.x % share);
+    auto settle = [&] { while (tc < nt && td >= nt) { ++tc; td += tc - nt; } };
+    settle();
+    float q1[TT / TY], q2[TT / TY];
+    auto fetch = [&](int c0, int d0) {
+        const float* X1 = X + (long long)c0 * ldx + d0;
+        const float* X2 = X + (long long)d0 * ldx + c0;
+        if (d0 + TT <= v) {
 #pragma unroll
-        for (int u = 0; u < TT / TY; ++u) {
-            const uint32_t c = (uint32_t)(tc * TT + ty + u * TY);
-            op[u] = c * (uint32_t)v - c * (c - 1) / 2 - c;
-        }
-        for (int td = tc; td < nt; ++td, buf ^= 1) {
-            float (&S1)[TT][TT + 1] = S[buf][0];
-            float (&S2)[TT][TT + 1] = S[buf][1];
-            const float* X1 = X + (long long)tc * TT * ldx + td * TT;
-            const float* X2 = X + (long long)td * TT * ldx + tc * TT;
-            float q1[TT / TY], q2[TT / TY];
+            for (int u = 0; u < TT / TY; ++u) {
+                const uint32_t o = (uint32_t)(ty + u * TY) * ld + (uint32_t)tx;
+                q1[u] = __ldg(X1 + o);
+                q2[u] = __ldg(X2 + o);
+            }
+        } else {
 #pragma unroll
             for (int u = 0; u < TT / TY; ++u) {
                 const int y = ty + u * TY;
                 const uint32_t o = (uint32_t)y * ld + (uint32_t)tx;
-                q1[u] = (tc * TT + y < v && td * TT + tx < v) ? __ldcs(X1 + o) : 0.0f;
-                q2[u] = (td * TT + y < v && tc * TT + tx < v) ? __ldcs(X2 + o) : 0.0f;
+                q1[u] = (c0 + y < v && d0 + tx < v) ? __ldg(X1 + o) : 0.0f;
+                q2[u] = (d0 + y < v && c0 + tx < v) ? __ldg(X2 + o) : 0.0f;
             }
+        }
+    };
+    for (; tc < nt; buf ^= 1) {
+        const int c0 = tc * TT, d0 = td * TT;
+        float (&S1)[TT][TT + 1] = S[buf][0];
+        float (&S2)[TT][TT + 1] = S[buf][1];
+        fetch(c0, d0);
 #pragma unroll
-            for (int u = 0; u < TT / TY; ++u) {
-                S1[ty + u * TY][tx] = q1[u];
-                S2[ty + u * TY][tx] = q2[u];
+        for (int u = 0; u < TT / TY; ++u) {
+            S1[ty + u * TY][tx] = q1[u];
+            S2[ty + u * TY][tx] = q2[u];
+        }
+        td += share;
+        settle();
+        __syncthreads();
+        auto put = [&](int y, bool diag) {
+            const int c = c0 + y, d = d0 + tx;
+            const float x1 = S1[y][tx], x2 = S2[tx][y];
+            // packed positions kp_of and km_of (c, d)
+            const uint32_t kp = (uint32_t)c * (uint32_t)v - (uint32_t)c * (uint32_t)(c - 1) / 2 - (uint32_t)c + (uint32_t)d;
+            const uint32_t km = kp - (uint32_t)c - 1;
+            if (BF16) {
+                // (2 x1 for the diagonal: the halves are exact)
+                float sp = __fadd_rn(x1, x2), sm = __fsub_rn(x1, x2);
+                if (((__float_as_uint(sp) & 0xffffu) == 0x8000u) | ((__float_as_uint(sm) & 0xffffu) == 0x8000u)) {
+                    sp = sum_for_bf16(x1, x2);
+                    sm = sum_for_bf16(x1, -x2);
+                }
+                if (diag && c == d) sp = x1 + x1;
+                const __nv_bfloat162 h = __floats2bfloat162_rn(0.5f * sp, 0.5f * sm);
+                const uint32_t w = *reinterpret_cast<const uint32_t*>(&h);
+                P[kp] = (out_t)(w & 0xffffu);
+                if (M && !(diag && c == d)) M[km] = (out_t)(w >> 16);
+            } else {
+                // (FP64 sums of two FP32 values round to the same FP32 as the FP32 sum)
+                P[kp] = (out_t)tf32_round(diag && c == d ? x1 : 0.5f * __fadd_rn(x1, x2));
+                if (M && !(diag && c == d)) M[km] = (out_t)tf32_round(0.5f * __fsub_rn(x1, x2));
             }
-            __syncthreads();
+        };
+        if (c0 < d0 && d0 + TT <= v) {
+#pragma unroll
+            for (int u = 0; u < TT / TY; ++u) put(ty + u * TY, false);
+        } else {
 #pragma unroll
             for (int u = 0; u < TT / TY; ++u) {
                 const int y = ty + u * TY;
-                const int c = tc * TT + y, d = td * TT + tx;
-                if (c >= v || d >= v || d < c) continue;
-                const float x1 = S1[y][tx], x2 = S2[tx][y];
-                const uint32_t kp = op[u] + (uint32_t)d, km = kp - (uint32_t)c - 1;
-                if (BF16) {
-                    // (2 x1 for the diagonal: the halves are exact)
-                    const float sp = c == d ? x1 + x1 : sum_for_bf16(x1, x2), sm = sum_for_bf16(x1, -x2);
-                    const __nv_bfloat162 h = __floats2bfloat162_rn(0.5f * sp, 0.5f * sm);
-                    const uint32_t w = *reinterpret_cast<const uint32_t*>(&h);
-                    P[kp] = (out_t)(w & 0xffffu);
-                    if (M && c != d) M[km] = (out_t)(w >> 16);
-                } else {
-                    // (FP64 sums of two FP32 values round to the same FP32 as the FP32 sum)
-                    P[kp] = (out_t)tf32_round(c == d ? x1 : 0.5f * __fadd_rn(x1, x2));
-                    if (M && c != d) M[km] = (out_t)tf32_round(0.5f * __fsub_rn(x1, x2));
-                }
+                if (c0 + y < v && d0 + tx < v && d0 + tx >= c0 + y) put(y, true);
             }
         }
     }
-    if (threadIdx.x == 0) {
+    if (threadIdx.x == 0 && blockIdx.x % share == 0) {
         if (ep) ep[r] = 0;
         if (em) em[r] = 0;
     }
@@ -527,8 +554,11 @@ cudaError_t pm_split_f32(const float* X, long long ldx, const long long* rtab, l
 {
     if (rows <= 0) return cudaSuccess;
     if (v < 1 || (kind != 1 && kind != 2) || rows > 0x7fffffffll) return cudaErrorInvalidValue;
-    if (kind == 1) pm_f32_kernel<true><<<(unsigned)rows, TT * TY, 0, st>>>(X, ldx, rtab, Nb, v, Dp, pitchp, ep, Dm, pitchm, em);
-    else pm_f32_kernel<false><<<(unsigned)rows, TT * TY, 0, st>>>(X, ldx, rtab, Nb, v, Dp, pitchp, ep, Dm, pitchm, em);
+    const long long nt = (v + TT - 1) / TT, pairs = nt * (nt + 1) / 2;
+    long long share = pairs < 8 ? pairs : 8;
+    if (rows * share > 0x7fffffffll) share = 1;
+    auto kern = kind == 1 ? pm_f32_kernel<true> : pm_f32_kernel<false>;
+    kern<<<(unsigned)(rows * share), TT * TY, 0, st>>>(X, ldx, rtab, Nb, v, Dp, pitchp, ep, Dm, pitchm, em, (int)share);
     count_launch();
     return cudaGetLastError();
 }
