@@ -18,13 +18,14 @@
 // TMEM) alternate between passes: the epilogue reduces pass p modulo p_l into registers while the MMAs of
 // pass p + 1 run, and the item's sum once more, to the byte it stores.  The reductions are packed FP32
 // (r = x - p rint(x / p), exact), 1.5 instructions per element and pass: converting to integers instead took 8000
-// clocks per tile, as long as the MMAs of K = 1000 (8192 x 8192 x 1024, 12 moduli: 1518 TFLOP/s then, see below).
+// clocks per tile, as long as the MMAs of K = 1000 (8192 x 8192 x 1024, 12 moduli: 1518 TFLOP/s then, 2010 now).
 //
 // The same kernel runs the mixed modes' GEMMs (one bf16 or tf32 operand each, passes of 16384 elements in FP32, FP64
 // across passes), storing the FP32 sums or FP64: on 128 x 128 tiles of single SMs they had no operand reuse and were
-// bound by the copies (integral build of o=27/v=301/n=1501 in BF16: 37.2 ms, see below).
+// bound by the copies (integral build of o=27/v=301/n=1501 in BF16: 37.2 ms then, 8.5 now).
 //
-// Bound: tensor pipe (power-capped).  o=40/v=400/n=2000 integral blocks: see the table in the design notes.
+// Bound: the tensor pipe, long calls its power cap (o=40/v=400/n=2000 integral blocks: 1925 TFLOP/s, against 1724 of
+// a library GEMM that runs for seconds); below K = 512 the epilogue, 2.5 us per item.
 //
 // Roles (384 threads): warp 0 issues the A copies and fetches items (leader CTA), warp 3 the B copies,
 // one thread of the leader's warp 2 the MMAs, warps 4-11 are the epilogue (one row and 128 columns per
@@ -49,13 +50,19 @@ constexpr int BM = 128;                        // tile rows per CTA (256 per pai
 constexpr int TM = 2 * BM;                     // tile rows per pair
 constexpr int TN = 256;                        // widest tile
 constexpr int TILE_BYTES = 128 * 128;          // 128 rows x 128 bytes
-constexpr int NS = 6;                          // ring slots (one K-step of A and B each)
-constexpr int RING_BYTES = NS * 2 * TILE_BYTES;  // 192 KB
+// Two K-steps share a slot: one wait and one commit per 8 MMAs.  With a slot per step the thread that issues the MMAs was
+// the bound (555 clocks per step of 512 clocks of MMAs; 8192 x 8192 x 2048: 1936 TFLOP/s then, 2108 now, with six slots or
+// five alike).  Three steps in each of two slots copy too little ahead (1737).
+constexpr int SUB = 2;                         // K-steps per ring slot
+constexpr int NS = 3;                          // ring slots
+constexpr int SLOT_BYTES = SUB * TILE_BYTES;   // of one operand
+constexpr int RING_BYTES = NS * 2 * SLOT_BYTES;  // 192 KB
 constexpr int QN = 16;                         // item queue slots
 constexpr int EPI_WARPS = 8;
 constexpr int THREADS = 128 + 32 * EPI_WARPS;  // 384
 constexpr int TMEM_COLS = 512;                 // two accumulators of 256 columns
 constexpr int CPT = TN / 2;                    // accumulator columns per epilogue thread
+static_assert(kCrtChunk % (64 * SUB) == 0, "passes end with a ring slot");
 constexpr int kReduceEvery = 60;               // passes between reductions of the running sums (far below 2^24)
 // setmaxnreg split of the launch's 384 x 168 registers: 128 x 56 + 256 x 216 = 62464 <= 64512
 constexpr int REG_LOW = 56, REG_HIGH = 216;
@@ -79,6 +86,19 @@ static_assert(SMEM_BYTES <= 227 * 1024, "shared memory");
 // What a kernel stores: residue bytes, the FP32 sums themselves (one pass), or FP64 through an index map.
 enum OutKind { OUT_RES = 0, OUT_F32 = 1, OUT_F64 = 2 };
 
+// Division of 0 <= n < 2^31 by a fixed d >= 1: with 2^s < d <= 2^(s + 1), mul = ceil(2^(32 + s) / d) is less than d above
+// the quotient, so n times the excess stays below 2^(32 + s).
+struct FastDiv {
+    uint32_t d, mul, s;
+    FastDiv() = default;
+    explicit FastDiv(long long div) : d((uint32_t)div), mul(0), s(0)
+    {
+        while (d > 1 && (2ull << s) < d) ++s;
+        if (d > 1) mul = (uint32_t)(((1ull << (32 + s)) + d - 1) / d);
+    }
+    __device__ __forceinline__ int div(int n) const { return d == 1 ? n : (int)(__umulhi((uint32_t)n, mul) >> s); }
+};
+
 struct Params {
     int M, N, K, nm;
     int chunk;                       // K elements per pass
@@ -86,6 +106,7 @@ struct Params {
     int ksplit, kper;                // K split s owns [s*kper, min(K, (s+1)*kper))
     long long tri;                   // triangular tile skip (0 = off): b(n) = n / tri < a(m) = m / tri
     int tiles_m, tiles_n, group_m, nitems;
+    FastDiv by_l, by_tiles, by_group, by_gm, by_last, by_tri;  // by_gm, by_last: rows of tiles in a group, in the last one
     uint32_t step_bytes;             // bytes both CTAs copy per K-step
     int ubase, urem;                 // tile column j: ubase units of 32 columns, one more where j < urem
     unsigned char* planes;           // [ksplit][nm][M][pitch]
@@ -171,6 +192,15 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long* b, uint32_t parity
         }
     }
 }
+
+// Ring slot of the next K-step and the parity of its turn.
+struct Ring {
+    uint32_t slot = 0, phase = 0;
+    __device__ __forceinline__ void next()
+    {
+        if (++slot == NS) { slot = 0; phase ^= 1; }
+    }
+};
 
 // Item k of this pair (-1: no work left, or abort); bounded.
 __device__ __forceinline__ int item_at(SmemCtl* ctl, uint32_t k, uint32_t rank, const Params& p)
@@ -294,7 +324,15 @@ __device__ __forceinline__ unsigned long long reduce2(unsigned long long x, unsi
     return fma2(add2(fma2(x, inv, big), nbig), neg, x);
 }
 
-// Item i: modulus-major, then K split, then tiles rastered in groups of group_m tile rows.
+// The same with the quotient of x + 1/4 (|x| < 2^16): ties of even p go to -p / 2, and -p / 2 <= result < p / 2.
+__device__ __forceinline__ unsigned long long reduce2_low(unsigned long long x, unsigned long long inv, unsigned long long neg)
+{
+    const unsigned long long big = f2(12582912.0f, 12582912.0f), nbig = f2(-12582912.0f, -12582912.0f);
+    return fma2(add2(fma2(add2(x, f2(0.25f, 0.25f)), inv, big), nbig), neg, x);
+}
+
+// Item i: modulus-major, then K split, then tiles rastered in groups of group_m tile rows.  Every role decodes every item,
+// so the divisions are multiplications (six 32-bit divisions: 0.2 us of an item's 2.6 at K = 64, and of its 5.7 at K = 1024).
 struct Item {
     int l, split, m0, n0, width;  // width: columns of the MMAs (a multiple of 32)
     bool skip;
@@ -302,33 +340,31 @@ struct Item {
 
 __device__ __forceinline__ Item item_of(const Params& p, int i)
 {
-    const int ntiles = p.tiles_m * p.tiles_n;
-    const int per_l = ntiles * p.ksplit;
     Item it;
-    it.l = i / per_l;
-    const int rem = i % per_l;
-    it.split = rem / ntiles;
-    const int t = rem % ntiles;
-    const int per_group = p.group_m * p.tiles_n;
-    const int first_m = (t / per_group) * p.group_m;
-    const int gm = min(p.tiles_m - first_m, p.group_m);
-    it.m0 = (first_m + (t % per_group) % gm) * TM;
-    const int j = (t % per_group) / gm;
+    it.l = p.by_l.div(i);
+    const int rem = i - it.l * (int)p.by_l.d;
+    it.split = p.by_tiles.div(rem);
+    const int t = rem - it.split * (int)p.by_tiles.d;
+    const int g = p.by_group.div(t), in = t - g * (int)p.by_group.d;
+    const int first_m = g * p.group_m;
+    const bool last = p.tiles_m - first_m < p.group_m;
+    const int j = last ? p.by_last.div(in) : p.by_gm.div(in);
+    it.m0 = (first_m + in - j * (int)(last ? p.by_last.d : p.by_gm.d)) * TM;
     it.n0 = 32 * (j * p.ubase + min(j, p.urem));
     it.width = 32 * (p.ubase + (j < p.urem ? 1 : 0));
     // every element of the tile has b(n) < a(m)
-    it.skip = p.tri > 0 && min(p.N - 1, it.n0 + it.width - 1) / (int)p.tri < it.m0 / (int)p.tri;
+    it.skip = p.tri > 0 && p.by_tri.div(min(p.N - 1, it.n0 + it.width - 1)) < p.by_tri.div(it.m0);
     return it;
 }
 
 // Number and index travel in one word: a count published with release semantics waited for the counter's answer, about
 // 2 us per item.  Leader: publishes the pair's item k to both CTAs, `item` being the counter's answer (the first one the pair's own
 // index), moved on past skipped tiles.  Slot k % QN is free: when item k is published, every copy of item k - 2 has
-// been issued, so the MMAs of item k - 8 have completed (a ring of 6 slots, at least one per item), so both epilogues
-// have drained item k - 10 and read its queue slot before.
+// been issued, so the MMAs of item k - 5 have completed (a ring of 3 slots, at least one per item), so both epilogues
+// have drained item k - 7 and read its queue slot before.
 __device__ __forceinline__ int publish_item(SmemCtl* ctl, const Params& p, uint32_t k, int item, int npairs)
 {
-    while (item < p.nitems && item_of(p, item).skip) item = npairs + atomicAdd(p.counter, 1);
+    while (p.tri > 0 && item < p.nitems && item_of(p, item).skip) item = npairs + atomicAdd(p.counter, 1);
     if (item >= p.nitems || ctl->abort) item = -1;
     const unsigned long long q = ((unsigned long long)(k + 1) << 32) | (uint32_t)item;
     for (uint32_t r = 0; r < 2; ++r)
@@ -345,7 +381,7 @@ gemm_crt_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* base = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     unsigned char* aring = base;
-    unsigned char* bring = base + NS * TILE_BYTES;
+    unsigned char* bring = base + NS * SLOT_BYTES;
     unsigned char* stage = base + RING_BYTES;
     SmemCtl* ctl = (SmemCtl*)(base + RING_BYTES + EPI_WARPS * STAGE_BYTES);
     constexpr int KSTEP = KIND == TC_BF16 ? 64 : 32;  // K elements per 128-byte swizzle atom
@@ -389,6 +425,7 @@ gemm_crt_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             unsigned char* ring = isA ? aring : bring;
             const bool fetcher = isA && rank == 0;
             uint32_t u = 0;  // K-steps issued
+            Ring at;
             bool ok = true;
             // The fetcher publishes the item after the one being copied, and asks the counter for one more whose answer
             // it only looks at an item later: the atomic's latency (about 1 us, as long as an item of K = 256) then
@@ -410,11 +447,14 @@ gemm_crt_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                 const int row = isA ? (int)(p.rowA0 + w.m0) + (int)rank * BM
                                     : (int)(p.rowB0 + w.n0) + (int)rank * (w.width >> 1);
                 const int kbeg = w.split * p.kper, kend = min(p.K, kbeg + p.kper);
-                for (int kb = kbeg; kb < kend; kb += KSTEP, ++u) {
-                    const uint32_t s = u % NS;
-                    if (!mbar_wait(&ctl->empty[s], ((u / NS) & 1) ^ 1, ctl, rank, p)) { ok = false; break; }
-                    if (fetcher) mbar_expect_tx(&ctl->full[s], p.step_bytes);  // A and B tiles of both CTAs
-                    tma_load(ring + s * TILE_BYTES, map, in_cta(&ctl->full[s], 0), kb, row, w.l);
+                for (int kb = kbeg; kb < kend; kb += SUB * KSTEP, ++u, at.next()) {
+                    const uint32_t s = at.slot;
+                    if (!mbar_wait(&ctl->empty[s], at.phase ^ 1, ctl, rank, p)) { ok = false; break; }
+                    const bool both = kb + KSTEP < kend;
+                    if (fetcher) mbar_expect_tx(&ctl->full[s], both ? SUB * p.step_bytes : p.step_bytes);  // A and B tiles of both CTAs
+                    const uint32_t bar = in_cta(&ctl->full[s], 0);
+                    tma_load(ring + s * SLOT_BYTES, map, bar, kb, row, w.l);
+                    if (both) tma_load(ring + s * SLOT_BYTES + TILE_BYTES, map, bar, kb + KSTEP, row, w.l);
                 }
             }
             // the last use of every slot is released: no commit still targets this CTA's barriers when it leaves
@@ -440,7 +480,8 @@ gemm_crt_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         } else if (warp == WARP_MMA && rank == 0 && lane == 0) {
             // ------------------------------------------------------------ MMA
             const unsigned long long adesc0 = smem_desc(aring), bdesc0 = smem_desc(bring);
-            uint32_t u = 0, npass = 0;
+            uint32_t npass = 0;
+            Ring at;
             bool ok = true, any = false;
             for (uint32_t k = 0; ok; ++k) {
                 const int item = item_at(ctl, k, rank, p);
@@ -455,12 +496,12 @@ gemm_crt_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                     const uint32_t d = tmem + (uint32_t)(buf * TN);
                     const int k1 = min(kend, k0 + p.chunk);
                     uint32_t acc = 0;
-                    for (int kb = k0; kb < k1; kb += KSTEP, ++u) {
-                        const uint32_t s = u % NS;
-                        if (!mbar_wait(&ctl->full[s], (u / NS) & 1, ctl, rank, p)) { ok = false; break; }
+                    for (int kb = k0; kb < k1; kb += SUB * KSTEP, at.next()) {
+                        const uint32_t s = at.slot;
+                        if (!mbar_wait(&ctl->full[s], at.phase, ctl, rank, p)) { ok = false; break; }
                         fence_after();
-                        const unsigned long long ad = adesc0 + (unsigned long long)(s * (TILE_BYTES >> 4));
-                        const unsigned long long bd = bdesc0 + (unsigned long long)(s * (TILE_BYTES >> 4));
+                        const unsigned long long ad = adesc0 + (unsigned long long)(s * (SLOT_BYTES >> 4));
+                        const unsigned long long bd = bdesc0 + (unsigned long long)(s * (SLOT_BYTES >> 4));
                         any = true;
                         // four MMAs per 128-byte row: advance the start address by 32 bytes each
                         mma<KIND>(d, ad, bd, idesc, acc);
@@ -468,6 +509,13 @@ gemm_crt_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                         mma<KIND>(d, ad + 4, bd + 4, idesc, 1u);
                         mma<KIND>(d, ad + 6, bd + 6, idesc, 1u);
                         acc = 1;
+                        if (kb + KSTEP < k1) {
+                            constexpr unsigned long long next = TILE_BYTES >> 4;
+                            mma<KIND>(d, ad + next, bd + next, idesc, 1u);
+                            mma<KIND>(d, ad + next + 2, bd + next + 2, idesc, 1u);
+                            mma<KIND>(d, ad + next + 4, bd + next + 4, idesc, 1u);
+                            mma<KIND>(d, ad + next + 6, bd + next + 6, idesc, 1u);
+                        }
                         commit_both(&ctl->empty[s]);
                     }
                     if (!ok) break;
@@ -576,8 +624,8 @@ gemm_crt_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             }
             if (!ok) break;
             if (OUT != OUT_RES || col0 >= w.width) continue;
-            // The bytes 128 + r, four columns to a word.  One pass leaves |r| <= (p + 1) / 2, which fits but for p = 255;
-            // sums of passes (and that modulus) are reduced once more.
+            // The bytes 128 + r, four columns to a word.  One pass leaves |r| <= (p + 1) / 2, which fits but for p = 256 and
+            // 255; sums of passes (and those moduli) are reduced once more, to -p / 2 <= r < p / 2.
             const int plane = w.split * p.nm + w.l;
             unsigned char* dst = p.planes + ((long long)plane * p.M + m) * p.pitch + w.n0 + col0;
             if (p.accumulate && m < p.M) {
@@ -591,16 +639,15 @@ gemm_crt_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                                                                  (float)((old >> (16 * e + 8)) & 255u) - 128.0f));
                 }
             }
-            if (pass > 1 || w.l == 1 || p.accumulate) {
+            if (pass > 1 || w.l <= 1 || p.accumulate) {
 #pragma unroll
-                for (int q = 0; q < CPT / 2; ++q) sum[q] = reduce2(sum[q], inv, neg);
+                for (int q = 0; q < CPT / 2; ++q) sum[q] = reduce2_low(sum[q], inv, neg);
             }
-            // 2^23 + 128 + r: the low byte is 128 + r (r = 128, modulo 256 only, wraps to -128)
+            // columns c and c + 2 as 2^23 + (128 + r_c) + 256 (128 + r_c+2), so two packed instructions and a permute make a word
             auto word = [&](int q) {
-                const unsigned long long off = f2(8388736.0f, 8388736.0f);
-                const unsigned long long a = add2(sum[2 * q], off), b = add2(sum[2 * q + 1], off);
-                return __byte_perm(__byte_perm((uint32_t)a, (uint32_t)(a >> 32), 0x0040),
-                                   __byte_perm((uint32_t)b, (uint32_t)(b >> 32), 0x0040), 0x5410);
+                const unsigned long long off = f2(8421504.0f, 8421504.0f), shift = f2(256.0f, 256.0f);
+                const unsigned long long a = fma2(sum[2 * q + 1], shift, add2(sum[2 * q], off));
+                return __byte_perm((uint32_t)a, (uint32_t)(a >> 32), 0x5140);
             };
             if (col0 + CPT <= w.width) {
                 // a whole half tile leaves as one TMA store per warp, 128-byte rows (16 bytes per lane and row straight
@@ -683,6 +730,13 @@ cudaError_t launch(const Sides& g, Params& p, cudaStream_t s)
     const long long nitems = (long long)p.tiles_m * p.tiles_n * p.ksplit * p.nm;
     if (nitems > 0x7fffffffll - (1 << 20)) return cudaErrorInvalidConfiguration;
     p.nitems = (int)nitems;
+    const long long ntiles = (long long)p.tiles_m * p.tiles_n;
+    p.by_l = FastDiv(ntiles * p.ksplit);
+    p.by_tiles = FastDiv(ntiles);
+    p.by_group = FastDiv((long long)p.group_m * p.tiles_n);
+    p.by_gm = FastDiv(p.group_m);
+    p.by_last = FastDiv(p.tiles_m % p.group_m ? p.tiles_m % p.group_m : p.group_m);
+    p.by_tri = FastDiv(p.tri > 0 ? std::min(p.tri, 0x7fffffffll) : 1);
 
     cudaLaunchConfig_t cfg{};
     cfg.blockDim = dim3(THREADS);
@@ -769,7 +823,7 @@ cudaError_t gemm_mix(const GemmMix& g, cudaStream_t s)
 {
     if (g.M <= 0 || g.N <= 0) return cudaSuccess;
     const int kstep = g.kind == TC_BF16 ? 64 : 32;
-    if (g.K <= 0 || g.chunk <= 0 || g.chunk % kstep || g.tri < 0) return cudaErrorInvalidValue;
+    if (g.K <= 0 || g.chunk <= 0 || g.chunk % (SUB * kstep) || g.tri < 0) return cudaErrorInvalidValue;
     if (g.f32 && (g.K > g.chunk || g.pitch < g.N || g.pitch % 4)) return cudaErrorInvalidValue;
     Params p{};
     p.M = g.M; p.N = g.N; p.K = g.K; p.nm = 1;
