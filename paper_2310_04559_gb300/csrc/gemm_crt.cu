@@ -357,6 +357,20 @@ __device__ __forceinline__ Item item_of(const Params& p, int i)
     return it;
 }
 
+// The first item after skipped item i that may not be skipped: a group's leading columns of tiles are skipped in all its
+// rows together.
+__device__ __forceinline__ int after_skipped(const Params& p, int i)
+{
+    const int rem = i - p.by_l.div(i) * (int)p.by_l.d, t = rem - p.by_tiles.div(rem) * (int)p.by_tiles.d;
+    const int g = p.by_group.div(t), in = t - g * (int)p.by_group.d;
+    const int first_m = g * p.group_m, gm = min(p.tiles_m - first_m, p.group_m);
+    const int amin = p.by_tri.div(first_m * TM);
+    auto end_of = [&](int j) { return min(p.N, 32 * ((j + 1) * p.ubase + min(j + 1, p.urem))); };  // columns up to tile j
+    int j = max(0, amin * (int)p.by_tri.d / 32 / (p.ubase + 1) - 1);  // (a tile has at most ubase + 1 units)
+    while (j < p.tiles_n && p.by_tri.div(end_of(j) - 1) < amin) ++j;
+    return max(i + 1, i - in + j * gm);
+}
+
 // Number and index travel in one word: a count published with release semantics waited for the counter's answer, about
 // 2 us per item.  Leader: publishes the pair's item k to both CTAs, `item` being the counter's answer (the first one the pair's own
 // index), moved on past skipped tiles.  Slot k % QN is free: when item k is published, every copy of item k - 2 has
@@ -364,7 +378,12 @@ __device__ __forceinline__ Item item_of(const Params& p, int i)
 // have drained item k - 7 and read its queue slot before.
 __device__ __forceinline__ int publish_item(SmemCtl* ctl, const Params& p, uint32_t k, int item, int npairs)
 {
-    while (p.tri > 0 && item < p.nitems && item_of(p, item).skip) item = npairs + atomicAdd(p.counter, 1);
+    while (p.tri > 0 && item < p.nitems && item_of(p, item).skip) {
+        // the counter jumps over a run of skipped items (one by one they took 1 us each, shared by the pairs)
+        const int to = after_skipped(p, item);
+        if (to > item + 1) atomicMax(p.counter, to - npairs);
+        item = npairs + atomicAdd(p.counter, 1);
+    }
     if (item >= p.nitems || ctl->abort) item = -1;
     const unsigned long long q = ((unsigned long long)(k + 1) << 32) | (uint32_t)item;
     for (uint32_t r = 0; r < 2; ++r)
