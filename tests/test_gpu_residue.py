@@ -125,3 +125,28 @@ def test_wait_expiry_in_the_ladder(dev):
     finally:
         lib.cc_ladder_set_wait_limit_ns(0)
     assert np.array_equal(B.ladder_forward(Lg, tg, symmetric=True).cpu().numpy(), want)
+
+
+@pytest.mark.parametrize("K", [1, 2, 3, 4, 5, 127, 128, 129, 255, 256, 257])
+def test_short_rows(dev, K):
+    """Rows up to 256 elements are split by a warp each, longer ones by a CTA; integers come out exactly."""
+    rng = np.random.default_rng(K)
+    A, Bm = rng.integers(-999, 1000, (13, K)).astype(np.float64), rng.integers(-999, 1000, (7, K)).astype(np.float64)
+    A[3] = 0.0
+    A[5] *= 2.0 ** -300
+    C = B.gemm(cu(A, dev), cu(Bm, dev)).cpu().numpy()
+    assert np.array_equal(C, A @ Bm.T)
+    A[12, K - 1] = np.nan
+    with pytest.raises(_lib.LadderError):
+        B.gemm(cu(A, dev), cu(Bm, dev))
+
+
+@pytest.mark.parametrize("o,v,n", [(1, 3, 2), (2, 5, 3), (3, 9, 7), (2, 33, 7), (2, 67, 4)])
+def test_short_rows_of_several_segments(dev, o, v, n):
+    """Cholesky-first order: L rows of v and of n segments of v entries, one side and the other of 256 elements."""
+    L, t2 = (x.numpy() for x in synth.ladder_inputs_torch(o, v, n, device="cpu"))
+    R = B.ladder_forward(cu(L, dev), cu(t2, dev), symmetric=True, order="cholesky_first").cpu().numpy()
+    ref = np.einsum("Pac,Pbd,ijcd->ijab", L, L, t2, optimize=True)
+    # two roundings of rows of v, and of n v, elements to 42 bits of their largest entry
+    scale = np.abs(L).max() ** 2 * np.abs(t2).max() * n * v * v
+    assert np.abs(R - ref).max() <= scale * 2.0 ** -38
