@@ -280,6 +280,14 @@ __device__ __forceinline__ void commit_both(unsigned long long* bar)
         ::"r"(smem_u32(bar)), "h"((unsigned short)3) : "memory");
 }
 
+// The same lane of a converged warp each time; what it issues keeps its operands in uniform registers.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t r;
+    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(r));
+    return r != 0;
+}
+
 __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
@@ -496,58 +504,65 @@ gemm_crt_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                 const unsigned long long t0 = gtime();
                 while (gtime() - t0 < kSettleNs) __nanosleep(1000);
             }
-        } else if (warp == WARP_MMA && rank == 0 && lane == 0) {
+        } else if (warp == WARP_MMA && rank == 0) {
             // ------------------------------------------------------------ MMA
             const unsigned long long adesc0 = smem_desc(aring), bdesc0 = smem_desc(bring);
             uint32_t npass = 0;
             Ring at;
             bool ok = true, any = false;
             for (uint32_t k = 0; ok; ++k) {
-                const int item = item_at(ctl, k, rank, p);
+                const int item = __shfl_sync(0xffffffffu, item_at(ctl, k, rank, p), 0);
                 if (item < 0) break;
                 const Item w = item_of(p, item);
                 const uint32_t idesc = instr_desc<KIND>(w.width);
                 const int kbeg = w.split * p.kper, kend = min(p.K, kbeg + p.kper);
                 for (int k0 = kbeg; k0 < kend && ok; k0 += p.chunk) {
                     const int buf = (int)(npass & 1);
-                    if (!mbar_wait(&ctl->tempty[buf], ((npass >> 1) & 1) ^ 1, ctl, rank, p)) { ok = false; break; }
+                    ok = __all_sync(0xffffffffu, mbar_wait(&ctl->tempty[buf], ((npass >> 1) & 1) ^ 1, ctl, rank, p));
+                    if (!ok) break;
                     fence_after();
                     const uint32_t d = tmem + (uint32_t)(buf * TN);
                     const int k1 = min(kend, k0 + p.chunk);
                     uint32_t acc = 0;
                     for (int kb = k0; kb < k1; kb += SUB * KSTEP, at.next()) {
                         const uint32_t s = at.slot;
-                        if (!mbar_wait(&ctl->full[s], at.phase, ctl, rank, p)) { ok = false; break; }
+                        ok = __all_sync(0xffffffffu, mbar_wait(&ctl->full[s], at.phase, ctl, rank, p));
+                        if (!ok) break;
                         fence_after();
                         const unsigned long long ad = adesc0 + (unsigned long long)(s * (SLOT_BYTES >> 4));
                         const unsigned long long bd = bdesc0 + (unsigned long long)(s * (SLOT_BYTES >> 4));
                         any = true;
-                        // four MMAs per 128-byte row: advance the start address by 32 bytes each
-                        mma<KIND>(d, ad, bd, idesc, acc);
-                        mma<KIND>(d, ad + 2, bd + 2, idesc, 1u);
-                        mma<KIND>(d, ad + 4, bd + 4, idesc, 1u);
-                        mma<KIND>(d, ad + 6, bd + 6, idesc, 1u);
-                        acc = 1;
-                        if (kb + KSTEP < k1) {
-                            constexpr unsigned long long next = TILE_BYTES >> 4;
-                            mma<KIND>(d, ad + next, bd + next, idesc, 1u);
-                            mma<KIND>(d, ad + next + 2, bd + next + 2, idesc, 1u);
-                            mma<KIND>(d, ad + next + 4, bd + next + 4, idesc, 1u);
-                            mma<KIND>(d, ad + next + 6, bd + next + 6, idesc, 1u);
+                        if (elect_one()) {
+                            // four MMAs per 128-byte row: advance the start address by 32 bytes each
+                            mma<KIND>(d, ad, bd, idesc, acc);
+                            mma<KIND>(d, ad + 2, bd + 2, idesc, 1u);
+                            mma<KIND>(d, ad + 4, bd + 4, idesc, 1u);
+                            mma<KIND>(d, ad + 6, bd + 6, idesc, 1u);
+                            if (kb + KSTEP < k1) {
+                                constexpr unsigned long long next = TILE_BYTES >> 4;
+                                mma<KIND>(d, ad + next, bd + next, idesc, 1u);
+                                mma<KIND>(d, ad + next + 2, bd + next + 2, idesc, 1u);
+                                mma<KIND>(d, ad + next + 4, bd + next + 4, idesc, 1u);
+                                mma<KIND>(d, ad + next + 6, bd + next + 6, idesc, 1u);
+                            }
+                            commit_both(&ctl->empty[s]);
                         }
-                        commit_both(&ctl->empty[s]);
+                        __syncwarp();
+                        acc = 1;
                     }
                     if (!ok) break;
-                    commit_both(&ctl->tfull[buf]);
+                    if (elect_one()) commit_both(&ctl->tfull[buf]);
+                    __syncwarp();
                     ++npass;
                 }
             }
             // both buffers' last drains (the peer's arrivals land here) are done
             for (uint32_t q = npass > 2 ? npass - 2 : 0; q < npass && ok; ++q)
-                ok = mbar_wait(&ctl->tempty[q & 1], (q >> 1) & 1, ctl, rank, p);
+                ok = __all_sync(0xffffffffu, mbar_wait(&ctl->tempty[q & 1], (q >> 1) & 1, ctl, rank, p));
             if (any) {
                 // every MMA has completed before TMEM is released
-                commit_both(&ctl->drain);
+                if (elect_one()) commit_both(&ctl->drain);
+                __syncwarp();
                 const unsigned long long t0 = gtime();
                 while (!mbar_try(&ctl->drain, 0)) {
                     if (gtime() - t0 > kDrainLimitNs) { atomicOr(p.status, kStatusDrainExpired); break; }
