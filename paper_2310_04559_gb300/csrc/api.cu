@@ -125,11 +125,18 @@ inline size_t planes_bytes(long long nm, long long M, long long N) { return (siz
 // Padded length of a row K = (o, i), o < outer, i < inner (crt_prep.cu).
 inline long long k_pad(long long outer, long long inner) { return outer * ((inner + 3) & ~3ll); }
 
-// Bytes for the result planes of an M x N residue GEMM, either orientation; small results get room for K splits.
-size_t result_bytes(long long nm, long long M, long long N)
+// Splits of a long K: the tiles that share rows through L2 drift apart along K, and beyond some 20000 elements the rows
+// are read from memory again (o=40/v=400/n=2000, 820 and 780 columns, K = 80640: 204 ms in one piece, 189 in two, 168 in
+// four, 172 in eight).
+constexpr int kMaxSplit = 8;
+inline int splits_of(long long K) { return (int)std::min<long long>(kMaxSplit, (K + 20479) / 20480); }
+
+// Bytes for the result planes of an M x N residue GEMM, either orientation, with room for its splits; small results get
+// room for more, which fill the SMs.
+size_t result_bytes(long long nm, long long M, long long N, long long K)
 {
     const size_t b = std::max(planes_bytes(nm, M, N), planes_bytes(nm, N, M));
-    return std::max(b, std::min(8 * b, (size_t)32 << 20));
+    return std::max(splits_of(K) * b, std::min(kMaxSplit * b, (size_t)32 << 20));
 }
 
 struct FwdLayout {
@@ -182,7 +189,7 @@ FwdLayout layout_packed(const Ctx& c, long long P)
     L.Vm = cv.take(es * s2 * P * pk(km));
     L.eVm = cv.take(4 * P);
     if (c.crt) {
-        L.Rw_bytes = result_bytes(c.nm2, c.PB, P);
+        L.Rw_bytes = result_bytes(c.nm2, c.PB, P, crt_kq_total((int)v));
         L.Rw = cv.take(L.Rw_bytes);
     }
     L.Rpc = cv.take(8 * c.PB * P);
@@ -217,7 +224,7 @@ FwdLayout layout_fwd(const Ctx& c, long long A)
             L.Vw = cv.take(es * s2 * (long long)A * v * pitch_of(c, kk));
             L.eV = cv.take(4 * (long long)A * v);
         }
-        if (c.crt) L.Rw_bytes = result_bytes(s2, P, A * v);
+        if (c.crt) L.Rw_bytes = result_bytes(s2, P, A * v, kk);
     } else {
         const long long kk = c.crt ? k_pad(n, v) : n * v;
         L.X2 = cv.take(c.crt ? planes_bytes(s1, A * n, P * v) : 8 * P * (long long)A * n * v);
@@ -232,7 +239,7 @@ FwdLayout layout_fwd(const Ctx& c, long long A)
             L.LwB = cv.take(es * s2 * v * pitch_of(c, kk));
             L.eLB = cv.take(4 * v);
         }
-        if (c.crt) L.Rw_bytes = result_bytes(s2, P * A, v);
+        if (c.crt) L.Rw_bytes = result_bytes(s2, P * A, v, k_pad(n, v));
     }
     if (c.crt) L.Rw = cv.take(L.Rw_bytes);
     L.total = cv.cur;
@@ -752,7 +759,8 @@ int run_crt(const char* name, const Ctx& c, int nm, int M, int N, int K, const O
 // out = sum_k A(m,k) B(n,k) in FP64 through result planes of `cap` bytes.  nm_src > 0: B's rows were made from
 // the planes of a contraction with nm_src moduli (kPlaneBits, CrtRec::frac left out).  The GEMM runs in the orientation whose
 // tiles waste less (M comes in whole 256-row tiles, N in columns of 32), and K is split where the items
-// (modulus x tile) would leave SM pairs idle; the splits' residues are summed by the conversion.
+// (modulus x tile) would leave SM pairs idle, and where it is long and several columns of tiles share rows; the splits'
+// residues are summed by the conversion.
 int run_crt_out(const char* name, const Ctx& c, int nm, int M, int N, int K, const Operand& A, const Operand& B,
                 const OutDesc& out, unsigned char* planes, size_t cap, cudaStream_t st, int nm_src)
 {
@@ -775,8 +783,9 @@ int run_crt_out(const char* name, const Ctx& c, int nm, int M, int N, int K, con
     const int pairs = std::max(1, device_sm_count() / 2);
     auto eff = [&](int S) { const double w = (double)items * S / pairs; return w / std::ceil(w); };
     int S = 1;
-    for (int t = 2; t <= 8 && K / t >= 2048 && planes_bytes((long long)nm * t, M, N) <= cap; ++t)
+    for (int t = 2; t <= kMaxSplit && K / t >= 2048 && planes_bytes((long long)nm * t, M, N) <= cap; ++t)
         if (eff(t) > eff(S) + 0.05) S = t;
+    while (N > 256 && S < splits_of(K) && planes_bytes((long long)nm * (S + 1), M, N) <= cap) ++S;
     const int kper = ((K + S - 1) / S + 63) / 64 * 64;  // the kernel's split, in whole K-steps
     g.ksplit = (K + kper - 1) / kper;
     CC_TRY(crt_gemm(name, g, st));
@@ -1352,7 +1361,7 @@ TermLayout layout_term(const TermCtx& tc, long long Pb)
         L.Vw = cv.take(es * s2 * Pb * tc.nq * pitch_of(c, kk));
         L.eV = cv.take(4 * Pb * tc.nq);
         if (c.crt) {
-            L.Rw_bytes = result_bytes(s2, o * o, Pb * tc.nq);
+            L.Rw_bytes = result_bytes(s2, o * o, Pb * tc.nq, kk);
             L.Rw = cv.take(L.Rw_bytes);
         }
     }
@@ -1520,7 +1529,7 @@ BwdLayout layout_bwd(const Ctx& c, int E, size_t fwd_bytes, bool sym)
         L.M1w = cv.take(es * s2 * (long long)E * v * pitch_of(c, kk));
         L.eM1 = cv.take(4 * (long long)E * v);
         if (c.crt) {
-            L.Rw_bytes = result_bytes(s2, n, E * v);
+            L.Rw_bytes = result_bytes(s2, n, E * v, k_pad(v, v));
             L.Rw = cv.take(L.Rw_bytes);
         }
     }
@@ -1940,7 +1949,7 @@ static size_t gemm_ws(int mode, int M, int N, int K, int s, int nm = 0, size_t* 
         cv.take((size_t)es * st * N * (nm > 0 ? pitch_crt(K) : pitch_for(K, es)));
         cv.take(4 * (size_t)N);
         if (nm > 0) {
-            const size_t rb = result_bytes(nm, M, N);
+            const size_t rb = result_bytes(nm, M, N, K);
             cv.take(rb);
             if (res) *res = rb;
         }
