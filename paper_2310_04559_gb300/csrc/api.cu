@@ -20,8 +20,11 @@
 //     R-[i< j][(a,b>=a)] = sum_{c< d} T-[ij][cd] V-[ab][cd]      (GEMM M=o(o-1)/2, K=v(v-1)/2)
 //     R[i,j,a,b] = R[j,i,b,a] = R+ + R-,  R[j,i,a,b] = R[i,j,b,a] = R+ - R-
 // which issues about (n + o^2/2) v^4 multiply-adds instead of 2 (n + o(o+1)/2) v^4.
-// In the emulated-FP64 and mixed modes every GEMM operand is first turned into
-// a slice stack (split.cu, pm.cu) and the GEMM runs on the tensor cores (gemm_tc.cu);
+// Without pair symmetry the same path runs with all o^2 rows (i, j) on both sides (emulated FP64 and FP64 modes).
+// In the emulated-FP64 mode every GEMM operand is first turned into residues modulo 12 or 13 numbers (crt.cuh,
+// crt_prep.cu) and the GEMMs run on pairs of SMs (gemm_crt.cu); other precisions than the default one, and workspaces
+// too small for that, use stacks of digit slices (split.cu, pm.cu, gemm_tc.cu).  The mixed modes' operands are
+// rounded once (split.cu, pm.cu), for the SM-pair GEMM on the packed path and gemm_tc.cu elsewhere;
 // in the FP64 mode the GEMMs run on FP64 FMAs (gemm_f64.cu) straight from FP64.
 #include <cuda_runtime.h>
 

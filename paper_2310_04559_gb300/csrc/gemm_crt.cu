@@ -18,13 +18,13 @@
 // TMEM) alternate between passes: the epilogue reduces pass p modulo p_l into registers while the MMAs of
 // pass p + 1 run, and the item's sum once more, to the byte it stores.  The reductions are packed FP32
 // (r = x - p rint(x / p), exact), 1.5 instructions per element and pass: converting to integers instead took 8000
-// clocks per tile, as long as the MMAs of K = 1000 (8192 x 8192 x 1024, 12 moduli: 1518 TFLOP/s then, 2010 now).
+// clocks per tile, as long as the MMAs of K = 1000 (8192 x 8192 x 1024, 12 moduli: 1518 TFLOP/s then, 2065 now).
 //
 // The same kernel runs the mixed modes' GEMMs (one bf16 or tf32 operand each, passes of 16384 elements in FP32, FP64
 // across passes), storing the FP32 sums or FP64: on 128 x 128 tiles of single SMs they had no operand reuse and were
-// bound by the copies (integral build of o=27/v=301/n=1501 in BF16: 37.2 ms then, 8.5 now).
+// bound by the copies (integral build of o=27/v=301/n=1501 in BF16: 37.2 ms then, 7.7 now).
 //
-// Bound: the tensor pipe, long calls its power cap (o=40/v=400/n=2000 integral blocks: 1925 TFLOP/s, against 1724 of
+// Bound: the tensor pipe, long calls its power cap (o=40/v=400/n=2000 integral blocks: 1930 TFLOP/s, against 1724 of
 // a library GEMM that runs for seconds); below K = 512 the epilogue, 2.5 us per item.
 //
 // Roles (384 threads): warp 0 issues the A copies and fetches items (leader CTA), warp 3 the B copies,
@@ -760,7 +760,12 @@ cudaError_t launch(const Sides& g, Params& p, cudaStream_t s)
     const int units = (p.N + 31) / 32;
     p.ubase = units / p.tiles_n;
     p.urem = units % p.tiles_n;
-    p.group_m = p.tiles_m < 8 ? p.tiles_m : 8;
+    // Every group of tile rows reads all of B again, from memory unless B fits in L2: 16 rows read it half as often as 8, as
+    // long as their own elements stay in L2 (integral build of o=40/v=400/n=2000 318 -> 312 ms, of o=20/v=200/n=1000 10.25
+    // -> 10.15, o=27/v=301/n=1501 in BF16 7.86 -> 7.74).  Along a long K fewer rows at once are better (ladder GEMM at v=400,
+    // K = 20160 per split: 170 ms with 8, 175 with 16).
+    const int group = p.K <= 4096 ? 16 : 8;
+    p.group_m = p.tiles_m < group ? p.tiles_m : group;
     const long long nitems = (long long)p.tiles_m * p.tiles_n * p.ksplit * p.nm;
     if (nitems > 0x7fffffffll - (1 << 20)) return cudaErrorInvalidConfiguration;
     p.nitems = (int)nitems;
