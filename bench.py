@@ -4,7 +4,7 @@ with (ac|bd) = sum_P L_Pac L_Pbd built on the fly in blocks of `a` (Eq. 5, 6).
 
 One step = one full ladder evaluation (integral blocks + ladder GEMMs + pair
 symmetry write) on the o=40, v=400, n_chol=2000 workload in emulated FP64
-(Ozaki BF16 slices on tcgen05 tensor cores), inputs resident in HBM (L 2.56 GB
+(BF16 residues on tcgen05 tensor cores), inputs resident in HBM (L 2.56 GB
 and t2 2.05 GB, both larger than the 129 MB L2).  Prints one JSON line.
 
   python bench.py [--gpus N --steps K --warmup W] [--impl reference]
@@ -37,7 +37,7 @@ WORKLOADS = {"o40_v400_n2000": (40, 400, 2000), "o20_v200_n1000": (20, 200, 1000
              "o125_v375_n2500": (125, 375, 2500)}
 METRIC = "ladder-term TFLOP/s (emulated FP64)"
 UNIT = "TFLOP/s"
-DTYPE = "f64 (emulated: bf16 Ozaki slices, exact fp32 level sums, int64/fp64 recombination)"
+DTYPE = "f64 (emulated: bf16 residues modulo coprime numbers, exact fp32 sums, exact recombination to fp64)"
 
 
 def algorithmic_flops(o, v, n):
@@ -183,16 +183,16 @@ def cpu_model() -> str:
 
 def traffic_record():
     """DRAM bytes over algorithmic bytes of the tensor-core GEMM, from the committed summary of an
-    ncu capture (profiles/gemm_tc_traffic.json), if the kernel source is unchanged since it was
+    ncu capture (profiles/gemm_crt_traffic.json), if the kernel source is unchanged since it was
     captured (else None)."""
     import hashlib
-    p = os.path.join(ROOT, "profiles", "gemm_tc_traffic.json")
+    p = os.path.join(ROOT, "profiles", "gemm_crt_traffic.json")
     if not os.path.exists(p):
         return None
     rec = json.load(open(p))
-    src = os.path.join(ROOT, "paper_2310_04559_gb300", "csrc", "gemm_tc.cu")
+    src = os.path.join(ROOT, "paper_2310_04559_gb300", "csrc", "gemm_crt.cu")
     sha = hashlib.sha256(open(src, "rb").read()).hexdigest()[:16]
-    return rec if rec.get("gemm_tc_sha") == sha else None
+    return rec if rec.get("gemm_crt_sha") == sha else None
 
 
 def timed(stream, fn, reps=1):
@@ -212,7 +212,7 @@ def timed(stream, fn, reps=1):
 def mode_peak(mode, probed, pk):
     """Peak (TFLOP/s) of the unit a mode's GEMMs run on, and where it comes from."""
     if mode == "fp64":
-        return probed.get("dmma"), "probed dmma (mma.sync.m8n8k4.f64)"
+        return probed.get("dfma"), "probed dfma (FP64 fused multiply-adds)"
     if mode == "tf32":
         return probed.get("tc_tf32"), "probed tcgen05 kind::tf32"
     return pk.get("bf16_tflops_sustained", pk["bf16_tflops"]), "MEASURED_PEAKS bf16_tflops_sustained"
@@ -276,8 +276,8 @@ def run_ours(a):
     t_max = dist_max(t_step, world, dev)
     value = flops / t_max / 1e12  # one problem, all ranks
 
-    # roofline of the dominant kernel (the tcgen05 slice GEMM): issued slice-MMA
-    # flops per launch over its average launch time, from the live events
+    # roofline of the dominant kernel (the tcgen05 residue GEMM): issued MMA flops (all moduli)
+    # per launch over its average launch time, from the live events
     tc = [k for k in prof if k.endswith("_tc")]
     tc_ms = sum(prof[k]["ms"] for k in tc)
     tc_fl = sum(prof[k]["flops"] for k in tc)
@@ -288,7 +288,7 @@ def run_ours(a):
     achieved = tc_fl / (tc_ms / 1e3) / 1e12 if tc_ms > 0 else None
     tr = traffic_record()
     alg_bytes = tc_by / max(tc_n, 1)
-    roofline = {"kernel": "gemm_tc_kernel<bf16>", "bound": "tensor", "achieved": achieved, "peak": peak,
+    roofline = {"kernel": "gemm_crt_kernel<bf16>", "bound": "tensor", "achieved": achieved, "peak": peak,
                 "unit": "TFLOP/s", "frac": (achieved / peak) if achieved else None,
                 "traffic": tr["ratio"] * alg_bytes if tr else None,
                 "algorithmic_bytes_per_launch": alg_bytes,
@@ -339,7 +339,7 @@ def run_ours(a):
     out = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": a.steps, "warmup": a.warmup,
            "ms_per_step": t_max * 1e3, "higher_is_better": True, "scaling": "strong" if world > 1 else "weak",
            "vs_baseline": None, "dtype": DTYPE,
-           "precision": "fp64 emulated (Ozaki: 6 bf16 slices x 7 bits, exact fp32 products, fp64 recombination)",
+           "precision": "fp64 emulated (42-bit rows, 12 or 13 bf16 residues, exact fp32 sums, Chinese remainder to fp64)",
            "data": "synthetic (seeded random Cholesky vectors and amplitudes, shapes of the paper's benchmarks)",
            "config": workload_config(a.workload),
            "plan": {"mode": mode, "order": plan["order"], "a_block": plan["a_block"], "n_blocks": plan["n_blocks"],
@@ -347,7 +347,7 @@ def run_ours(a):
                     "parallelism": f"a-range partition over {world} ranks" if world > 1 else "single GPU",
                     "workspace_gb": round(ws_bytes / 1e9, 2),
                     "peak_device_gb": round(torch.cuda.max_memory_allocated(dev) / 1e9, 2),
-                    "flops_algorithmic_per_step": flops, "flops_issued_per_step_this_rank": plan["flops_issued"]},
+                    "flops_algorithmic_per_step": flops, "flops_issued_per_step_this_rank": tc_fl / a.steps},
            "e2e": e2e, "roofline": roofline, "clocks": clk.summary(), "gpu_launches": launches,
            "phases_ms_per_step": {k: round(v_["ms"] / a.steps, 3) for k, v_ in sorted(prof.items())}}
 
@@ -394,10 +394,17 @@ def extras(a, out, o, v, n, mode, L_np, t2_np, Lg, tg, R, ws, E_e2e, value, dev,
     Rs, t_cpu, threads = oracle_sample(L_np, t2_np, a_list)
     rel = lambda X: float(np.linalg.norm(X[:, :, a_list, :] - Rs) / np.linalg.norm(Rs))
     full_R = R if world == 1 else None
-    plan_of = lambda m: B.plan(o, v, n, ws_bytes=ws.numel(), mode=m, symmetric=True)
 
-    def mode_entry(m, ms, Rm):
-        issued = plan_of(m)["flops_issued"]
+    def issued_flops(call):
+        """GEMM flops that one call issues, counted by the library's profile."""
+        B.profile_enable(True)
+        call()
+        torch.cuda.synchronize(dev)
+        p = B.profile_read()
+        B.profile_enable(False)
+        return sum(p[k]["flops"] for k in p if k.endswith(("_tc", "_f64")))
+
+    def mode_entry(m, ms, Rm, issued):
         peak, src = mode_peak(m, probed, pk)
         ach = issued / (ms / 1e3) / 1e12
         return {"tflops": algorithmic_flops(o, v, n) / (ms / 1e3) / 1e12, "ms": ms,
@@ -406,21 +413,24 @@ def extras(a, out, o, v, n, mode, L_np, t2_np, Lg, tg, R, ws, E_e2e, value, dev,
 
     modes = {}
     if full_R is not None:
-        modes[mode] = mode_entry(mode, out["ms_per_step"], full_R)
+        modes[mode] = mode_entry(mode, out["ms_per_step"], full_R, out["plan"]["flops_issued_per_step_this_rank"])
         modes[mode]["rel_err_columns"] = a_list
     for m in [x for x in a.other_modes.split(",") if x]:
         Rm = torch.empty_like(tg)
-        ms = timed(stream, lambda: B.ladder_forward(Lg, tg, R=Rm, mode=m, symmetric=True, workspace=ws))
-        modes[m] = mode_entry(m, ms, Rm)
+        call = lambda: B.ladder_forward(Lg, tg, R=Rm, mode=m, symmetric=True, workspace=ws)
+        ms = timed(stream, call)
+        modes[m] = mode_entry(m, ms, Rm, issued_flops(call))
         del Rm
     if a.fp64_full:
         R64 = torch.empty_like(tg)
         f0, f1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-        f0.record(stream)
-        B.ladder_forward(Lg, tg, R=R64, mode="fp64", symmetric=True, workspace=ws)
-        f1.record(stream)
-        torch.cuda.synchronize(dev)
-        modes["fp64"] = mode_entry("fp64", f0.elapsed_time(f1), R64)
+        def call64():
+            f0.record(stream)
+            B.ladder_forward(Lg, tg, R=R64, mode="fp64", symmetric=True, workspace=ws)
+            f1.record(stream)
+
+        issued64 = issued_flops(call64)
+        modes["fp64"] = mode_entry("fp64", f0.elapsed_time(f1), R64, issued64)
         modes["fp64"]["timed_on"] = "the full workload, one call"
         del R64
     out["modes"] = modes
@@ -561,7 +571,7 @@ def large_leg(a, dev, stream, mode):
             "order": tune["order"], "n_blocks": plan["n_blocks"], "peak_device_gb":
             round(torch.cuda.max_memory_allocated(dev) / 1e9, 2),
             "roofline": {"achieved": ach, "peak": peak, "frac": ach / peak if ach else None,
-                         "unit": "TFLOP/s", "flops_issued_per_step": plan["flops_issued"]},
+                         "unit": "TFLOP/s", "flops_issued_per_step": tc_fl / 3},
             "rel_err_sampled_entries": float(np.linalg.norm(got - ref) / np.linalg.norm(ref)),
             "inputs": f"drawn on the device with torch's generator, same recipe ({t_gen:.1f} s)"}
 

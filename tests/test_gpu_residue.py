@@ -150,3 +150,11 @@ def test_short_rows_of_several_segments(dev, o, v, n):
     # two roundings of rows of v, and of n v, elements to 42 bits of their largest entry
     scale = np.abs(L).max() ** 2 * np.abs(t2).max() * n * v * v
     assert np.abs(R - ref).max() <= scale * 2.0 ** -38
+
+
+@pytest.mark.parametrize("M,N,K", [(300, 257, 20480), (260, 300, 20481), (300, 513, 41000), (257, 300, 61441)])
+def test_long_k_is_split(dev, M, N, K):
+    """More than 256 columns and more than 20480 elements: partial residues of uneven splits, summed by the conversion."""
+    rng = np.random.default_rng(K)
+    A, Bm = rng.integers(-400, 400, (M, K)).astype(np.float64), rng.integers(-400, 400, (N, K)).astype(np.float64)
+    assert np.array_equal(B.gemm(cu(A, dev), cu(Bm, dev)).cpu().numpy(), A @ Bm.T)
