@@ -287,7 +287,7 @@ void cc_ladder_set_wait_limit_ns(unsigned long long ns);
 
 /* Building block used by every contraction above, exposed for direct use and testing:
  *   C[m*ldc + n] (= or +=) sum_k A[m*lda + k] * B[n*ldb + k]     (row-major, K-contiguous FP64)
- * in the arithmetic of `mode` (CC_FP64: FP64 FMAs; CC_OZAKI_BF16: split BF16 slices on tcgen05 with
+ * in the arithmetic of `mode` (CC_FP64: FP64 FMAs; CC_OZAKI_BF16: BF16 residues or slices on tcgen05 with
  * FP64 recombination; CC_TF32 / CC_BF16: one rounded copy, FP32 accumulation per K-chunk).
  * accumulate != 0 adds into C.  Workspace from cc_ladder_gemm_workspace_size.
  * CC_OZAKI_BF16 is exact in its FP32 sums for any K and any input (see cc_precision). */
@@ -308,7 +308,7 @@ typedef struct cc_ladder_profile_entry {
     int launches;
     double ms;
     double flops;
-    double bytes;   /* algorithmic DRAM bytes of the slice GEMMs: every operand slice read once and
+    double bytes;   /* algorithmic DRAM bytes of the tensor-core GEMMs: every operand stack read once and
                        the output written once (read too when accumulated); 0 for other phases */
 } cc_ladder_profile_entry;
 void cc_ladder_profile_enable(int on);

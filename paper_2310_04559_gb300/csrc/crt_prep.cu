@@ -270,6 +270,7 @@ struct RowsArg {
     int outer, inner;
 };
 
+// Bound: HBM and the residues' arithmetic (96 rows of 46080: 37 us, 30% of HBM, 49% of the multipliers).
 __global__ void __launch_bounds__(NT) crt_rows_kernel(const RowsArg a, int nm, unsigned short* __restrict__ D,
                                                       long long pitch, int* __restrict__ e_out, int* __restrict__ status)
 {
@@ -365,6 +366,7 @@ __device__ __forceinline__ long long col_off(const ColSrc& s, long long r)
 
 constexpr int CR = 32, CK = 64;  // transpose tile: 32 rows x 64 k
 
+// Bound: the transposition's latency and HBM (o=8/v=160/n=800: 0.16 GB read twice, 0.49 GB written, 218 us, 42% of HBM).
 // PREMAX: mx holds every row's largest |x| (over a K range longer than this call's); else it is found first, over the
 // whole K by the cluster's CTAs, each taking every cs-th tile of k in both walks.
 template <bool PREMAX>
@@ -479,6 +481,7 @@ struct QuadPos {
     }
 };
 
+// One pass over HBM: the second walk reads L2.  A small share everywhere (o=16/v=160: 82 us of 28 ms).
 // T+ and T- of the pairs i <= j (or of all pairs, each with both rows): row p of D+ holds t_cd + t_dc (the diagonal t_cc), row p - (i + 1) - s0 of D-
 // (pairs i < j) holds t_cd - t_dc; each with its own row exponent.
 struct PmRows {
@@ -564,6 +567,10 @@ __global__ void __launch_bounds__(NT) crt_pm_f64_kernel(const PmRows a, int nm, 
 // V+ and V- of the integral rows (a, b >= a) of one block from the byte planes of the integral GEMM,
 // planes[l][(al, c)][(b', d)], each element's fraction y scaled by 2^(eA[al v + c] + eB[b' v + d]) (the factor CrtRec::frac is left to the result).  Both halves share the row exponent E of the largest |V|,
 // as Y = round(V 2^(43 - E)) (one guard bit), V+- = (Y1 +- Y2) / 4.
+// Bound: arithmetic and HBM together (o=16/v=160/n=800: alu 50%, FP32/integer multiply 57%, issue 61%, HBM 53% of
+// their peaks, 10 ps per element): twelve 96-bit products to put an element together, 13 residues to take it apart, 12 bytes
+// read and 26 written.  The row's second walk finds it in L2 (2.7 GB read for 4.1 GB of planes).  o=40/v=400/n=2000: 342 ms
+// with one CTA per row, 205 with 4 x 4 blocks in registers, 171 with entries in the order of c and d, 157 now.
 struct PmPlanes {
     const unsigned char* planes;
     long long plane, pitch_in;  // bytes between planes, per GEMM row
@@ -718,6 +725,8 @@ __global__ void __launch_bounds__(NT, 4) crt_pm_planes_kernel(const PmPlanes a, 
 // ------------------------------------------- plain rows from the planes of an intermediate
 // Row r = (al, q), K = (o, i): the fractions of planes[l][(al outer + o)][q inner + i], scaled by
 // 2^(eA[al outer + o] + eB[q inner + i]) (the factor CrtRec::frac is left to the result).
+// Bound as crt_pm_planes: 9.3 ps per element (o=16/v=160/n=800, M1 of the adjoint: 4.1 TB/s); five CTAs per SM (10.0 ms for
+// all splits of that adjoint with four, 10.7 with five) or clusters twice as wide (11.6) are slower.
 struct PlaneRows {
     const unsigned char* planes;
     long long plane, pitch_in;
@@ -814,6 +823,7 @@ __device__ __forceinline__ double pow2(int e)
     return __longlong_as_double((long long)(e + 1023) << 52);
 }
 
+// Bound: HBM and L2, nm bytes read per split and 8 written (o=40/v=400/n=2000, four splits: 3.4 ms of 650).
 // C[rmap(m) + cmap(n)] (= or +=) x(m, n) * 2^(eA[m] + eB[n] + base) * factor, x from the planes summed over the K splits.
 // MFAST: m is the output's contiguous index (the GEMM ran on the transposed problem).
 template <bool MFAST>

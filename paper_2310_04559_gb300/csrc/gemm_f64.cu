@@ -14,6 +14,8 @@
 //   - a CTA's four warps take 32 rows, or split K between them where there are no more than 16 or 8 rows;
 //   - NT and a split of K over a cluster of up to eight CTAs are chosen so that the CTAs fill whole
 //     waves of the device; partial sums meet in distributed shared memory and are added in a fixed order.
+// Against 64 x 64 tiles on mma.m8n8k4.f64: o=4/v=24/n=60 976 -> 157 us, o=10/v=100/n=500 62.1 -> 47.6 ms (1.21 TFLOP/s of the
+// 1.25 that the FMA units reach), 55 x 5050 x 5050 6.6 -> 2.7 ms.
 #include <algorithm>
 #include <cmath>
 
