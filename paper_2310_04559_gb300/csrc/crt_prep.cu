@@ -22,6 +22,7 @@ namespace cc {
 namespace {
 
 constexpr int NT = 256;  // threads per CTA
+constexpr size_t kMaxSmem = 227 * 1024;  // shared memory of one CTA at most
 constexpr unsigned long long kAbs = 0x7fffffffffffffffull;
 constexpr unsigned long long kInf = 0x7ff0000000000000ull;
 
@@ -587,7 +588,7 @@ __global__ void __launch_bounds__(NT, 4) crt_pm_planes_kernel(const PmPlanes a, 
                                                            unsigned short* __restrict__ Dm, int* __restrict__ em,
                                                            long long rows, long long pitch)
 {
-    extern __shared__ int esm[];  // exponents of c and of d, then their codes (each padded to a multiple of four)
+    extern __shared__ __align__(16) int esm[];  // exponents of c and of d, then their codes (each padded to a multiple of four)
     __shared__ long long S[2][2][TT][TT + 1];  // two buffers: one barrier per tile pair
     __shared__ long long red[NT / 32 + 1];
     const uint32_t cs = cluster_size(), rank = cluster_rank();
@@ -902,9 +903,16 @@ template <typename... KArgs, typename... Args>
 cudaError_t launch_rows(void (*kern)(KArgs...), long long rows, int cs, size_t smem, cudaStream_t st, Args... args)
 {
     if (rows * cs > 0x7fffffffll) return cudaErrorInvalidConfiguration;
-    if (smem > 30 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (smem > 0) {
+        // (a launch gets 48 KB unasked, static and dynamic together; the kernel's static part is the compiler's to say)
+        cudaFuncAttributes fa{};
+        cudaError_t e = cudaFuncGetAttributes(&fa, kern);
         if (e != cudaSuccess) return e;
+        if (fa.sharedSizeBytes + smem > kMaxSmem) return cudaErrorInvalidValue;
+        if (fa.sharedSizeBytes + smem > 48 * 1024) {
+            e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return e;
+        }
     }
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)(rows * cs));
@@ -969,8 +977,7 @@ cudaError_t crt_pm_planes(const CrtPlanes& src, bool all_b, long long rows, int 
                           const int* eB, int diag, int nm, void* Dp, int* ep, void* Dm, int* em, long long pitch, cudaStream_t st)
 {
     if (rows <= 0) return cudaSuccess;
-    const size_t smem = sizeof(int) * 4 * (size_t)((v + 3) & ~3);  // v up to about 12800
-    if (smem > 200 * 1024) return cudaErrorInvalidValue;
+    const size_t smem = sizeof(int) * 4 * (size_t)((v + 3) & ~3);  // v up to about 12400 (one `a` of such a block is 20 TB)
     const PmPlanes a{src.planes, src.plane, src.pitch, all_b ? 1 : 0, Nb, v, eA, eB, diag};
     const CrtRec rec = crt_rec(src.nm);
     const long long elems = (long long)v * v;

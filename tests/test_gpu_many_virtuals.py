@@ -1,0 +1,43 @@
+"""Many virtual orbitals in the emulated-FP64 mode: the integral rows' split keeps the exponents of a row's c and d in
+dynamic shared memory beside its tiles, so from v = 953 on the two together pass the 48 KB that a launch gets unasked.
+
+Bound: operand rows carry 42 bits, intermediate rows at least 42 bits of the largest entry, so an entry of R is off by at
+most n v^2 max|L|^2 max|t2| 2^-38 (both roundings and the FP64 conversion)."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2310_04559_gb300 import binding as B
+from paper_2310_04559_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def dev():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    return torch.device("cuda", 0)
+
+
+# the last size whose shared memory stays within 48 KB, the first beyond, one no multiple of four, a larger one
+@pytest.mark.parametrize("v", [952, 956, 957, 1000])
+@pytest.mark.parametrize("sym", [True, False])
+def test_range_of_a(dev, v, sym):
+    o, n, a = 2, 3, (v - 2, v - 1)
+    L, t2 = synth.ladder_inputs_torch(o, v, n, seed=v, device="cuda")
+    if not sym:
+        t2 = torch.randn(t2.shape, dtype=torch.float64, device=dev, generator=torch.Generator(device=dev).manual_seed(v))
+    R = torch.zeros_like(t2)
+    B.ladder_forward(L, t2, R=R, symmetric=sym, order="integral_first", a_range=a, budget=48 << 30)
+    # R[i,j,a,b] = sum_P (L_P[a,:] t_ij) . L_P[b,:]
+    X = torch.einsum("Pc,ijcd->Pijd", L[:, a[0]], t2)
+    ref = torch.einsum("Pijd,Pbd->ijb", X, L)
+    got = R[:, :, a[0]]
+    if sym:  # written for b >= a only
+        got, ref = got[:, :, a[0]:], ref[:, :, a[0]:]
+    bound = n * v * v * float(L.abs().max()) ** 2 * float(t2.abs().max()) * 2.0 ** -38
+    assert float((got - ref).abs().max()) <= bound
+    assert float(ref.abs().max()) > 0 and np.isfinite(bound)
+    # and close in the norm, far below that worst case
+    assert float((got - ref).norm() / ref.norm()) < 1e-10
