@@ -499,7 +499,13 @@ int make_ctx(const cc_ladder_args* a, Ctx* c, bool tuning = false)
 
 bool aligned(const void* p, size_t al) { return ((uintptr_t)p % al) == 0; }
 
-int check_cuda(cudaError_t e) { return e == cudaSuccess ? CC_OK : CC_ERR_CUDA; }
+// (a refused runtime call or launch is reported here and taken off the thread's record, where the next call would find it)
+int check_cuda(cudaError_t e)
+{
+    if (e == cudaSuccess) return CC_OK;
+    cudaGetLastError();
+    return CC_ERR_CUDA;
+}
 
 int run_f64(const char* name, const GemmF64& g, cudaStream_t st, double elems = -1.0)
 {
