@@ -818,10 +818,14 @@ __global__ void __launch_bounds__(NT, 4) crt_rows_planes_kernel(const PlaneRows 
 }
 
 // ------------------------------------------------------------------- results
-__device__ __forceinline__ double pow2(int e)
+// r * 2^e, rounded once, over the whole range of doubles: the exponent goes into r's own, and what leaves the normal
+// numbers goes through scalbn.  (As x * 2^e * factor the first product passed 2^1024 for results from 2^972 on, their factor
+// being about 2^-51.)
+__device__ __forceinline__ double times_pow2(double r, int e)
 {
-    e = e < -1022 ? -1022 : (e > 1023 ? 1023 : e);
-    return __longlong_as_double((long long)(e + 1023) << 52);
+    const int ex = (__double2hiint(r) >> 20) & 0x7ff, to = ex + e;
+    if (ex != 0 && to > 0 && to < 0x7ff) return __hiloint2double(__double2hiint(r) + (e << 20), __double2loint(r));
+    return scalbn(r, e);
 }
 
 // Bound: HBM and L2, nm bytes read per split and 8 written (o=40/v=400/n=2000, four splits: 3.4 ms of 650).
@@ -864,7 +868,7 @@ __global__ void __launch_bounds__(NT) crt_to_f64_kernel(int M, int N, const unsi
         for (int j = 0; j < 4; ++j) {
             const int n = n0 + qx + j;
             if (n >= N) continue;
-            const double x = (double)crt_scale(a[j].fraction(), rec) * pow2(em + eB[n]) * factor;
+            const double x = times_pow2((double)crt_scale(a[j].fraction(), rec) * factor, em + eB[n]);
             if (MFAST) {
                 S[qy][qx + j] = x;
             } else {
