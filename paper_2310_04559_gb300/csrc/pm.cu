@@ -30,6 +30,7 @@
 // in shared memory, so that X[c][d] and X[d][c] are both read coalesced.
 #include <cuda_bf16.h>
 
+#include <cfloat>
 #include <climits>
 #include <type_traits>
 
@@ -300,19 +301,9 @@ __global__ void pm_fixed_kernel(const PmFixedSrc src, int s, int beta, __nv_bflo
     }
 }
 
-// s = x1 + x2 in FP32, to be rounded on to bf16: only where s sits exactly between two bf16 numbers does the part that
-// s left out decide, and there the sum is moved by one unit towards it (about one sum in 65536).
-__device__ __forceinline__ float sum_for_bf16(float x1, float x2)
-{
-    const float s = __fadd_rn(x1, x2);
-    uint32_t b = __float_as_uint(s);
-    if ((b & 0xffffu) == 0x8000u) {
-        const float t = __fsub_rn(s, x1);
-        const float err = __fadd_rn(__fsub_rn(x1, __fsub_rn(s, t)), __fsub_rn(x2, t));  // x1 + x2 = s + err
-        if (err != 0.0f) b += ((__float_as_uint(err) ^ b) >> 31) ? 0xffffffffu : 1u;
-    }
-    return __uint_as_float(b);
-}
+// Whether a bf16 rounding of h may differ from that of the number h stands for: h is next to, or exactly, the middle of two
+// bf16 numbers (about one number in 22000).
+__device__ __forceinline__ bool near_bf16_tie(float h) { return ((__float_as_uint(h) - 0x7fffu) & 0xffffu) <= 2u; }
 
 // Integral block of the mixed modes in FP32 (the integral GEMM's own sums): V+ and V- of one row in one walk over its
 // tile pairs, 4 bytes read and 2 (4) written per element.  Bound: HBM.  A row's tile pairs are shared by `share` CTAs,
@@ -374,7 +365,17 @@ __global__ void __launch_bounds__(TT * TY) pm_f32_kernel(const float* __restrict
         }
         td += share;
         settle();
-        __syncthreads();
+        // tf32: sums of numbers from 2^126 on may leave FP32's range before they are halved.  A tile pair that holds such a
+        // number goes through FP64 as a whole (a test per element cost 1% of o=20/v=200/n=1000 in TF32).
+        bool huge = false;
+        if (BF16) {
+            __syncthreads();
+        } else {
+            float top = 0.0f;
+#pragma unroll
+            for (int u = 0; u < TT / TY; ++u) top = fmaxf(top, fmaxf(fabsf(q1[u]), fabsf(q2[u])));
+            huge = __syncthreads_or(top >= 0.25f * FLT_MAX);
+        }
         auto put = [&](int y, bool diag) {
             const int c = c0 + y, d = d0 + tx;
             const float x1 = S1[y][tx], x2 = S2[tx][y];
@@ -382,14 +383,15 @@ __global__ void __launch_bounds__(TT * TY) pm_f32_kernel(const float* __restrict
             const uint32_t kp = (uint32_t)c * (uint32_t)v - (uint32_t)c * (uint32_t)(c - 1) / 2 - (uint32_t)c + (uint32_t)d;
             const uint32_t km = kp - (uint32_t)c - 1;
             if (BF16) {
-                // (2 x1 for the diagonal: the halves are exact)
-                float sp = __fadd_rn(x1, x2), sm = __fsub_rn(x1, x2);
-                if (((__float_as_uint(sp) & 0xffffu) == 0x8000u) | ((__float_as_uint(sm) & 0xffffu) == 0x8000u)) {
-                    sp = sum_for_bf16(x1, x2);
-                    sm = sum_for_bf16(x1, -x2);
+                // A sum of halves: within a unit of FP32 of V+- (a half may lose a bit among the denormals), so only next to
+                // a tie is the rounding to bf16 left to FP64.
+                const float h1 = 0.5f * x1, h2 = 0.5f * x2;
+                const float vp = diag && c == d ? x1 : __fadd_rn(h1, h2), vm = __fsub_rn(h1, h2);
+                __nv_bfloat162 h = __floats2bfloat162_rn(vp, vm);
+                if (near_bf16_tie(vp) | near_bf16_tie(vm)) {
+                    const double y1 = x1, y2 = x2;
+                    h = __nv_bfloat162(__double2bfloat16(diag && c == d ? y1 : 0.5 * (y1 + y2)), __double2bfloat16(0.5 * (y1 - y2)));
                 }
-                if (diag && c == d) sp = x1 + x1;
-                const __nv_bfloat162 h = __floats2bfloat162_rn(0.5f * sp, 0.5f * sm);
                 const uint32_t w = *reinterpret_cast<const uint32_t*>(&h);
                 P[kp] = (out_t)(w & 0xffffu);
                 if (M && !(diag && c == d)) M[km] = (out_t)(w >> 16);
@@ -399,7 +401,15 @@ __global__ void __launch_bounds__(TT * TY) pm_f32_kernel(const float* __restrict
                 if (M && !(diag && c == d)) M[km] = (out_t)tf32_round(0.5f * __fsub_rn(x1, x2));
             }
         };
-        if (c0 < d0 && d0 + TT <= v) {
+        if (!BF16 && huge) {
+            for (int y = ty; y < TT; y += TY) {
+                const int c = c0 + y, d = d0 + tx;
+                if (c >= v || d >= v || d < c) continue;
+                const double x1 = S1[y][tx], x2 = S2[tx][y];
+                P[kp_of(c, d, v)] = (out_t)tf32_of(c == d ? x1 : 0.5 * (x1 + x2));
+                if (M && d > c) M[km_of(c, d, v)] = (out_t)tf32_of(0.5 * (x1 - x2));
+            }
+        } else if (c0 < d0 && d0 + TT <= v) {
 #pragma unroll
             for (int u = 0; u < TT / TY; ++u) put(ty + u * TY, false);
         } else {

@@ -51,3 +51,38 @@ def test_emulated_results_scale_with_the_inputs(dev, order, sym, top):
         assert np.isfinite(ref).all()
         tiny = 2.0 ** -1073 if top < 0 else 0.0
         assert np.all(np.abs(g - ref) <= tiny), (name, np.abs(g - ref).max())
+
+
+@pytest.mark.parametrize("mode,u", [("bf16", 2.0 ** -8), ("tf32", 2.0 ** -11)])
+def test_mixed_integrals_above_half_of_the_largest_float(dev, mode, u):
+    """Integrals of 1.9e38 to 3.2e38, whose sums pass FP32's range and whose half sums V+ do not.  Bound as in
+    test_gpu_mixed: L rounded twice per product, V+- and T+- once each."""
+    o, v, n = 2, 35, 1
+    rng = np.random.default_rng(8)
+    L = rng.uniform(1.0, 1.29, (n, v, v))
+    L = 0.5 * (L + L.transpose(0, 2, 1)) * np.sqrt(1.9e38)
+    t2 = np.zeros((o, o, v, v))
+    for i in range(o):
+        for j in range(i, o):
+            for c, d in ((0, 34), (7, 7), (3, 20)):
+                t2[i, j, c, d] = t2[j, i, d, c] = 1e-3 * rng.uniform(0.5, 2.0)
+    V = np.einsum("nac,nbd->abcd", L, L)
+    assert 3.4e38 < 2 * V.min() and V.max() < 3.25e38
+    ref = np.einsum("abcd,ijcd->ijab", V, t2)
+    bound = 4.1 * u * np.einsum("abcd,ijcd->ijab", V + V.transpose(0, 1, 3, 2), np.abs(t2))
+    R = B.ladder_forward(torch.from_numpy(L).to(dev), torch.from_numpy(t2).to(dev), mode=mode, symmetric=True,
+                         order="integral_first").cpu().numpy()
+    assert np.all(np.abs(R - ref) <= bound)
+
+
+@pytest.mark.parametrize("mode", ["bf16", "tf32"])
+@pytest.mark.parametrize("e", [0, -50, -62, -66, -70])
+def test_mixed_denormal_integrals_round_once(dev, mode, e):
+    """Streamed L keeps its integral block in FP64, where V+- are exact before their one rounding: the FP32 block of
+    resident L gives the same bits, also where the integrals (about 2^(2 e)) are denormal in FP32."""
+    o, v, n = 2, 97, 4
+    L, t2 = synth.ladder_inputs_torch(o, v, n, seed=12, device="cpu")
+    L, t2 = L * 2.0 ** e, t2 * 2.0 ** 20
+    R = B.ladder_forward(L.to(dev), t2.to(dev), mode=mode, symmetric=True, order="integral_first")
+    S = B.ladder_forward(L.pin_memory(), t2.to(dev), mode=mode, symmetric=True, host_L=True, chol_chunk=n)
+    assert torch.equal(R, S), float((R - S).abs().max() / S.abs().max())
