@@ -369,7 +369,8 @@ void set_gen(Ctx* c, bool on)
 
 // The residue form needs up to about twice the slices' memory (bf16 residues for 12 or 13 moduli instead of 6
 // digits): where it does not fit -- or, with host-resident amplitudes, would not hold all pairs at once next to
-// blocks of 4 `a` values, so that t2 would be split again for every block -- the digit slices run as before.
+// blocks of 4 `a` values, so that t2 would be split again for every block, or would read a streamed L too often -- the
+// digit slices run as before.
 long long pick_block(Ctx& c, size_t bytes, int requested, size_t* need)
 {
     if (c.gen) {
@@ -381,8 +382,22 @@ long long pick_block(Ctx& c, size_t bytes, int requested, size_t* need)
         Ctx t = c;
         const long long P = pick_block_form(t, bytes, requested, need);
         const bool whole = !(t.host && t.packed) || (t.PB == t.pp && P >= (long long)std::min(t.v, 4) * t.v);
-        if (P >= 0 && whole) { c = t; return P; }
         c.crt = false;
+        if (P >= 0 && whole) {
+            // Streamed L comes over the host link and is split again for every block, so blocks that are too much smaller
+            // than those of the digit slices cost more than the residues save: 2.3 to 3 times as many blocks run in
+            // 0.69 to 0.94 of the slices' time (o=20/v=160/n=800 at 0.8 GiB 41 against 60 ms, o=6/v=200/n=1200 at 1 GiB 158
+            // against 177, o=10/v=100/n=500 at 0.15 GiB 14.6 against 15.5), 3.3 to 4.1 times as many in 1.09 to 1.2 of it
+            // (o=10/v=100/n=500 at 0.1 GiB 25.6 against 23.0, o=20/v=160/n=800 at 0.4 GiB 118 against 108, o=40/v=400/n=2000
+            // at 8 GiB 2750 to 2910 against 2400).
+            Ctx d = c;
+            size_t nd = 0;
+            const long long Pd = t.hostL ? pick_block_form(d, bytes, requested, &nd) : -1;
+            if (Pd < 0 || block_list(t, P, 0, t.v, requested).size() <= 3 * block_list(d, Pd, 0, d.v, requested).size()) {
+                c = t;
+                return P;
+            }
+        }
     }
     return pick_block_form(c, bytes, requested, need);
 }
