@@ -25,7 +25,10 @@
  *  - The library never allocates device memory.  Scratch comes from the
  *    caller's `workspace` (256-byte aligned); query its size first.  The
  *    planner sizes the block of `a` values so that the workspace fits the
- *    caller's budget.
+ *    caller's budget.  Of page-locked host memory it holds 8 bytes per host
+ *    thread that makes synchronising calls, where the status word arrives
+ *    (cudaHostAlloc in the thread's first such call, cudaFreeHost when the
+ *    thread ends; without them the word is copied on its own).
  *  - Work is enqueued on `stream` (a cudaStream_t; NULL = legacy default
  *    stream).  Unless CC_FLAG_NO_STATUS_SYNC is given, the call synchronises
  *    the stream once at the end to read the device status word, so the
@@ -155,8 +158,9 @@ typedef struct cc_ladder_args {
                               devices (each R zeroed first) assemble R by a sum
                               (cc_ladder_partition balances the ranges' work).                   */
     int chol_chunk;        /* CC_FLAG_HOST_L: Cholesky vectors per streamed chunk of L (0 = planner's
-                              choice: two chunks and their slices in about an eighth of the budget,
-                              halved until the plan fits); ignored otherwise                       */
+                              choice: two chunks and their digit slices in about an eighth of the
+                              budget, or their residues in about a fifth, halved until the plan
+                              fits); ignored otherwise                                             */
 } cc_ladder_args;
 
 /* What the planner decided for a call (for reporting and tests). */

@@ -340,7 +340,10 @@ long long pick_block_pb(const Ctx& c, size_t bytes, int requested, size_t* need)
 long long pick_block_host(Ctx& c, size_t bytes, int requested, size_t* need);
 
 // Streamed L: the chunk of Cholesky vectors starts at the caller's chol_chunk or at the one whose
-// two FP64 buffers and slices take an eighth of the budget, and halves until a plan fits.
+// two FP64 buffers and six digit slices take an eighth of the budget, and halves until a plan fits.  The residue form
+// takes the same chunk, with 12 or 13 residues (about 1.5 eighths of the budget): chunks that keep to the eighth are
+// shorter and add to the residue planes more often, which costs more than the larger blocks save (o=20/v=160/n=800 at
+// 0.8 GiB 69 ms against 41, o=6/v=200/n=1200 at 1 GiB 237 against 158, o=40/v=400/n=2000 at 20 GiB 1225 against 1070).
 long long pick_block_form(Ctx& c, size_t bytes, int requested, size_t* need)
 {
     if (!c.hostL) return pick_block_host(c, bytes, requested, need);
