@@ -495,7 +495,11 @@ int make_ctx(const cc_ladder_args* a, Ctx* c, bool tuning = false)
     // without pair symmetry: FP64 and the residue form (the mixed modes' results would round differently)
     set_crt(c, a->n_chol, vv);
     const bool whole = a->a_hi == 0 || (a->a_lo == 0 && a->a_hi == a->v);
-    const bool can_gen = !c->sym && !hostflags && (a->mode == CC_FP64 ? whole || tuning : c->crt);
+    // Not with far more occupied than virtual orbitals: the o^2 rows of T+- are then most of the work, in kernels that give
+    // a row to a CTA (o=128/v=16/n=336: 423 us packed, 179 unpacked, 290 with the digit slices; o=128/v=48/n=496 2033, 1821,
+    // 3479; FP64 o=300/v=8/n=640 1183, 752; o=64/v=12/n=188 230, 255).
+    const bool few_virtuals = a->o > 2 * a->v && a->v <= (a->mode == CC_FP64 ? 8 : 48);
+    const bool can_gen = !c->sym && !hostflags && !few_virtuals && (a->mode == CC_FP64 ? whole || tuning : c->crt);
     c->part = can_gen && !whole && !tuning;
     if (can_gen) set_gen(c, true);
     // host-resident amplitudes and streamed L run through the integral-first order only

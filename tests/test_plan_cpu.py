@@ -20,3 +20,12 @@ def test_streamed_L_is_not_read_far_more_often_than_digit_slices_would(o, v, n, 
     default = _plan(o, v, n, gib * GIB, host_L=True)
     digits = _plan(o, v, n, gib * GIB, host_L=True, slices=7)
     assert default["n_blocks"] <= 3 * digits["n_blocks"]
+
+
+# Amplitudes without pair symmetry: packed, a call issues little more than half of 2 (o^2 + n) v^4 per product, else all of it.
+@pytest.mark.parametrize("mode,o,v,n", [("ozaki_bf16", 128, 16, 336), ("ozaki_bf16", 300, 8, 20), ("ozaki_bf16", 128, 48, 200),
+                                        ("fp64", 300, 8, 20), ("fp64", 64, 4, 40)])
+def test_far_more_occupied_than_virtual_orbitals_run_unpacked(mode, o, v, n):
+    p = _plan(o, v, n, 64 * GIB, mode=mode, symmetric=False)
+    products = 1 if mode == "fp64" else 12  # at least 12 residues
+    assert p["flops_issued"] >= products * p["flops_algorithmic"]
