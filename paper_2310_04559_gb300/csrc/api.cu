@@ -1120,7 +1120,7 @@ int fwd_packed(const Ctx& c, const cc_ladder_args* a, const double* Lsrc, const 
             }
             ProfScope ps("scatter", st);
             if (c.part) CC_CU(pm_combine_rows(c.pp, c.v, a0, nr, Rpc, mb ? Rmc : nullptr, a->R, accum, st));
-            else if (c.gen) CC_CU(pm_combine_general(c.pp, c.v, a0, Ab, Nb, nr, Rpc, mb ? Rmc : nullptr, a->R, accum, st));
+            else if (c.gen) CC_CU(pm_combine_general(c.pp, c.v, a0, Ab, Nb, nr, Rpc, mb ? Rmc : nullptr, a->R, accum, f64 ? V : nullptr, t2, st));
             else CC_CU(pm_combine(c.o, c.v, a0, Ab, Nb, nr, q0, q1, s0, Rpc, mb ? Rmc : nullptr, a->R, accum, st));
         }
     }

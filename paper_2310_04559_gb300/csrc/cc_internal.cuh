@@ -169,9 +169,11 @@ cudaError_t fill_rtab(int Ab, int Nb, long long* rtab, cudaStream_t st);
 cudaError_t pm_combine(int o, int v, int a0, int Ab, int Nb, long long nr, long long q0, long long q1, long long s0,
                        const double* Rp, const double* Rm, double* R, int accumulate, cudaStream_t st);
 // R[p, a, b] (=|+=) R+ + R-, R[p, b, a] (=|+=) R+ - R- for the block a = a0 + al, b = a0 + b' >= a and the
-// `pairs` rows p = i o + j of Rp and Rm (amplitudes without pair symmetry).
+// `pairs` rows p = i o + j of Rp and Rm (amplitudes without pair symmetry).  V (nullable): the block's integrals
+// V[al][b'][c][d], T: the amplitudes, for entries that are not finite.
 cudaError_t pm_combine_general(long long pairs, int v, int a0, int Ab, int Nb, long long nr, const double* Rp,
-                               const double* Rm, double* R, int accumulate, cudaStream_t st);
+                               const double* Rm, double* R, int accumulate, const double* V, const double* T,
+                               cudaStream_t st);
 // R[p, a, b] (=|+=) R+ + R- (b >= a), R+ - R- (b < a) for the rows r = al v + b, a = a0 + al, of Rp and Rm.
 cudaError_t pm_combine_rows(long long pairs, int v, int a0, long long nr, const double* Rp, const double* Rm, double* R,
                             int accumulate, cudaStream_t st);

@@ -448,10 +448,24 @@ __device__ __forceinline__ void pair_ij(int o, int p, int& i, int& j)
 // A 32 x 32 tile (al, b') is written as it is and, through shared memory, transposed, so that both halves of R are
 // written along the last index (entry by entry, the transposed half took host-resident R 4.3 ms of 19 at o=30, v=150,
 // 8 bytes per write over the host link).
+//
+// Not finite: R+ and R- can overflow, or be two infinities of which one sum is NaN, where the plain product is neither
+// (an infinite amplitude, or t_cd + t_dc beyond 2^1024).  With V (GEN in FP64) such entries are the plain product of the
+// block's integrals and the amplitudes, by the entry's whole warp; it costs nothing elsewhere.
+__device__ __forceinline__ double plain_product(const double* __restrict__ V, const double* __restrict__ T, int v, bool swap, int lane)
+{
+    double s = 0.0;
+    for (int c = 0; c < v; ++c)
+        for (int d = lane; d < v; d += 32) s = fma(V[swap ? (long long)d * v + c : (long long)c * v + d], T[(long long)c * v + d], s);
+    for (int w = 16; w > 0; w >>= 1) s += __shfl_xor_sync(0xffffffffu, s, w);
+    return s;
+}
+
 template <bool GEN>
 __global__ void pm_combine_kernel(int o, int v, int a0, int Ab, int Nb, long long nr, long long np, long long q0,
                                   long long s0, const double* __restrict__ Rp, const double* __restrict__ Rm,
-                                  double* __restrict__ R, int accumulate)
+                                  double* __restrict__ R, int accumulate, const double* __restrict__ V,
+                                  const double* __restrict__ T)
 {
     __shared__ double E1[TT][TT + 1], E2[TT][TT + 1];
     const long long pl = (long long)blockIdx.y + (long long)blockIdx.z * gridDim.y;
@@ -472,11 +486,20 @@ __global__ void pm_combine_kernel(int o, int v, int a0, int Ab, int Nb, long lon
 #pragma unroll
     for (int y = ty; y < TT; y += TY) {
         const int al = ta + y, bq = tb + tx;
-        if (al >= Ab || bq >= Nb || bq < al) continue;
+        const bool in = al < Ab && bq < Nb && bq >= al;
         const long long r = (long long)al * Nb - (long long)al * (al - 1) / 2 + (bq - al);
-        const double plus = rp[r];
-        const double minus = (rm && bq != al) ? rm[r] : 0.0;
-        const double e1 = plus + minus, e2 = plus - minus;
+        const double plus = in ? rp[r] : 0.0;
+        const double minus = (in && rm && bq != al) ? rm[r] : 0.0;
+        double e1 = plus + minus, e2 = plus - minus;
+        if (GEN && V) {
+            for (unsigned bad = __ballot_sync(0xffffffffu, in && !(isfinite(e1) && isfinite(e2))); bad; bad &= bad - 1) {
+                const int q = __ffs(bad) - 1;
+                const double* row = V + ((long long)al * Nb + tb + q) * vv;
+                const double x1 = plain_product(row, T + pl * vv, v, false, tx), x2 = plain_product(row, T + pl * vv, v, true, tx);
+                if (tx == q) { e1 = x1; e2 = x2; }
+            }
+        }
+        if (!in) continue;
         E1[y][tx] = e1;
         E2[y][tx] = e2;
         const long long ab = (long long)(a0 + al) * v + a0 + bq;
@@ -596,17 +619,19 @@ cudaError_t pm_combine(int o, int v, int a0, int Ab, int Nb, long long nr, long 
     const long long np = q1 - q0;
     if (Ab <= 0 || np <= 0) return cudaSuccess;
     if (Ab > 65535 || np > 0x7fffffffll || q0 < 0 || q1 > (long long)o * (o + 1) / 2) return cudaErrorInvalidValue;
-    pm_combine_kernel<false><<<combine_grid(Ab, Nb, np), TT * TY, 0, st>>>(o, v, a0, Ab, Nb, nr, np, q0, s0, Rp, Rm, R, accumulate);
+    pm_combine_kernel<false><<<combine_grid(Ab, Nb, np), TT * TY, 0, st>>>(o, v, a0, Ab, Nb, nr, np, q0, s0, Rp, Rm, R, accumulate,
+                                                                          nullptr, nullptr);
     count_launch();
     return cudaGetLastError();
 }
 
 cudaError_t pm_combine_general(long long pairs, int v, int a0, int Ab, int Nb, long long nr, const double* Rp,
-                               const double* Rm, double* R, int accumulate, cudaStream_t st)
+                               const double* Rm, double* R, int accumulate, const double* V, const double* T, cudaStream_t st)
 {
     if (Ab <= 0 || pairs <= 0) return cudaSuccess;
     if (Ab > 65535 || pairs > 0x7fffffffll) return cudaErrorInvalidValue;
-    pm_combine_kernel<true><<<combine_grid(Ab, Nb, pairs), TT * TY, 0, st>>>(0, v, a0, Ab, Nb, nr, pairs, 0, 0, Rp, Rm, R, accumulate);
+    pm_combine_kernel<true><<<combine_grid(Ab, Nb, pairs), TT * TY, 0, st>>>(0, v, a0, Ab, Nb, nr, pairs, 0, 0, Rp, Rm, R, accumulate,
+                                                                             V, T);
     count_launch();
     return cudaGetLastError();
 }

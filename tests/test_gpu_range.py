@@ -86,3 +86,37 @@ def test_mixed_denormal_integrals_round_once(dev, mode, e):
     R = B.ladder_forward(L.to(dev), t2.to(dev), mode=mode, symmetric=True, order="integral_first")
     S = B.ladder_forward(L.pin_memory(), t2.to(dev), mode=mode, symmetric=True, host_L=True, chol_chunk=n)
     assert torch.equal(R, S), float((R - S).abs().max() / S.abs().max())
+
+
+@pytest.mark.parametrize("a_block", [0, 5])
+@pytest.mark.parametrize("exchange", [False, True])
+def test_fp64_general_amplitudes_propagate_as_the_plain_product(dev, a_block, exchange):
+    """Infinite and NaN amplitudes, and finite ones whose sum t_cd + t_dc overflows, give the entries of the plain
+    product sum_cd (ac|bd) t_ijcd: infinities of its sign, NaN where it is NaN, else finite within FP64's rounding."""
+    o, v, n = 3, 37, 6
+    rng = np.random.default_rng(5)
+    L = rng.uniform(0.1, 1.0, (n, v, v)) * rng.choice([-1.0, 1.0], (n, v, v))
+    t2 = rng.standard_normal((o, o, v, v))
+    t2[0, 1, 4, 30] = np.inf
+    t2[1, 0, 7, 7] = -np.inf
+    t2[1, 2, 3, 5], t2[1, 2, 5, 3] = np.inf, -np.inf
+    t2[2, 1, 9, 8] = np.nan
+    t2[2, 2, 10, 36] = t2[2, 2, 36, 10] = 1.5e308
+    L *= 0.02  # |(ac|bd)| <= 2.4e-3: those results stay finite
+    V = np.einsum("nac,nbd->abcd", L, L)
+    t = t2.transpose(0, 1, 3, 2) if exchange else t2
+    with np.errstate(invalid="ignore", over="ignore"):
+        ref = (V.reshape(v * v, 1, v * v) * t.reshape(1, o * o, v * v)).sum(-1).T.reshape(o, o, v, v)
+        mag = (np.abs(V).reshape(v * v, 1, v * v) * np.abs(t).reshape(1, o * o, v * v)).sum(-1).T.reshape(o, o, v, v)
+    assert np.isinf(ref[0, 1]).all() and np.isnan(ref[2, 1]).all() and np.isfinite(ref[2, 2]).all()
+    assert 0 < np.isnan(ref[1, 2]).sum() < v * v
+    R0 = rng.standard_normal(ref.shape)
+    for acc in (False, True):
+        R = torch.from_numpy(R0.copy()).to(dev)
+        B.ladder_forward(torch.from_numpy(L).to(dev), torch.from_numpy(t2).to(dev), R=R, mode="fp64", symmetric=False,
+                         order="integral_first", a_block=a_block, exchange=exchange, accumulate=acc)
+        R = R.cpu().numpy() - (R0 if acc else 0.0)
+        fin = np.isfinite(ref)
+        assert np.array_equal(np.isnan(R), np.isnan(ref))
+        assert np.array_equal(R[np.isinf(ref)], ref[np.isinf(ref)])
+        assert np.all(np.abs(R[fin] - ref[fin]) <= 1e-13 * mag[fin] + (1e-13 if acc else 0.0))
