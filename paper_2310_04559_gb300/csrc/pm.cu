@@ -450,8 +450,8 @@ __device__ __forceinline__ void pair_ij(int o, int p, int& i, int& j)
 // 8 bytes per write over the host link).
 //
 // Not finite: R+ and R- can overflow, or be two infinities of which one sum is NaN, where the plain product is neither
-// (an infinite amplitude, or t_cd + t_dc beyond 2^1024).  With V (GEN in FP64) such entries are the plain product of the
-// block's integrals and the amplitudes, by the entry's whole warp; it costs nothing elsewhere.
+// (an infinite amplitude, or t_cd + t_dc beyond 2^1024).  With PLAIN (GEN in FP64) such entries are the plain product of the
+// block's integrals and the amplitudes, by the entry's whole warp.
 __device__ __forceinline__ double plain_product(const double* __restrict__ V, const double* __restrict__ T, int v, bool swap, int lane)
 {
     double s = 0.0;
@@ -461,7 +461,7 @@ __device__ __forceinline__ double plain_product(const double* __restrict__ V, co
     return s;
 }
 
-template <bool GEN>
+template <bool GEN, bool PLAIN>
 __global__ void pm_combine_kernel(int o, int v, int a0, int Ab, int Nb, long long nr, long long np, long long q0,
                                   long long s0, const double* __restrict__ Rp, const double* __restrict__ Rm,
                                   double* __restrict__ R, int accumulate, const double* __restrict__ V,
@@ -491,7 +491,7 @@ __global__ void pm_combine_kernel(int o, int v, int a0, int Ab, int Nb, long lon
         const double plus = in ? rp[r] : 0.0;
         const double minus = (in && rm && bq != al) ? rm[r] : 0.0;
         double e1 = plus + minus, e2 = plus - minus;
-        if (GEN && V) {
+        if (PLAIN) {
             for (unsigned bad = __ballot_sync(0xffffffffu, in && !(isfinite(e1) && isfinite(e2))); bad; bad &= bad - 1) {
                 const int q = __ffs(bad) - 1;
                 const double* row = V + ((long long)al * Nb + tb + q) * vv;
@@ -619,7 +619,7 @@ cudaError_t pm_combine(int o, int v, int a0, int Ab, int Nb, long long nr, long 
     const long long np = q1 - q0;
     if (Ab <= 0 || np <= 0) return cudaSuccess;
     if (Ab > 65535 || np > 0x7fffffffll || q0 < 0 || q1 > (long long)o * (o + 1) / 2) return cudaErrorInvalidValue;
-    pm_combine_kernel<false><<<combine_grid(Ab, Nb, np), TT * TY, 0, st>>>(o, v, a0, Ab, Nb, nr, np, q0, s0, Rp, Rm, R, accumulate,
+    pm_combine_kernel<false, false><<<combine_grid(Ab, Nb, np), TT * TY, 0, st>>>(o, v, a0, Ab, Nb, nr, np, q0, s0, Rp, Rm, R, accumulate,
                                                                           nullptr, nullptr);
     count_launch();
     return cudaGetLastError();
@@ -630,8 +630,8 @@ cudaError_t pm_combine_general(long long pairs, int v, int a0, int Ab, int Nb, l
 {
     if (Ab <= 0 || pairs <= 0) return cudaSuccess;
     if (Ab > 65535 || pairs > 0x7fffffffll) return cudaErrorInvalidValue;
-    pm_combine_kernel<true><<<combine_grid(Ab, Nb, pairs), TT * TY, 0, st>>>(0, v, a0, Ab, Nb, nr, pairs, 0, 0, Rp, Rm, R, accumulate,
-                                                                             V, T);
+    auto kern = V ? pm_combine_kernel<true, true> : pm_combine_kernel<true, false>;
+    kern<<<combine_grid(Ab, Nb, pairs), TT * TY, 0, st>>>(0, v, a0, Ab, Nb, nr, pairs, 0, 0, Rp, Rm, R, accumulate, V, T);
     count_launch();
     return cudaGetLastError();
 }
