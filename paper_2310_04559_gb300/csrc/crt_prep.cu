@@ -509,9 +509,10 @@ __global__ void __launch_bounds__(NT) crt_pm_f64_kernel(const PmRows a, int nm, 
     const long long rm = a.all_pairs ? r : a.q0 + r - (i + 1) - a.s0;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const int nt = (v + TT - 1) / TT, nb = crt_blocks(v);
+    unsigned long long m1 = 0, m2 = 0;
     int e1 = 0, e2 = 0;
-    for (int pass = 0; pass < 2; ++pass) {
-        unsigned long long m1 = 0, m2 = 0;
+    // one walk over the row's tile pairs: its maxima, or (PUT) its residues
+    auto walk = [&](auto PUT, bool half) {
         for (TilePair t(nt, (int)rank); t.ok(); t.skip((int)cs)) {
             __syncthreads();
 #pragma unroll
@@ -530,10 +531,11 @@ __global__ void __launch_bounds__(NT) crt_pm_f64_kernel(const PmRows a, int nm, 
             for (int q = 0; q < 4; ++q) {
                 const int d = d0 + q;
                 const bool in = d >= c && d < v;
-                const double x1 = S1[pos.cl][pos.dl + q], x2 = S2[pos.dl + q][pos.cl];
+                double x1 = S1[pos.cl][pos.dl + q], x2 = S2[pos.dl + q][pos.cl];
+                if (half) { x1 *= 0.5; x2 *= 0.5; }
                 const double zp = !in ? 0.0 : (d == c ? x1 : x1 + x2);
                 const double zm = (!in || d == c || !minus) ? 0.0 : x1 - x2;
-                if (pass == 0) {
+                if (!PUT.value) {
                     const unsigned long long bp = (unsigned long long)__double_as_longlong(zp) & kAbs;
                     const unsigned long long bm = (unsigned long long)__double_as_longlong(zm) & kAbs;
                     m1 = bp > m1 ? bp : m1;
@@ -543,26 +545,33 @@ __global__ void __launch_bounds__(NT) crt_pm_f64_kernel(const PmRows a, int nm, 
                     xm[q] = fixed_of(zm, e2);
                 }
             }
-            if (pass == 1) {
+            if (PUT.value) {
                 put_quad(xp, nm, Dp + r * pitch, rows_p * pitch, pos.k);
                 if (minus) put_quad(xm, nm, Dm + rm * pitch, rows_m * pitch, pos.k);
             }
         }
-        if (pass == 0) {
-            m1 = cluster_max(m1, red);
-            cluster_done();
-            m2 = cluster_max(m2, red);
-            cluster_done();
-            e1 = exp_of_maxbits(m1);
-            e2 = exp_of_maxbits(m2);
-            if (rank == 0 && threadIdx.x == 0) {
-                ep[r] = e1;
-                if (minus) em[rm] = e2;
-                // NaN or Inf in the row (or an overflowing sum t_cd + t_dc)
-                if (status && (m1 >= kInf || m2 >= kInf)) atomicOr(status, kStatusNonfinite);
-            }
-        }
+    };
+    auto maxima = [&](bool half) {
+        m1 = m2 = 0;
+        walk(std::false_type(), half);
+        m1 = cluster_max(m1, red);
+        cluster_done();
+        m2 = cluster_max(m2, red);
+        cluster_done();
+    };
+    maxima(false);
+    // A finite row whose sums t_cd +- t_dc pass 2^1024 goes by halves (exact, or below the row's last bit).
+    const bool half = a.all_pairs && (m1 >= kInf || m2 >= kInf);  // (the same for the whole cluster)
+    if (half) maxima(true);
+    e1 = exp_of_maxbits(m1);
+    e2 = exp_of_maxbits(m2);
+    if (rank == 0 && threadIdx.x == 0) {
+        ep[r] = e1 + (half ? 1 : 0);
+        if (minus) em[rm] = e2 + (half ? 1 : 0);
+        // NaN or Inf in the row (or, where pair symmetry is promised, an overflowing sum)
+        if (status && (m1 >= kInf || m2 >= kInf)) atomicOr(status, kStatusNonfinite);
     }
+    walk(std::true_type(), half);
 }
 
 // V+ and V- of the integral rows (a, b >= a) of one block from the byte planes of the integral GEMM,

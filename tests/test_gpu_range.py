@@ -7,6 +7,7 @@ import numpy as np
 import pytest
 import torch
 
+from paper_2310_04559_gb300 import _lib
 from paper_2310_04559_gb300 import binding as B
 from paper_2310_04559_gb300 import synth
 
@@ -120,3 +121,24 @@ def test_fp64_general_amplitudes_propagate_as_the_plain_product(dev, a_block, ex
         assert np.array_equal(np.isnan(R), np.isnan(ref))
         assert np.array_equal(R[np.isinf(ref)], ref[np.isinf(ref)])
         assert np.all(np.abs(R[fin] - ref[fin]) <= 1e-13 * mag[fin] + (1e-13 if acc else 0.0))
+
+
+@pytest.mark.parametrize("v", [9, 37, 160])
+def test_emulated_general_amplitudes_up_to_the_largest_double(dev, v):
+    """Finite amplitudes whose sums t_cd + t_dc pass 2^1024 are no infinities: the same bits as their 2^-200th, times
+    2^200 (v = 160: rows walked by a cluster); infinite ones are still refused."""
+    o, n = 2, 5
+    L, _ = synth.ladder_inputs_torch(o, v, n, seed=3, device="cuda")
+    L *= 2.0 ** -80
+    g = torch.Generator(device=dev).manual_seed(v)
+    t2 = (0.5 + 0.49 * torch.rand((o, o, v, v), dtype=torch.float64, device=dev, generator=g)) * 2.0 ** 824
+    t2[1, 1] *= 2.0 ** -30  # a row without such sums
+    want = B.ladder_forward(L, t2, symmetric=False, order="integral_first")
+    huge = t2 * 2.0 ** 200
+    assert torch.isfinite(huge).all() and torch.isinf(huge[0, 0] + huge[0, 0].T).any()
+    got = B.ladder_forward(L, huge, symmetric=False, order="integral_first")
+    assert torch.isfinite(got).all() and torch.equal(got, want * 2.0 ** 200)
+    huge[1, 0, 3, 5] = float("inf")
+    with pytest.raises(_lib.LadderError) as e:
+        B.ladder_forward(L, huge, symmetric=False, order="integral_first")
+    assert e.value.status == -11
