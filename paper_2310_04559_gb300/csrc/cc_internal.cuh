@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "../../include/cc_ladder.h"
 
 namespace cc {
@@ -98,6 +100,20 @@ struct GemmTc {
 cudaError_t gemm_tc(const GemmTc& g, cudaStream_t s);
 int tc_gemm_available();
 int device_sm_count();
+
+// A positive figure of the current device, found once for each device.
+struct PerDevice {
+    std::atomic<int> known[64] = {};
+    template <typename F>
+    int get(F&& find)
+    {
+        int dev = -1;
+        if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return find();
+        int n = known[dev].load(std::memory_order_relaxed);
+        if (n == 0) known[dev].store(n = find(), std::memory_order_relaxed);
+        return n;
+    }
+};
 // C[rmap(m) + cmap(n)] (int64 fixed point) -> FP64: X * 2^(eA[rowA0+m] + eB[rowB0+n] + base)
 cudaError_t fixed_to_f64(int M, int N, const OutDesc& out, const int* eA, long long rowA0, const int* eB,
                          long long rowB0, int base, cudaStream_t s);

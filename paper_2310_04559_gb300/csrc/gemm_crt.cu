@@ -38,6 +38,7 @@
 #include <cudaTypedefs.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "cc_internal.cuh"
@@ -804,21 +805,21 @@ cudaError_t launch(const Sides& g, Params& p, cudaStream_t s)
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    static std::once_flag once;
-    static cudaError_t attr_err = cudaSuccess;
-    static int max_pairs = 0;
-    std::call_once(once, [&cfg] {
-        attr_err = cudaFuncSetAttribute(gemm_crt_kernel<KIND, OUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
-        // persistent: as many pairs as are resident on the device at once
+    // (per context, so set for every launch: a process may call on several devices, or after a device reset)
+    const cudaError_t attr_err =
+        cudaFuncSetAttribute(gemm_crt_kernel<KIND, OUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
+    if (attr_err != cudaSuccess) return attr_err;
+    // persistent: as many pairs as are resident on the device at once
+    static PerDevice resident;
+    const int max_pairs = resident.get([&cfg] {
         int n = 0;
         cfg.gridDim = dim3(2 * 64);
-        if (attr_err != cudaSuccess || cudaOccupancyMaxActiveClusters(&n, gemm_crt_kernel<KIND, OUT>, &cfg) != cudaSuccess || n <= 0) {
+        if (cudaOccupancyMaxActiveClusters(&n, gemm_crt_kernel<KIND, OUT>, &cfg) != cudaSuccess || n <= 0) {
             cudaGetLastError();
-            n = device_sm_count() / 2;
+            n = std::max(1, device_sm_count() / 2);
         }
-        max_pairs = n;
+        return n;
     });
-    if (attr_err != cudaSuccess) return attr_err;
 
     CUtensorMap ma, mb, mc{};
     if (OUT != OUT_F64) {

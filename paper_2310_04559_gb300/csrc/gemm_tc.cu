@@ -889,24 +889,22 @@ bool make_map(CUtensorMap* m, const void* base, int kind, long long K, long long
 template <int KIND, bool FIXED>
 cudaError_t launch(const CUtensorMap& ma, const CUtensorMap& mb, const Params& p, cudaStream_t s)
 {
-    static std::once_flag once;
-    static cudaError_t attr_err = cudaSuccess;
-    static int max_ctas = 0;
-    std::call_once(once, [] {
-        attr_err = cudaFuncSetAttribute(gemm_tc_kernel<KIND, FIXED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)SMEM_BYTES);
-        // persistent: as many CTAs as are resident on the device at once (one per SM)
+    // (per context, so set for every launch: a process may call on several devices, or after a device reset)
+    const cudaError_t attr_err = cudaFuncSetAttribute(gemm_tc_kernel<KIND, FIXED>,
+                                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
+    if (attr_err != cudaSuccess) return attr_err;
+    // persistent: as many CTAs as are resident on the device at once (one per SM)
+    static PerDevice resident;
+    const int max_ctas = resident.get([] {
         int per_sm = 0;
-        if (attr_err != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, gemm_tc_kernel<KIND, FIXED>, THREADS, SMEM_BYTES) !=
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, gemm_tc_kernel<KIND, FIXED>, THREADS, SMEM_BYTES) !=
                 cudaSuccess ||
             per_sm <= 0) {
             cudaGetLastError();
             per_sm = 1;
         }
-        max_ctas = per_sm * device_sm_count();
+        return per_sm * device_sm_count();
     });
-    if (attr_err != cudaSuccess) return attr_err;
     const int ctas = p.nitems < max_ctas ? p.nitems : max_ctas;
     gemm_tc_kernel<KIND, FIXED><<<ctas, THREADS, SMEM_BYTES, s>>>(ma, mb, p);
     return cudaGetLastError();
