@@ -1803,10 +1803,12 @@ int cc_ladder_plan_query(const cc_ladder_args* args, cc_ladder_plan* plan)
     double issued = 0.0;
     if (c.packed) {
         for (const auto& b : blocks) {
-            const long long Ab = b.second, Nb = c.v - b.first;
-            const double nr = (double)Ab * Nb - (double)Ab * (Ab - 1) / 2;
-            const double e1 = c.mode == CC_FP64 ? tri_elems(Ab * c.v, Nb * c.v, c.v, 64, 64)
-                                                : tri_elems(Ab * c.v, Nb * c.v, c.v);
+            // (a range of `a` without pair symmetry builds the rows (a, all b))
+            const long long Ab = b.second, Nb = c.part ? c.v : c.v - b.first;
+            const double nr = c.part ? (double)Ab * Nb : (double)Ab * Nb - (double)Ab * (Ab - 1) / 2;
+            const long long tri = c.part ? 0 : c.v;
+            const double e1 = c.mode == CC_FP64 ? tri_elems(Ab * c.v, Nb * c.v, tri, 64, 64)
+                                                : tri_elems(Ab * c.v, Nb * c.v, tri);
             issued += 2.0 * c.n * e1 + 2.0 * nr * ((double)c.pp * c.Kp + (double)c.pm * c.Km);
         }
     } else {
@@ -1830,7 +1832,7 @@ int cc_ladder_partition(const cc_ladder_args* args, int parts, int* bounds)
     // and the ladder columns of the same pairs, so its work is proportional to v - a; on the other
     // paths every `a` costs the same.
     const double v = c.v;
-    const bool tri = c.packed && !c.gen;  // (a range of one without pair symmetry runs unpacked)
+    const bool tri = c.packed && !c.gen;  // (a range of one without pair symmetry does the unpacked product's work)
     auto W = [&](int a) { return tri ? (double)a * v - (double)a * (a - 1) / 2.0 : (double)a; };
     const double total = W(c.v);
     bounds[0] = 0;

@@ -29,3 +29,11 @@ def test_far_more_occupied_than_virtual_orbitals_run_unpacked(mode, o, v, n):
     p = _plan(o, v, n, 64 * GIB, mode=mode, symmetric=False)
     products = 1 if mode == "fp64" else 12  # at least 12 residues
     assert p["flops_issued"] >= products * p["flops_algorithmic"]
+
+
+# A range of `a` without pair symmetry builds the integrals (a, all b): the work of the plain product, wherever it lies.
+@pytest.mark.parametrize("mode,a_range", [("ozaki_bf16", (0, 7)), ("ozaki_bf16", (90, 100)), ("fp64", (90, 100)), ("bf16", (90, 100))])
+def test_flops_of_a_range_without_pair_symmetry(mode, a_range):
+    p = _plan(6, 100, 300, 8 * GIB, mode=mode, symmetric=False, a_range=a_range)
+    products = 12 if mode == "ozaki_bf16" else 1  # at least 12 residues
+    assert p["flops_issued"] >= products * p["flops_algorithmic"]
