@@ -6,8 +6,9 @@
 // (gemm_crt.cu) gives C_l = (A_l B_l^T) mod p_l, and the Chinese remainder theorem returns the exact
 // integer sum_k X_A X_B as long as it lies in (-P/2, P/2), P = prod p_l.  That holds for ANY input
 // when K 2^82 < P/2, and crt_moduli() takes as many moduli as that needs: 12 up to K = 3574, 13 up
-// to K = 754155.  So 12 or 13 bf16 GEMMs do what the digit slices do with 21, and nothing is dropped (the slices
-// drop every level above 5).  This is the modular form of the Ozaki scheme (Ozaki, Uchino, Imamura,
+// to K = 754155.  (A second contraction, one of whose sides are 43-bit rows made from the first one's results, needs
+// K 2^83 < P/2: 12 up to K = 1787, 13 up to 377077.)  So 12 or 13 bf16 GEMMs do what the digit slices do with 21, and
+// nothing is dropped (the slices drop every level above 5).  This is the modular form of the Ozaki scheme (Ozaki, Uchino, Imamura,
 // "Ozaki Scheme II", 2025), here with the fixed row scale of the slices and with partial sums kept exact by
 // draining the FP32 accumulators every 1024 elements: |r| <= 128, so 1024 products stay within 2^24.
 //
@@ -130,8 +131,10 @@ __host__ __device__ inline int crt_tile_off(int tc, int td, int nb)
 
 #ifdef __CUDACC__
 // Sum of r_l W_l modulo 1 as the top 64 bits, from bytes r_l + 128; add() one byte per modulus (and split).  WIDE sums
-// 96 bits (error 2^-64); without, the 64-bit sum is off by up to nm * 128 units of 2^-64, 2^-53
-// of the largest value: for rows that are rounded to 43 bits.
+// 96 bits (error 2^-64); without, the 64-bit sum is off by up to nm * 128 units of 2^-64: for rows that are rounded to
+// 43 bits.  With 12 moduli that is at most 2^41.4 of an X_A X_B product, 2^-40.6 of max|row A| max|row B| 4: an absolute
+// error, so a row of integrals that all cancel to far below that product keeps fewer than 42 bits of its own largest entry
+// (the digit slices resolve 2^44 there).
 template <bool WIDE>
 struct CrtAcc {
     unsigned long long a0, a1;
