@@ -42,3 +42,13 @@ def test_range_of_a(dev, v, sym):
     assert float(ref.abs().max()) > 0 and np.isfinite(bound)
     # and close in the norm, far below that worst case
     assert float((got - ref).norm() / ref.norm()) < 1e-10
+
+
+@pytest.mark.parametrize("n", [12275, 12276, 12280, 12283, 12284])
+def test_digit_rows_of_many_segments(dev, n):
+    """Cholesky-first in digit slices: the exponents of n + v segments beside 32 bytes of static shared memory."""
+    o, v = 1, 5
+    L, t2 = synth.ladder_inputs_torch(o, v, n, seed=1, device="cuda")
+    R = B.ladder_forward(L, t2, symmetric=True, order="cholesky_first", slices=7)
+    ref = torch.einsum("Pad,Pbd->ab", torch.einsum("Pac,cd->Pad", L, t2[0, 0]), L)
+    assert float((R[0, 0] - ref).norm() / ref.norm()) < 1e-10
