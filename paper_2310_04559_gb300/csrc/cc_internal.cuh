@@ -101,7 +101,7 @@ cudaError_t gemm_tc(const GemmTc& g, cudaStream_t s);
 int tc_gemm_available();
 int device_sm_count();
 
-// A positive figure of the current device, found once for each device.
+// A positive figure of the current device, found once for each device (0: not found, looked for again).
 struct PerDevice {
     std::atomic<int> known[64] = {};
     template <typename F>

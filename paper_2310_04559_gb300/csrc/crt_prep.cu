@@ -591,6 +591,12 @@ struct PmPlanes {
     int diag;                   // b' < al + diag: V- of (b, a)
 };
 
+// Its static shared memory: 33.9 KB, so that the exponents beside it pass 48 KB from about v = 950 on (launch_rows).
+struct PmTiles {
+    long long S[2][2][TT][TT + 1];  // two buffers: one barrier per tile pair
+    long long red[NT / 32 + 1];
+};
+
 template <bool AL, bool WIDE>
 __global__ void __launch_bounds__(NT, 4) crt_pm_planes_kernel(const PmPlanes a, const CrtRec rec, int nm,
                                                            unsigned short* __restrict__ Dp, int* __restrict__ ep,
@@ -598,8 +604,9 @@ __global__ void __launch_bounds__(NT, 4) crt_pm_planes_kernel(const PmPlanes a, 
                                                            long long rows, long long pitch)
 {
     extern __shared__ __align__(16) int esm[];  // exponents of c and of d, then their codes (each padded to a multiple of four)
-    __shared__ long long S[2][2][TT][TT + 1];  // two buffers: one barrier per tile pair
-    __shared__ long long red[NT / 32 + 1];
+    __shared__ PmTiles tiles;
+    long long (&S)[2][2][TT][TT + 1] = tiles.S;
+    long long (&red)[NT / 32 + 1] = tiles.red;
     const uint32_t cs = cluster_size(), rank = cluster_rank();
     const long long r = blockIdx.x / cs;
     const int v = a.v, v4 = (v + 3) & ~3;
@@ -912,20 +919,17 @@ int cluster_for(long long rows, long long elems, long long bytes)
     return cs;
 }
 
+// smem: dynamic shared memory; fixed: the static part of a kernel that takes any, or a little more.
 template <typename... KArgs, typename... Args>
-cudaError_t launch_rows(void (*kern)(KArgs...), long long rows, int cs, size_t smem, cudaStream_t st, Args... args)
+cudaError_t launch_rows(void (*kern)(KArgs...), long long rows, int cs, size_t smem, size_t fixed, cudaStream_t st, Args... args)
 {
     if (rows * cs > 0x7fffffffll) return cudaErrorInvalidConfiguration;
-    if (smem > 0) {
-        // (a launch gets 48 KB unasked, static and dynamic together; the kernel's static part is the compiler's to say)
-        cudaFuncAttributes fa{};
-        cudaError_t e = cudaFuncGetAttributes(&fa, kern);
+    // (a launch gets 48 KB unasked, static and dynamic together; always the same opt-in, so that threads with different v
+    // do not take it from each other)
+    if (smem + fixed > kMaxSmem) return cudaErrorInvalidValue;
+    if (smem + fixed > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kMaxSmem - fixed));
         if (e != cudaSuccess) return e;
-        if (fa.sharedSizeBytes + smem > kMaxSmem) return cudaErrorInvalidValue;
-        if (fa.sharedSizeBytes + smem > 48 * 1024) {
-            e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return e;
-        }
     }
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)(rows * cs));
@@ -955,9 +959,9 @@ cudaError_t crt_rows(const RowSrc& src, int outer, int inner, long long ostride,
     const RowsArg a{src, ostride, outer, inner};
     const long long elems = (long long)outer * inner;
     if ((long long)outer * ((inner + 3) / 4) <= 32 * WQ)
-        return launch_rows(crt_rows_warp_kernel, (src.rows + NT / 32 - 1) / (NT / 32), 1, 0, st, a, nm, (unsigned short*)D,
+        return launch_rows(crt_rows_warp_kernel, (src.rows + NT / 32 - 1) / (NT / 32), 1, 0, 0, st, a, nm, (unsigned short*)D,
                            pitch, e, status);
-    return launch_rows(crt_rows_kernel, src.rows, cluster_for(src.rows, elems, 8 * elems), 0, st, a, nm,
+    return launch_rows(crt_rows_kernel, src.rows, cluster_for(src.rows, elems, 8 * elems), 0, 0, st, a, nm,
                        (unsigned short*)D, pitch, e, status);
 }
 
@@ -970,8 +974,8 @@ cudaError_t crt_cols(const ColSrc& src, int nm, void* D, long long pitch, int* e
     int cs = 1;
     while (cs < 8 && blocks * cs < 4ll * device_sm_count() && src.K > 2ll * CK * cs) cs *= 2;
     if (premax)
-        return launch_rows(crt_cols_kernel<true>, blocks, cs, 0, st, src, nm, premax, (unsigned short*)D, pitch, e, status);
-    return launch_rows(crt_cols_kernel<false>, blocks, cs, 0, st, src, nm, (const unsigned long long*)nullptr,
+        return launch_rows(crt_cols_kernel<true>, blocks, cs, 0, 0, st, src, nm, premax, (unsigned short*)D, pitch, e, status);
+    return launch_rows(crt_cols_kernel<false>, blocks, cs, 0, 0, st, src, nm, (const unsigned long long*)nullptr,
                        (unsigned short*)D, pitch, e, status);
 }
 
@@ -982,7 +986,7 @@ cudaError_t crt_pm_f64(const double* t2, bool all_pairs, int o, int v, long long
     if (rows_p <= 0) return cudaSuccess;
     const PmRows a{t2, all_pairs ? 1 : 0, o, v, q0, s0};
     const long long elems = (long long)v * v;
-    return launch_rows(crt_pm_f64_kernel, rows_p, cluster_for(rows_p, elems, 8 * elems), 0, st, a, nm, (unsigned short*)Dp,
+    return launch_rows(crt_pm_f64_kernel, rows_p, cluster_for(rows_p, elems, 8 * elems), 0, 0, st, a, nm, (unsigned short*)Dp,
                        ep, rows_p, rows_m > 0 ? (unsigned short*)Dm : nullptr, em, rows_m, pitch, status);
 }
 
@@ -998,7 +1002,7 @@ cudaError_t crt_pm_planes(const CrtPlanes& src, bool all_b, long long rows, int 
     const bool al = v % 4 == 0 && src.pitch % 4 == 0 && src.plane % 4 == 0, wide = src.nm > 12;
     return launch_rows(al ? (wide ? crt_pm_planes_kernel<true, true> : crt_pm_planes_kernel<true, false>)
                           : (wide ? crt_pm_planes_kernel<false, true> : crt_pm_planes_kernel<false, false>),
-                       rows, cs, smem, st, a, rec, nm, (unsigned short*)Dp, ep, (unsigned short*)Dm, em, rows, pitch);
+                       rows, cs, smem, sizeof(PmTiles) + 1024, st, a, rec, nm, (unsigned short*)Dp, ep, (unsigned short*)Dm, em, rows, pitch);
 }
 
 cudaError_t crt_rows_planes(const CrtPlanes& src, int nal, int nq, bool q_major, int outer, int inner, const int* eA,
@@ -1014,7 +1018,7 @@ cudaError_t crt_rows_planes(const CrtPlanes& src, int nal, int nq, bool q_major,
     const bool al = inner % 4 == 0 && src.pitch % 4 == 0 && src.plane % 4 == 0, wide = src.nm > 12;
     return launch_rows(al ? (wide ? crt_rows_planes_kernel<true, true> : crt_rows_planes_kernel<true, false>)
                           : (wide ? crt_rows_planes_kernel<false, true> : crt_rows_planes_kernel<false, false>),
-                       rows, cs, 0, st, a, rec, nm, (unsigned short*)D, pitch, e);
+                       rows, cs, 0, 0, st, a, rec, nm, (unsigned short*)D, pitch, e);
 }
 
 cudaError_t crt_to_f64(int M, int N, const CrtPlanes& src, int nsplit, const OutDesc& out, int base, double factor,

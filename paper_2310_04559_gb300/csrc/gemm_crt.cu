@@ -805,13 +805,11 @@ cudaError_t launch(const Sides& g, Params& p, cudaStream_t s)
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    // (per context, so set for every launch: a process may call on several devices, or after a device reset)
-    const cudaError_t attr_err =
-        cudaFuncSetAttribute(gemm_crt_kernel<KIND, OUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
-    if (attr_err != cudaSuccess) return attr_err;
     // persistent: as many pairs as are resident on the device at once
     static PerDevice resident;
     const int max_pairs = resident.get([&cfg] {
+        if (cudaFuncSetAttribute(gemm_crt_kernel<KIND, OUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES) != cudaSuccess)
+            return 0;
         int n = 0;
         cfg.gridDim = dim3(2 * 64);
         if (cudaOccupancyMaxActiveClusters(&n, gemm_crt_kernel<KIND, OUT>, &cfg) != cudaSuccess || n <= 0) {
@@ -820,6 +818,7 @@ cudaError_t launch(const Sides& g, Params& p, cudaStream_t s)
         }
         return n;
     });
+    if (max_pairs == 0) return cudaErrorInvalidConfiguration;
 
     CUtensorMap ma, mb, mc{};
     if (OUT != OUT_F64) {

@@ -889,13 +889,12 @@ bool make_map(CUtensorMap* m, const void* base, int kind, long long K, long long
 template <int KIND, bool FIXED>
 cudaError_t launch(const CUtensorMap& ma, const CUtensorMap& mb, const Params& p, cudaStream_t s)
 {
-    // (per context, so set for every launch: a process may call on several devices, or after a device reset)
-    const cudaError_t attr_err = cudaFuncSetAttribute(gemm_tc_kernel<KIND, FIXED>,
-                                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
-    if (attr_err != cudaSuccess) return attr_err;
     // persistent: as many CTAs as are resident on the device at once (one per SM)
     static PerDevice resident;
     const int max_ctas = resident.get([] {
+        if (cudaFuncSetAttribute(gemm_tc_kernel<KIND, FIXED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)SMEM_BYTES) != cudaSuccess)
+            return 0;
         int per_sm = 0;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, gemm_tc_kernel<KIND, FIXED>, THREADS, SMEM_BYTES) !=
                 cudaSuccess ||
@@ -905,6 +904,7 @@ cudaError_t launch(const CUtensorMap& ma, const CUtensorMap& mb, const Params& p
         }
         return per_sm * device_sm_count();
     });
+    if (max_ctas == 0) return cudaErrorInvalidConfiguration;
     const int ctas = p.nitems < max_ctas ? p.nitems : max_ctas;
     gemm_tc_kernel<KIND, FIXED><<<ctas, THREADS, SMEM_BYTES, s>>>(ma, mb, p);
     return cudaGetLastError();
