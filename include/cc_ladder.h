@@ -293,7 +293,8 @@ void cc_ladder_set_wait_limit_ns(unsigned long long ns);
  *   C[m*ldc + n] (= or +=) sum_k A[m*lda + k] * B[n*ldb + k]     (row-major, K-contiguous FP64)
  * in the arithmetic of `mode` (CC_FP64: FP64 FMAs; CC_OZAKI_BF16: BF16 residues or slices on tcgen05 with
  * FP64 recombination; CC_TF32 / CC_BF16: one rounded copy, FP32 accumulation per K-chunk).
- * accumulate != 0 adds into C.  Workspace from cc_ladder_gemm_workspace_size.
+ * accumulate != 0 adds into C.  Workspace from cc_ladder_gemm_workspace_size (CC_OZAKI_BF16: the residue form's where
+ * that is at most 150 GB, else the digit slices', which also run in any workspace between the two).
  * CC_OZAKI_BF16 is exact in its FP32 sums for any K and any input (see cc_precision). */
 int cc_ladder_gemm_workspace_size(int mode, int M, int N, int K, int slices, size_t* bytes);
 int cc_ladder_gemm(int mode, int M, int N, int K, const double* A, int lda, const double* B, int ldb, double* C,

@@ -2004,7 +2004,11 @@ int cc_ladder_gemm_workspace_size(int mode, int M, int N, int K, int slices, siz
     if (mode < CC_FP64 || mode > CC_BF16) return CC_ERR_ARG;
     if (mode == CC_OZAKI_BF16 && slices != 0 && (slices < 2 || slices > 8)) return CC_ERR_ARG;
     const int s = slices_of(mode, slices);
-    *bytes = std::max(gemm_ws(mode, M, N, K, s), gemm_ws(mode, M, N, K, s, gemm_nm(mode, K, s)));
+    // what the residue form takes (up to about twice the slices' operands, and its result planes) as long as that stays
+    // within the budget that other calls have by default; products beyond it run in the slices' workspace as they did
+    const size_t res = gemm_ws(mode, M, N, K, s, gemm_nm(mode, K, s));
+    *bytes = gemm_ws(mode, M, N, K, s);
+    if (res <= kDefaultBudget) *bytes = std::max(*bytes, res);
     return CC_OK;
 }
 
@@ -2016,7 +2020,7 @@ int cc_ladder_gemm(int mode, int M, int N, int K, const double* A, int lda, cons
     // the residue form where its workspace is there, the digit slices in less
     const int ns = slices_of(mode, slices);
     int nm = gemm_nm(mode, K, ns);
-    if (nm > 0 && ws_bytes < need) nm = 0;
+    if (nm > 0 && ws_bytes < std::max(need, gemm_ws(mode, M, N, K, ns, nm))) nm = 0;
     if (nm == 0) need = gemm_ws(mode, M, N, K, ns);
     if (!A || !B || !C || !workspace) return CC_ERR_NULL;
     if (lda < K || ldb < K || ldc < N) return CC_ERR_ARG;

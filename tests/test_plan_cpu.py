@@ -1,6 +1,9 @@
 """What the planner decides, on the CPU."""
+import ctypes
+
 import pytest
 
+from paper_2310_04559_gb300 import _lib
 from paper_2310_04559_gb300 import binding as B
 
 GIB = 1 << 30
@@ -37,3 +40,13 @@ def test_flops_of_a_range_without_pair_symmetry(mode, a_range):
     p = _plan(6, 100, 300, 8 * GIB, mode=mode, symmetric=False, a_range=a_range)
     products = 12 if mode == "ozaki_bf16" else 1  # at least 12 residues
     assert p["flops_issued"] >= products * p["flops_algorithmic"]
+
+
+# The GEMM building block's workspace is what its caller allocates, beside 8 (M K + N K + M N) bytes of its own.
+@pytest.mark.parametrize("M,N,K", [(60000, 60000, 60000), (125000, 125000, 1000), (50000, 50000, 50000), (8192, 8192, 8192)])
+def test_gemm_workspace_leaves_room_for_the_operands(M, N, K):
+    out = ctypes.c_size_t()
+    assert _lib.load().cc_ladder_gemm_workspace_size(1, M, N, K, 0, ctypes.byref(out)) == 0
+    digits = 2 * 6 * (M + N) * (K + 8) + 4 * (M + N) + 5 * 256
+    assert out.value <= max(150 * GIB, digits)
+    assert out.value + 8 * (M * K + N * K + M * N) < 275e9
