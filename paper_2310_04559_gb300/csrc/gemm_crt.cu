@@ -281,6 +281,12 @@ __device__ __forceinline__ void commit_both(unsigned long long* bar)
         ::"r"(smem_u32(bar)), "h"((unsigned short)3) : "memory");
 }
 
+// The same on this CTA's barrier alone.
+__device__ __forceinline__ void commit_own(unsigned long long* bar)
+{
+    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+
 // The same lane of a converged warp each time; what it issues keeps its operands in uniform registers.
 __device__ __forceinline__ bool elect_one()
 {
@@ -561,8 +567,9 @@ gemm_crt_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             for (uint32_t q = npass > 2 ? npass - 2 : 0; q < npass && ok; ++q)
                 ok = __all_sync(0xffffffffu, mbar_wait(&ctl->tempty[q & 1], (q >> 1) & 1, ctl, rank, p));
             if (any) {
-                // every MMA has completed before TMEM is released
-                if (elect_one()) commit_both(&ctl->drain);
+                // every MMA has completed before TMEM is released (on this CTA's barrier only: nobody in the peer would wait
+                // for the arrival there, which might then find a CTA that has left)
+                if (elect_one()) commit_own(&ctl->drain);
                 __syncwarp();
                 const unsigned long long t0 = gtime();
                 while (!mbar_try(&ctl->drain, 0)) {
